@@ -43,23 +43,35 @@ __device__ __forceinline__ int cap_steps(const DashPattern& P, uint32_t path) {
   }
 }
 
-// Ribs k = 0..J of a dash cap about boundary rib v (start: pivot from psi + pi,
-// end: from psi; both through +pi).
-__device__ __forceinline__ void emit_cap(float4 v, int J, bool square, bool start, uint32_t tg,
-                                         float sv, int32_t src, int64_t o, float4* out_rib,
-                                         float* out_s, uint32_t* out_tag, int32_t* out_src) {
+// A dash cap about boundary rib v (start: pivot from psi + pi, end: from psi; both
+// through +pi): its centre, radius and first angle.
+struct DashCap {
+  float cx, cy, r, psi0;
+};
+__device__ __forceinline__ DashCap make_cap(float4 v, bool start) {
   const float PI_F = 3.14159265358979323846f;
-  float cx = 0.5f * (v.x + v.z), cy = 0.5f * (v.y + v.w);
-  float vx = v.z - v.x, vy = v.w - v.y;
-  float r = 0.5f * sqrtf(vx * vx + vy * vy);
-  float psi = atan2f(-vx, vy);  // the rib is 2r n(psi), n = (-sin psi, cos psi)
-  float psi0 = start ? psi + PI_F : psi;
-  for (int k = 0; k <= J; ++k) {
-    float ang = k == J ? psi0 + PI_F : psi0 + PI_F * (float)k / (float)J;
+  DashCap c;
+  c.cx = 0.5f * (v.x + v.z);
+  c.cy = 0.5f * (v.y + v.w);
+  const float vx = v.z - v.x, vy = v.w - v.y;
+  c.r = 0.5f * sqrtf(vx * vx + vy * vy);
+  const float psi = atan2f(-vx, vy);  // the rib is 2r n(psi), n = (-sin psi, cos psi)
+  c.psi0 = start ? psi + PI_F : psi;
+  return c;
+}
+
+// Ribs k = k0, k0 + dk, .. <= J of a cap whose first rib goes to out[o].
+__device__ __forceinline__ void emit_cap(const DashCap& c, int J, bool square, int k0, int dk,
+                                         uint32_t tg, float sv, int32_t src, int64_t o,
+                                         float4* out_rib, float* out_s, uint32_t* out_tag,
+                                         int32_t* out_src) {
+  const float PI_F = 3.14159265358979323846f;
+  for (int k = k0; k <= J; k += dk) {
+    const float ang = k == J ? c.psi0 + PI_F : c.psi0 + PI_F * (float)k / (float)J;
     float sn, cs;
     sincosf(ang, &sn, &cs);
-    float rn = (square && (k == 1 || k == 3)) ? r * 1.41421356237309515f : r;
-    out_rib[o + k] = make_float4(cx + rn * sn, cy - rn * cs, cx, cy);
+    const float rn = (square && (k == 1 || k == 3)) ? c.r * 1.41421356237309515f : c.r;
+    out_rib[o + k] = make_float4(c.cx + rn * sn, c.cy - rn * cs, c.cx, c.cy);
     out_s[o + k] = sv;
     out_tag[o + k] = (tg & ~(PS_TAG_SEGMENT | PS_TAG_LINK_START)) | (k == 0 ? PS_TAG_LINK_START : 0u);
     if (out_src) out_src[o + k] = src;
@@ -70,7 +82,7 @@ constexpr int DASH_NT = 256;
 constexpr int DASH_QPT = 4;  // quads per thread
 constexpr int DASH_TILE = DASH_NT * DASH_QPT;
 
-// End vertex of a whole quad as dash_quad computes it (f1 = 1): a0 + (a1 - a0)
+// End vertex of a whole quad as the FP64 rule computes it (f1 = 1): a0 + (a1 - a0)
 // in FP64, which is a1 itself whenever a1 - a0 is exact in FP64 (exponents at
 // most 28 apart, or a zero); otherwise the FP64 sum is taken as is.
 __device__ __forceinline__ float whole_end(float a0, float a1) {
@@ -88,7 +100,7 @@ __device__ __forceinline__ float whole_end(float a0, float a1) {
 // periods plus k * 2^-48 period, under 1e-6 of the period for k < 2^24, while
 // the pattern's own FP32 rounding adds at most 2^-24 of it.  eps is 1e-4 of the
 // period.  1: inside an on-stretch (the quad is emitted whole), 0: inside a gap
-// (nothing), -1: within eps of a boundary (decided in FP64 by dash_quad).
+// (nothing), -1: within eps of a boundary (decided in FP64 by DashWalk).
 __device__ __forceinline__ int dash_quick(const DashPattern& P, float sa, float sb) {
   const float per = P.period_f;
   const float eps = 1e-4f * per;
@@ -108,94 +120,59 @@ __device__ __forceinline__ int dash_quick(const DashPattern& P, float sa, float 
   return -1;
 }
 
-template <bool EMIT>
-__device__ __forceinline__ int dash_quad(const DashPattern& P, double sa, double sb, int64_t r,
-                                         const float4* rib, float sa_f, float sb_f,
-                                         uint32_t tg, int64_t out0, float4* out_rib,
-                                         float* out_s, uint32_t* out_tag, int32_t* out_src,
-                                         int64_t out_cap, int32_t* status) {
-  int n = 0;  // output ribs
-  const int J = cap_steps(P, tg >> 2);
-  const bool square = J == 4 && P.path_cap && P.path_cap[tg >> 2] == PS_CAP_SQUARE;
-  double k0 = floor(__ddiv_rn(__dadd_rn(sa, P.offset), P.period)) - 1.0;
-  float4 v0, v1;
-  if (EMIT) {
-    v0 = rib[r - 1];
-    v1 = rib[r];
+// Walk of a quad [sa, sb] over the on-stretches of the pattern, in FP64 with
+// explicitly rounded operations.  next() finds the next stretch that the quad
+// keeps a piece [lo, hi] of, and whether that piece carries caps.
+struct DashWalk {
+  double sa, sb, k0;
+  int guard, i;
+  __device__ __forceinline__ void start(const DashPattern& P, float sa_f, float sb_f) {
+    sa = (double)sa_f;
+    sb = (double)sb_f;
+    k0 = floor(__ddiv_rn(__dadd_rn(sa, P.offset), P.period)) - 1.0;
+    guard = 0;
+    i = 0;
   }
-  for (int guard = 0; guard < (1 << 20); ++guard) {
-    double k = k0 + (double)guard;
-    double base = __dmul_rn(k, P.period);
-    if (__dsub_rn(base, P.offset) > sb) break;
-    for (int i = 0; i < P.m2; i += 2) {
-      double a = __dsub_rn(__dadd_rn(base, P.cum[i]), P.offset);
-      double b = __dsub_rn(__dadd_rn(base, P.cum[i + 1]), P.offset);
-      if (!(b > a)) continue;
-      double lo, hi;
-      bool keep;
-      if (sb > sa) {
-        lo = a > sa ? a : sa;
-        hi = b < sb ? b : sb;
-        keep = hi > lo;
-      } else {
-        lo = sa;
-        hi = sb;
-        keep = (sa >= a && sa < b);
+  __device__ __forceinline__ bool next(const DashPattern& P, bool capped, double& lo, double& hi,
+                                       bool& cap0, bool& cap1) {
+    for (; guard < (1 << 20); ++guard, i = 0) {
+      const double base = __dmul_rn(k0 + (double)guard, P.period);
+      if (__dsub_rn(base, P.offset) > sb) {
+        guard = 1 << 20;
+        break;
       }
-      if (!keep) continue;
-      const bool cap0 = J > 0 && sb > sa && a >= sa && a < sb && a > 0.0;
-      const bool cap1 = J > 0 && sb > sa && b > sa && b <= sb;
-      const int nr = 2 + (cap0 ? J + 1 : 0) + (cap1 ? J + 1 : 0);
-      if (EMIT) {
-        int64_t o = out0 + n + (cap0 ? J + 1 : 0);
-        if (out0 + n + nr <= out_cap) {
-          double f0 = 0.0, f1 = 1.0;
-          if (sb > sa) {
-            double d = __dsub_rn(sb, sa);
-            f0 = __ddiv_rn(__dsub_rn(lo, sa), d);
-            f1 = __ddiv_rn(__dsub_rn(hi, sa), d);
-          }
-          float a0[4] = {v0.x, v0.y, v0.z, v0.w}, a1[4] = {v1.x, v1.y, v1.z, v1.w};
-          float p0[4], p1[4];
-#pragma unroll
-          for (int c = 0; c < 4; ++c) {
-            double dv = __dsub_rn((double)a1[c], (double)a0[c]);
-            p0[c] = (float)__dadd_rn((double)a0[c], __dmul_rn(f0, dv));
-            p1[c] = (float)__dadd_rn((double)a0[c], __dmul_rn(f1, dv));
-          }
-          out_rib[o] = make_float4(p0[0], p0[1], p0[2], p0[3]);
-          out_rib[o + 1] = make_float4(p1[0], p1[1], p1[2], p1[3]);
-          out_s[o] = (float)lo;
-          out_s[o + 1] = (float)hi;
-          out_tag[o] = tg | PS_TAG_LINK_START;
-          out_tag[o + 1] = tg;
-          if (out_src) {
-            out_src[o] = (int32_t)r;
-            out_src[o + 1] = (int32_t)r;
-          }
-          if (cap0)
-            emit_cap(out_rib[o], J, square, true, tg, (float)lo, (int32_t)r, out0 + n, out_rib,
-                     out_s, out_tag, out_src);
-          if (cap1)
-            emit_cap(out_rib[o + 1], J, square, false, tg, (float)hi, (int32_t)r, o + 2, out_rib,
-                     out_s, out_tag, out_src);
+      while (i < P.m2) {
+        const double a = __dsub_rn(__dadd_rn(base, P.cum[i]), P.offset);
+        const double b = __dsub_rn(__dadd_rn(base, P.cum[i + 1]), P.offset);
+        i += 2;
+        if (!(b > a)) continue;
+        bool keep;
+        if (sb > sa) {
+          lo = a > sa ? a : sa;
+          hi = b < sb ? b : sb;
+          keep = hi > lo;
         } else {
-          ps_record_error(status, PS_ERR_CAPACITY);
+          lo = sa;
+          hi = sb;
+          keep = (sa >= a && sa < b);
         }
+        if (!keep) continue;
+        cap0 = capped && sb > sa && a >= sa && a < sb && a > 0.0;
+        cap1 = capped && sb > sa && b > sa && b <= sb;
+        return true;
       }
-      n += nr;
     }
+    return false;
   }
-  return n;
-}
+};
 
 // One pass over tiles of 1,024 quads (4 per thread): the FP32 prefilter
 // settles most quads; the rest (near a stretch boundary) are queued in shared
-// memory and run through the FP64 dash_quad densely -- the FP64 pipe is slow,
+// memory and run through the FP64 walk densely -- the FP64 pipe is slow,
 // and quads left in place would keep almost every warp on it.  Then a block
 // scan of the piece counts, a warp-wide decoupled look-back for the tile's
 // output offset, and emission (queued quads again densely).
-__global__ void __launch_bounds__(DASH_NT) k_dash(
+__global__ void __launch_bounds__(DASH_NT, 3) k_dash(
     const float4* __restrict__ rib, const float* __restrict__ s, const uint32_t* __restrict__ tag,
     const int64_t* __restrict__ n_rib, int64_t capacity, DashPattern P,
     float4* __restrict__ out_rib, float* __restrict__ out_s, uint32_t* __restrict__ out_tag,
@@ -263,9 +240,15 @@ __global__ void __launch_bounds__(DASH_NT) k_dash(
     for (int i = threadIdx.x; i < qtot; i += DASH_NT) {
       const int lq = s_queue[i];
       const int64_t r = t0 + lq;
-      s_cnt[lq] = dash_quad<false>(P, (double)__ldg(s + r - 1), (double)__ldg(s + r), r, rib, 0.f,
-                                   0.f, __ldg(tag + r), 0, nullptr, nullptr, nullptr, nullptr, 0,
-                                   status);
+      const int J = cap_steps(P, __ldg(tag + r) >> 2);
+      DashWalk w;
+      w.start(P, __ldg(s + r - 1), __ldg(s + r));
+      double lo, hi;
+      bool cap0, cap1;
+      int n = 0;
+      while (w.next(P, J > 0, lo, hi, cap0, cap1))
+        n += 2 + (cap0 ? J + 1 : 0) + (cap1 ? J + 1 : 0);
+      s_cnt[lq] = n;
     }
     __syncthreads();
     int cnt[DASH_QPT];
@@ -300,7 +283,7 @@ __global__ void __launch_bounds__(DASH_NT) k_dash(
       if (mode[q] < 0) {
         s_out[q0 + q] = o;  // emitted from the queue below
       } else if (mode[q] == 1) {
-        // inside an on-stretch: the quad itself (f0 = 0, f1 = 1 in dash_quad)
+        // inside an on-stretch: the quad itself (f0 = 0, f1 = 1 below)
         const uint32_t tq = tg[q] & ~PS_TAG_LINK_START;
         if (o + 2 <= out_cap) {
           const float4 v0 = __ldg(rib + r - 1), v1 = __ldg(rib + r);
@@ -322,13 +305,96 @@ __global__ void __launch_bounds__(DASH_NT) k_dash(
       o += cnt[q];
     }
     __syncthreads();
-    for (int i = threadIdx.x; i < qtot; i += DASH_NT) {
-      const int lq = s_queue[i];
-      if (s_cnt[lq] == 0) continue;
+    // queued quads: one per lane, each round one piece of each; long caps are
+    // written by the whole warp (a lane alone would write a round cap's 181 ribs
+    // at 1 degree in turn: 2.81 ms -> 1.18 ms for 1,000 paths
+    // with capped dashes, 24.4 M ribs out)
+    for (int i0 = wid * 32; i0 < qtot; i0 += DASH_NT) {
+      const int lq = i0 + lane < qtot ? s_queue[i0 + lane] : -1;
+      bool more = lq >= 0 && s_cnt[lq] != 0;
       const int64_t r = t0 + lq;
-      dash_quad<true>(P, (double)__ldg(s + r - 1), (double)__ldg(s + r), r, rib, 0.f, 0.f,
-                      __ldg(tag + r) & ~PS_TAG_LINK_START, s_out[lq], out_rib, out_s, out_tag,
-                      out_src, out_cap, status);
+      int64_t o = 0;
+      uint32_t tq = 0u;
+      int J = 0;
+      float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
+      DashWalk w;
+      if (more) {
+        o = s_out[lq];
+        tq = __ldg(tag + r) & ~PS_TAG_LINK_START;
+        J = cap_steps(P, tq >> 2);
+        v0 = rib[r - 1];
+        v1 = rib[r];
+        w.start(P, __ldg(s + r - 1), __ldg(s + r));
+      }
+      const bool square = J == 4 && P.path_cap[tq >> 2] == PS_CAP_SQUARE;
+      while (__any_sync(0xffffffffu, more)) {
+        bool cap0 = false, cap1 = false;
+        double lo = 0.0, hi = 0.0;
+        if (more) more = w.next(P, J > 0, lo, hi, cap0, cap1);
+        float4 p0 = v0, p1 = v1;
+        const int64_t o0 = o;                      // a start cap's first rib
+        const int64_t op = o + (cap0 ? J + 1 : 0);  // the piece
+        if (more) {
+          o = op + 2 + (cap1 ? J + 1 : 0);
+          if (o > out_cap) {
+            ps_record_error(status, PS_ERR_CAPACITY);
+            cap0 = cap1 = false;
+          } else {
+            double f0 = 0.0, f1 = 1.0;
+            if (w.sb > w.sa) {
+              const double d = __dsub_rn(w.sb, w.sa);
+              f0 = __ddiv_rn(__dsub_rn(lo, w.sa), d);
+              f1 = __ddiv_rn(__dsub_rn(hi, w.sa), d);
+            }
+            const float a0[4] = {v0.x, v0.y, v0.z, v0.w}, a1[4] = {v1.x, v1.y, v1.z, v1.w};
+            float c0[4], c1[4];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) {
+              const double dv = __dsub_rn((double)a1[c], (double)a0[c]);
+              c0[c] = (float)__dadd_rn((double)a0[c], __dmul_rn(f0, dv));
+              c1[c] = (float)__dadd_rn((double)a0[c], __dmul_rn(f1, dv));
+            }
+            p0 = make_float4(c0[0], c0[1], c0[2], c0[3]);
+            p1 = make_float4(c1[0], c1[1], c1[2], c1[3]);
+            out_rib[op] = p0;
+            out_rib[op + 1] = p1;
+            out_s[op] = (float)lo;
+            out_s[op + 1] = (float)hi;
+            out_tag[op] = tq | PS_TAG_LINK_START;
+            out_tag[op + 1] = tq;
+            if (out_src) {
+              out_src[op] = (int32_t)r;
+              out_src[op + 1] = (int32_t)r;
+            }
+          }
+        } else {
+          cap0 = cap1 = false;
+        }
+#pragma unroll 1
+        for (int end = 0; end < 2; ++end) {
+          const bool cap = end ? cap1 : cap0;
+          if (!__any_sync(0xffffffffu, cap)) continue;
+          DashCap C{0.f, 0.f, 0.f, 0.f};
+          if (cap) C = make_cap(end ? p1 : p0, end == 0);
+          const int64_t oc = end ? op + 2 : o0;
+          const float sv = (float)(end ? hi : lo);
+          const bool shared = cap && J > 4;
+          if (cap && !shared)
+            emit_cap(C, J, square, 0, 1, tq, sv, (int32_t)r, oc, out_rib, out_s, out_tag, out_src);
+          for (unsigned m = __ballot_sync(0xffffffffu, shared); m; m &= m - 1u) {
+            const int from = __ffs(m) - 1;
+            DashCap B;
+            B.cx = __shfl_sync(0xffffffffu, C.cx, from);
+            B.cy = __shfl_sync(0xffffffffu, C.cy, from);
+            B.r = __shfl_sync(0xffffffffu, C.r, from);
+            B.psi0 = __shfl_sync(0xffffffffu, C.psi0, from);
+            emit_cap(B, __shfl_sync(0xffffffffu, J, from), false, lane, 32,
+                     __shfl_sync(0xffffffffu, tq, from), __shfl_sync(0xffffffffu, sv, from),
+                     __shfl_sync(0xffffffffu, (int32_t)r, from),
+                     __shfl_sync(0xffffffffu, oc, from), out_rib, out_s, out_tag, out_src);
+          }
+        }
+      }
     }
     if (tile == n_tiles - 1 && threadIdx.x == DASH_NT - 1) {
       long long tot = s_prefix + total;
