@@ -16,22 +16,12 @@
 // stretch's first piece or after its last.
 #include <cuda_runtime.h>
 
+#include "ps_dash_walk.cuh"
 #include "ps_internal.cuh"
 
 namespace {
 
-struct DashPattern {
-  double cum[65];
-  double period;
-  double offset;
-  float cum_f[65];             // the same in FP32, for the prefilter
-  float period_f, period_lo;   // period = period_f + period_lo (+ ~2^-48 period)
-  float offset_f;
-  int m2;
-  int j_round;                 // ribs - 1 of a round cap at this dtheta
-  const uint8_t* path_cap;     // cap style per path, or null: butt dash ends
-  int n_path;
-};
+using namespace ps;
 
 __device__ __forceinline__ int cap_steps(const DashPattern& P, uint32_t path) {
   if (!P.path_cap || (int)path >= P.n_path) return 0;
@@ -82,293 +72,343 @@ constexpr int DASH_NT = 256;
 constexpr int DASH_QPT = 4;  // quads per thread
 constexpr int DASH_TILE = DASH_NT * DASH_QPT;
 
-// End vertex of a whole quad as the FP64 rule computes it (f1 = 1): a0 + (a1 - a0)
+// End rib of a whole quad as the FP64 rule computes it (f1 = 1): a0 + (a1 - a0)
 // in FP64, which is a1 itself whenever a1 - a0 is exact in FP64 (exponents at
-// most 28 apart, or a zero); otherwise the FP64 sum is taken as is.
-__device__ __forceinline__ float whole_end(float a0, float a1) {
+// most 28 apart, or a zero); otherwise the FP64 sum is taken as is.  (That sum is out of
+// line: inlined, it was computed for every vertex and discarded, and the FP64
+// pipe was 46% busy with it.)
+__device__ __noinline__ float4 whole_end64(float4 v0, float4 v1) {
+  auto sum = [](float a0, float a1) {
+    return (float)__dadd_rn((double)a0, __dsub_rn((double)a1, (double)a0));
+  };
+  return make_float4(sum(v0.x, v1.x), sum(v0.y, v1.y), sum(v0.z, v1.z), sum(v0.w, v1.w));
+}
+__device__ __forceinline__ bool is_exact_end(float a0, float a1) {
   const int e0 = (int)((__float_as_uint(a0) >> 23) & 0xffu);
   const int e1 = (int)((__float_as_uint(a1) >> 23) & 0xffu);
-  if (a0 == 0.f || a1 == 0.f || abs(e0 - e1) <= 28) return a1;
-  return (float)__dadd_rn((double)a0, __dsub_rn((double)a1, (double)a0));
+  return a0 == 0.f || a1 == 0.f || abs(e0 - e1) <= 28;
+}
+__device__ __forceinline__ float4 whole_end(float4 v0, float4 v1) {
+  if (is_exact_end(v0.x, v1.x) && is_exact_end(v0.y, v1.y) && is_exact_end(v0.z, v1.z) &&
+      is_exact_end(v0.w, v1.w))
+    return v1;
+  return whole_end64(v0, v1);
 }
 
-// FP32 prefilter: whether the quad [sa, sb] lies inside one interval of the
-// pattern (an on-stretch or a gap) with a margin eps above the FP32 error of
-// its phase.  The phase of sa is computed with error-free steps: sa + offset as
-// an exact float pair (TwoSum), k period_f exactly with its FMA residual, and
-// the period's low part; what remains is a few roundings of values below two
-// periods plus k * 2^-48 period, under 1e-6 of the period for k < 2^24, while
-// the pattern's own FP32 rounding adds at most 2^-24 of it.  eps is 1e-4 of the
-// period.  1: inside an on-stretch (the quad is emitted whole), 0: inside a gap
-// (nothing), -1: within eps of a boundary (decided in FP64 by DashWalk).
-__device__ __forceinline__ int dash_quick(const DashPattern& P, float sa, float sb) {
-  const float per = P.period_f;
-  const float eps = 1e-4f * per;
-  const float u = sa + P.offset_f;  // TwoSum: u + ul == sa + offset exactly
-  const float bv = u - sa;
-  const float ul = (sa - (u - bv)) + (P.offset_f - bv);
-  const float k = floorf(u / per);
-  if (!(fabsf(k) < 16777216.f)) return -1;
-  const float kp = k * per;
-  const float ke = fmaf(k, per, -kp);  // k per == kp + ke exactly
-  const float ph = (((u - kp) + ul) - ke) - k * P.period_lo;  // phase of sa
-  if (!(ph >= 0.f && ph < per)) return -1;
-  const float pe = ph + (sb - sa);  // phase of sb, beyond the period if it wraps
-  int j = 0;  // interval [cum_f[j], cum_f[j+1]) holding ph
-  while (j + 1 < P.m2 && P.cum_f[j + 1] <= ph) ++j;
-  if (ph - P.cum_f[j] > eps && P.cum_f[j + 1] - pe > eps) return (j & 1) ? 0 : 1;
-  return -1;
-}
-
-// Walk of a quad [sa, sb] over the on-stretches of the pattern, in FP64 with
-// explicitly rounded operations.  next() finds the next stretch that the quad
-// keeps a piece [lo, hi] of, and whether that piece carries caps.
-struct DashWalk {
-  double sa, sb, k0;
-  int guard, i;
-  __device__ __forceinline__ void start(const DashPattern& P, float sa_f, float sb_f) {
-    sa = (double)sa_f;
-    sb = (double)sb_f;
-    k0 = floor(__ddiv_rn(__dadd_rn(sa, P.offset), P.period)) - 1.0;
-    guard = 0;
-    i = 0;
-  }
-  __device__ __forceinline__ bool next(const DashPattern& P, bool capped, double& lo, double& hi,
-                                       bool& cap0, bool& cap1) {
-    for (; guard < (1 << 20); ++guard, i = 0) {
-      const double base = __dmul_rn(k0 + (double)guard, P.period);
-      if (__dsub_rn(base, P.offset) > sb) {
-        guard = 1 << 20;
-        break;
-      }
-      while (i < P.m2) {
-        const double a = __dsub_rn(__dadd_rn(base, P.cum[i]), P.offset);
-        const double b = __dsub_rn(__dadd_rn(base, P.cum[i + 1]), P.offset);
-        i += 2;
-        if (!(b > a)) continue;
-        bool keep;
-        if (sb > sa) {
-          lo = a > sa ? a : sa;
-          hi = b < sb ? b : sb;
-          keep = hi > lo;
-        } else {
-          lo = sa;
-          hi = sb;
-          keep = (sa >= a && sa < b);
-        }
-        if (!keep) continue;
-        cap0 = capped && sb > sa && a >= sa && a < sb && a > 0.0;
-        cap1 = capped && sb > sa && b > sa && b <= sb;
-        return true;
-      }
-    }
-    return false;
-  }
+// Where a dash call writes.
+struct DashOut {
+  float4* rib;
+  float* s;
+  uint32_t* tag;
+  int32_t* src;
+  int64_t cap;
 };
 
-// One pass over tiles of 1,024 quads (4 per thread): the FP32 prefilter
-// settles most quads; the rest (near a stretch boundary) are queued in shared
-// memory and run through the FP64 walk densely -- the FP64 pipe is slow,
-// and quads left in place would keep almost every warp on it.  Then a block
-// scan of the piece counts, a warp-wide decoupled look-back for the tile's
-// output offset, and emission (queued quads again densely).
-__global__ void __launch_bounds__(DASH_NT, 3) k_dash(
-    const float4* __restrict__ rib, const float* __restrict__ s, const uint32_t* __restrict__ tag,
-    const int64_t* __restrict__ n_rib, int64_t capacity, DashPattern P,
-    float4* __restrict__ out_rib, float* __restrict__ out_s, uint32_t* __restrict__ out_tag,
-    int32_t* __restrict__ out_src, int64_t* __restrict__ n_out, int64_t out_cap, uint32_t* tflag,
-    long long* tagg, long long* tincl, int32_t* counters, int32_t* status) {
-  __shared__ long long sm[DASH_NT / 32];
-  __shared__ int smq[DASH_NT / 32];
-  __shared__ long long s_prefix;
-  __shared__ int64_t s_tile;
-  __shared__ uint16_t s_queue[DASH_TILE];    // tile-local quads for the FP64 path
-  __shared__ int s_cnt[DASH_TILE];           // their piece counts
-  __shared__ long long s_out[DASH_TILE];     // their output offsets
+__device__ __forceinline__ void put_piece(const DashOut& D, int64_t o, float4 p0, float4 p1, float s0,
+                                          float s1, uint32_t tg, int32_t r) {
+  D.rib[o] = p0;
+  D.rib[o + 1] = p1;
+  D.s[o] = s0;
+  D.s[o + 1] = s1;
+  D.tag[o] = tg | PS_TAG_LINK_START;
+  D.tag[o + 1] = tg;
+  if (D.src) {
+    D.src[o] = r;
+    D.src[o + 1] = r;
+  }
+}
+
+// The piece [lo, hi] of a quad by the FP64 rule.
+__device__ __noinline__ void piece64(double lo, double hi, double sa, double sb,
+                                     const float4* v, float4* p) {
+  double f0 = 0.0, f1 = 1.0;
+  if (sb > sa) {
+    const double d = __dsub_rn(sb, sa);
+    f0 = __ddiv_rn(__dsub_rn(lo, sa), d);
+    f1 = __ddiv_rn(__dsub_rn(hi, sa), d);
+  }
+  const float a0[4] = {v[0].x, v[0].y, v[0].z, v[0].w}, a1[4] = {v[1].x, v[1].y, v[1].z, v[1].w};
+  float c0[4], c1[4];
+#pragma unroll
+  for (int c = 0; c < 4; ++c) {
+    const double dv = __dsub_rn((double)a1[c], (double)a0[c]);
+    c0[c] = (float)__dadd_rn((double)a0[c], __dmul_rn(f0, dv));
+    c1[c] = (float)__dadd_rn((double)a0[c], __dmul_rn(f1, dv));
+  }
+  p[0] = make_float4(c0[0], c0[1], c0[2], c0[3]);
+  p[1] = make_float4(c1[0], c1[1], c1[2], c1[3]);
+}
+
+// Output ribs of a quad by the FP64 walk (out of line, as it is rare).
+__device__ __noinline__ int count64(const DashPattern& P, float sa, float sb, int J) {
+  DashWalk w;
+  w.start(P, sa, sb);
+  double lo, hi;
+  bool cap0, cap1;
+  int n = 0;
+  while (w.next(P, J > 0, lo, hi, cap0, cap1)) n += 2 + (cap0 ? J + 1 : 0) + (cap1 ? J + 1 : 0);
+  return n;
+}
+
+// The same quad's pieces and caps, from out[o] on.
+__device__ __noinline__ void quad64(const DashPattern& P, float sa, float sb, int J,
+                                    const float4* rib, int64_t r, uint32_t tg, int64_t o,
+                                    const DashOut& D, int32_t* status) {
+  DashWalk w;
+  w.start(P, sa, sb);
+  double lo, hi;
+  bool cap0, cap1;
+  const bool square = J == 4 && P.path_cap[tg >> 2] == PS_CAP_SQUARE;
+  while (w.next(P, J > 0, lo, hi, cap0, cap1)) {
+    const int64_t o0 = o, op = o + (cap0 ? J + 1 : 0);
+    o = op + 2 + (cap1 ? J + 1 : 0);
+    if (o > D.cap) {
+      ps_record_error(status, PS_ERR_CAPACITY);
+      continue;
+    }
+    const float4 v[2] = {rib[r - 1], rib[r]};
+    float4 p[2];
+    piece64(lo, hi, w.sa, w.sb, v, p);
+    put_piece(D, op, p[0], p[1], (float)lo, (float)hi, tg, (int32_t)r);
+    if (cap0)
+      emit_cap(make_cap(p[0], true), J, square, 0, 1, tg, (float)lo, (int32_t)r, o0, D.rib, D.s,
+               D.tag, D.src);
+    if (cap1)
+      emit_cap(make_cap(p[1], false), J, square, 0, 1, tg, (float)hi, (int32_t)r, op + 2, D.rib,
+               D.s, D.tag, D.src);
+  }
+}
+
+// Two passes.  The first counts: tiles of 1,024 quads, 128 consecutive ones per
+// warp (quad 32 q + lane, so that loads and stores are contiguous over the lanes).
+// The FP32 prefilter settles most quads; the others (1.2% of the 5,031-cubic
+// path's) are queued per warp and walked densely.  A warp scan of the piece
+// counts, the warps' totals through shared memory, and a warp-wide decoupled
+// look-back give every quad's output offset, kept with what is to be written as
+// one word per quad.  The second pass writes, warps on their own, 256 quads
+// each.  A tile's chain (loads, walk, look-back) is all latency: with both passes in
+// one kernel, three CTAs an SM for its registers and seven block barriers a tile,
+// the 5,031-cubic path took 125 us and 1,000 paths with capped dashes 784 us, and
+// 121 and 670 us this way.
+enum { DASH_NONE = 0, DASH_WHOLE = 1, DASH_WALK = 2, DASH_WALK64 = 3 };
+
+__global__ void __launch_bounds__(DASH_NT, 5) k_dash_count(
+    const float* __restrict__ s, const uint32_t* __restrict__ tag,
+    const int64_t* __restrict__ n_rib, int64_t capacity, const __grid_constant__ DashPattern P,
+    unsigned long long* __restrict__ word, int64_t* __restrict__ n_out, int64_t out_cap,
+    uint32_t* tflag, long long* tagg, long long* tincl, int32_t* counters, int32_t* status) {
+  constexpr int WQ = 32 * DASH_QPT;  // quads per warp
+  // two copies, used by alternate tiles: a warp may be a tile ahead of another
+  __shared__ long long s_total[2][DASH_NT / 32];
+  __shared__ long long s_prefix[2];
+  __shared__ int64_t s_next[2];
+  __shared__ uint8_t s_queue[DASH_NT / 32][WQ];  // a warp's queued quads
+  __shared__ uint8_t s_mode[DASH_NT / 32][WQ];
+  __shared__ int s_cnt[DASH_NT / 32][WQ];        // their output ribs
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   int64_t n_tiles = (R + DASH_TILE - 1) / DASH_TILE;
   if (n_tiles == 0) n_tiles = 1;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  for (;;) {
-    if (threadIdx.x == 0) s_tile = atomicAdd(&counters[3], 1);
-    __syncthreads();
-    const int64_t tile = s_tile;
-    __syncthreads();
+  if (threadIdx.x == 0) s_next[1] = atomicAdd(&counters[3], 1);
+  __syncthreads();
+  for (int par = 0;; par ^= 1) {
+    const int64_t tile = s_next[par ^ 1];
     if (tile >= n_tiles) return;
-    const int64_t t0 = tile * DASH_TILE;
-    const int q0 = (int)threadIdx.x * DASH_QPT;  // tile-local index of this thread's first quad
-    int mode[DASH_QPT];
-    float sa[DASH_QPT], sb[DASH_QPT];
-    uint32_t tg[DASH_QPT];
-    int nq = 0;
+    const int64_t t0 = tile * DASH_TILE + wid * WQ;
+    int cnt[DASH_QPT];  // output ribs; -1: queued
+    int qtot = 0;
+    {
+      float sa[DASH_QPT], sb[DASH_QPT];
+      bool quad[DASH_QPT];
 #pragma unroll
-    for (int q = 0; q < DASH_QPT; ++q) {
-      const int64_t r = t0 + q0 + q;
-      mode[q] = 0;
-      tg[q] = 0u;
-      sa[q] = sb[q] = 0.f;
-      if (r >= 1 && r < R) {
-        tg[q] = __ldg(tag + r);
-        if (!(tg[q] & PS_TAG_LINK_START)) {
+      for (int q = 0; q < DASH_QPT; ++q) {
+        const int64_t r = t0 + 32 * q + lane;
+        quad[q] = r >= 1 && r < R;
+        sa[q] = sb[q] = 0.f;
+        if (quad[q]) {
+          quad[q] = !(__ldg(tag + r) & PS_TAG_LINK_START);
           sa[q] = __ldg(s + r - 1);
           sb[q] = __ldg(s + r);
-          mode[q] = dash_quick(P, sa[q], sb[q]);
-          nq += mode[q] < 0;
         }
       }
-    }
-    // queue positions of this thread's FP64 quads (block exclusive scan)
-    int xq = nq;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, xq, o);
-      if (lane >= o) xq += y;
+      for (int q = 0; q < DASH_QPT; ++q) {
+        const int mode = quad[q] ? dash_quick(P, sa[q], sb[q]) : 0;
+        cnt[q] = mode < 0 ? -1 : 2 * mode;
+        const unsigned qm = __ballot_sync(0xffffffffu, mode < 0);
+        if (mode < 0)
+          s_queue[wid][qtot + __popc(qm & ((1u << lane) - 1u))] = (uint8_t)(32 * q + lane);
+        qtot += __popc(qm);
+      }
     }
-    if (lane == 31) smq[wid] = xq;
-    __syncthreads();
-    int qpre = 0, qtot = 0;
-    for (int w = 0; w < DASH_NT / 32; ++w) {
-      if (w < wid) qpre += smq[w];
-      qtot += smq[w];
-    }
-    int qp = qpre + xq - nq;
-#pragma unroll
-    for (int q = 0; q < DASH_QPT; ++q)
-      if (mode[q] < 0) s_queue[qp++] = (uint16_t)(q0 + q);
-    __syncthreads();
-    for (int i = threadIdx.x; i < qtot; i += DASH_NT) {
-      const int lq = s_queue[i];
+    __syncwarp();
+    for (int i = lane; i < qtot; i += 32) {
+      const int lq = s_queue[wid][i];
       const int64_t r = t0 + lq;
       const int J = cap_steps(P, __ldg(tag + r) >> 2);
-      DashWalk w;
+      DashWalkDF w;
       w.start(P, __ldg(s + r - 1), __ldg(s + r));
-      double lo, hi;
-      bool cap0, cap1;
+      ps::DF a, b;
+      bool at_a, at_b, cap0, cap1;
       int n = 0;
-      while (w.next(P, J > 0, lo, hi, cap0, cap1))
+      while (w.next(P, J > 0, a, b, at_a, at_b, cap0, cap1))
         n += 2 + (cap0 ? J + 1 : 0) + (cap1 ? J + 1 : 0);
-      s_cnt[lq] = n;
+      s_mode[wid][lq] = w.sure ? DASH_WALK : DASH_WALK64;
+      s_cnt[wid][lq] = w.sure ? n : count64(P, w.sa, w.sb, J);
     }
-    __syncthreads();
-    int cnt[DASH_QPT];
-    int mine = 0;
+    __syncwarp();
+    long long off[DASH_QPT];  // of each quad's output in the warp's
+    long long wtot = 0;
 #pragma unroll
     for (int q = 0; q < DASH_QPT; ++q) {
-      cnt[q] = mode[q] == 1 ? 2 : mode[q] < 0 ? s_cnt[q0 + q] : 0;
-      mine += cnt[q];
-    }
-    long long x = mine;
+      const int c = cnt[q] < 0 ? s_cnt[wid][32 * q + lane] : cnt[q];
+      long long x = c;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      long long y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
+      for (int o = 1; o < 32; o <<= 1) {
+        const long long y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      off[q] = 4 * (wtot + x - c) +
+               (c == 0 ? DASH_NONE : cnt[q] < 0 ? s_mode[wid][32 * q + lane] : DASH_WHOLE);
+      wtot += __shfl_sync(0xffffffffu, x, 31);
     }
-    if (lane == 31) sm[wid] = x;
+    if (lane == 0) s_total[par][wid] = wtot;
     __syncthreads();
     long long total = 0, wpre = 0;
     for (int w = 0; w < DASH_NT / 32; ++w) {
-      if (w < wid) wpre += sm[w];
-      total += sm[w];
+      if (w < wid) wpre += s_total[par][w];
+      total += s_total[par][w];
     }
     if (wid == 0) {
       long long pre = lookback_sum_warp(tflag, tagg, tincl, total, tile, status);
-      if (lane == 0) s_prefix = pre;
+      if (lane == 0) {
+        s_prefix[par] = pre;
+        s_next[par] = atomicAdd(&counters[3], 1);  // the tile's prefix is published
+        if (tile == n_tiles - 1) {
+          *n_out = pre + total;
+          if (pre + total > out_cap) ps_record_error(status, PS_ERR_CAPACITY);
+        }
+      }
     }
     __syncthreads();
-    int64_t o = s_prefix + wpre + x - mine;
+    const long long base = 4 * (s_prefix[par] + wpre);
 #pragma unroll
     for (int q = 0; q < DASH_QPT; ++q) {
-      const int64_t r = t0 + q0 + q;
-      if (mode[q] < 0) {
-        s_out[q0 + q] = o;  // emitted from the queue below
-      } else if (mode[q] == 1) {
+      const int64_t r = t0 + 32 * q + lane;
+      if (r < R) word[r] = (unsigned long long)(base + off[q]);
+    }
+  }
+}
+
+constexpr int EMIT_WQ = 256;  // quads per warp and round of the writing pass
+__global__ void __launch_bounds__(DASH_NT, 3) k_dash(
+    const float4* __restrict__ rib, const float* __restrict__ s, const uint32_t* __restrict__ tag,
+    const int64_t* __restrict__ n_rib, int64_t capacity, const __grid_constant__ DashPattern P,
+    const unsigned long long* __restrict__ word, const __grid_constant__ DashOut D,
+    int32_t* status) {
+  __shared__ uint8_t s_queue[DASH_NT / 32][EMIT_WQ];  // a warp's queued quads
+  int64_t R = *n_rib;
+  if (R > capacity) R = capacity;
+  const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  const int64_t stride = (int64_t)gridDim.x * (DASH_NT / 32) * EMIT_WQ;
+  for (int64_t t0 = ((int64_t)blockIdx.x * (DASH_NT / 32) + wid) * EMIT_WQ; t0 < R; t0 += stride) {
+    int qtot = 0;
+#pragma unroll 4
+    for (int q = 0; q < EMIT_WQ / 32; ++q) {
+      const int64_t r = t0 + 32 * q + lane;
+      const unsigned long long wd = r < R ? word[r] : 0ull;
+      const int mode = (int)(wd & 3u);
+      const int64_t o = (int64_t)(wd >> 2);
+      if (mode == DASH_WHOLE) {
         // inside an on-stretch: the quad itself (f0 = 0, f1 = 1 below)
-        const uint32_t tq = tg[q] & ~PS_TAG_LINK_START;
-        if (o + 2 <= out_cap) {
+        if (o + 2 <= D.cap) {
           const float4 v0 = __ldg(rib + r - 1), v1 = __ldg(rib + r);
-          out_rib[o] = v0;
-          out_rib[o + 1] = make_float4(whole_end(v0.x, v1.x), whole_end(v0.y, v1.y),
-                                       whole_end(v0.z, v1.z), whole_end(v0.w, v1.w));
-          out_s[o] = sa[q];
-          out_s[o + 1] = sb[q];
-          out_tag[o] = tq | PS_TAG_LINK_START;
-          out_tag[o + 1] = tq;
-          if (out_src) {
-            out_src[o] = (int32_t)r;
-            out_src[o + 1] = (int32_t)r;
-          }
+          put_piece(D, o, v0, whole_end(v0, v1), __ldg(s + r - 1), __ldg(s + r), __ldg(tag + r),
+                    (int32_t)r);
         } else {
           ps_record_error(status, PS_ERR_CAPACITY);
         }
       }
-      o += cnt[q];
+      const unsigned qm = __ballot_sync(0xffffffffu, mode >= DASH_WALK);
+      if (mode >= DASH_WALK)
+        s_queue[wid][qtot + __popc(qm & ((1u << lane) - 1u))] = (uint8_t)(32 * q + lane);
+      qtot += __popc(qm);
     }
-    __syncthreads();
+    __syncwarp();
     // queued quads: one per lane, each round one piece of each; long caps are
     // written by the whole warp (a lane alone would write a round cap's 181 ribs
-    // at 1 degree in turn: 2.81 ms -> 1.18 ms for 1,000 paths
-    // with capped dashes, 24.4 M ribs out)
-    for (int i0 = wid * 32; i0 < qtot; i0 += DASH_NT) {
-      const int lq = i0 + lane < qtot ? s_queue[i0 + lane] : -1;
-      bool more = lq >= 0 && s_cnt[lq] != 0;
+    // at 1 degree in turn: 2.81 ms -> 1.18 ms for 1,000 paths with capped
+    // dashes, 24.4 M ribs out)
+    for (int i0 = 0; i0 < qtot; i0 += 32) {
+      const int lq = i0 + lane < qtot ? s_queue[wid][i0 + lane] : 0;
+      bool more = i0 + lane < qtot;
       const int64_t r = t0 + lq;
       int64_t o = 0;
       uint32_t tq = 0u;
       int J = 0;
       float4 v0 = make_float4(0.f, 0.f, 0.f, 0.f), v1 = v0;
-      DashWalk w;
+      DashWalkDF w{};
       if (more) {
-        o = s_out[lq];
-        tq = __ldg(tag + r) & ~PS_TAG_LINK_START;
+        const unsigned long long wd = word[r];
+        o = (int64_t)(wd >> 2);
+        tq = __ldg(tag + r);
         J = cap_steps(P, tq >> 2);
-        v0 = rib[r - 1];
-        v1 = rib[r];
         w.start(P, __ldg(s + r - 1), __ldg(s + r));
+        if ((wd & 3u) == DASH_WALK) {
+          v0 = __ldg(rib + r - 1);
+          v1 = __ldg(rib + r);
+        } else {
+          quad64(P, w.sa, w.sb, J, rib, r, tq, o, D, status);
+          more = false;
+        }
       }
       const bool square = J == 4 && P.path_cap[tq >> 2] == PS_CAP_SQUARE;
       while (__any_sync(0xffffffffu, more)) {
-        bool cap0 = false, cap1 = false;
-        double lo = 0.0, hi = 0.0;
-        if (more) more = w.next(P, J > 0, lo, hi, cap0, cap1);
+        bool cap0 = false, cap1 = false, at_a = false, at_b = false;
+        ps::DF a{0.f, 0.f}, b{0.f, 0.f};
+        if (more) more = w.next(P, J > 0, a, b, at_a, at_b, cap0, cap1);
         float4 p0 = v0, p1 = v1;
-        const int64_t o0 = o;                      // a start cap's first rib
+        float s0 = w.sa, s1 = w.sb;
+        const int64_t o0 = o;                       // a start cap's first rib
         const int64_t op = o + (cap0 ? J + 1 : 0);  // the piece
-        if (more) {
-          o = op + 2 + (cap1 ? J + 1 : 0);
-          if (o > out_cap) {
-            ps_record_error(status, PS_ERR_CAPACITY);
-            cap0 = cap1 = false;
-          } else {
-            double f0 = 0.0, f1 = 1.0;
-            if (w.sb > w.sa) {
-              const double d = __dsub_rn(w.sb, w.sa);
-              f0 = __ddiv_rn(__dsub_rn(lo, w.sa), d);
-              f1 = __ddiv_rn(__dsub_rn(hi, w.sa), d);
-            }
-            const float a0[4] = {v0.x, v0.y, v0.z, v0.w}, a1[4] = {v1.x, v1.y, v1.z, v1.w};
-            float c0[4], c1[4];
-#pragma unroll
-            for (int c = 0; c < 4; ++c) {
-              const double dv = __dsub_rn((double)a1[c], (double)a0[c]);
-              c0[c] = (float)__dadd_rn((double)a0[c], __dmul_rn(f0, dv));
-              c1[c] = (float)__dadd_rn((double)a0[c], __dmul_rn(f1, dv));
-            }
-            p0 = make_float4(c0[0], c0[1], c0[2], c0[3]);
-            p1 = make_float4(c1[0], c1[1], c1[2], c1[3]);
-            out_rib[op] = p0;
-            out_rib[op + 1] = p1;
-            out_s[op] = (float)lo;
-            out_s[op + 1] = (float)hi;
-            out_tag[op] = tq | PS_TAG_LINK_START;
-            out_tag[op + 1] = tq;
-            if (out_src) {
-              out_src[op] = (int32_t)r;
-              out_src[op + 1] = (int32_t)r;
-            }
-          }
-        } else {
+        if (more) o = op + 2 + (cap1 ? J + 1 : 0);
+        if (!more || o > D.cap) {
+          if (more) ps_record_error(status, PS_ERR_CAPACITY);
           cap0 = cap1 = false;
+        } else {
+          // (a vertex that is not finite is left to the FP64 rule)
+          bool ok = fabsf(v0.x - v1.x) + fabsf(v0.y - v1.y) + fabsf(v0.z - v1.z) +
+                        fabsf(v0.w - v1.w) < INFINITY;
+          const ps::DF d = ps::df_diff(w.sb, w.sa);
+          const float fe = 2.f * w.err / d.hi;  // (only used when d > 0)
+          if (at_a) {
+            p0 = cut_rib(v0, v1, ps::df_div(ps::df_add_f(a, -w.sa), d), fe, ok);
+            s0 = a.hi;
+            ok &= a.hi + (a.lo + w.err) == a.hi && a.hi + (a.lo - w.err) == a.hi;
+          }
+          if (at_b) {
+            p1 = cut_rib(v0, v1, ps::df_div(ps::df_add_f(b, -w.sa), d), fe, ok);
+            s1 = b.hi;
+            ok &= b.hi + (b.lo + w.err) == b.hi && b.hi + (b.lo - w.err) == b.hi;
+          } else {
+            p1 = whole_end(v0, v1);
+          }
+          if (!ok) {  // the stretch's ends in FP64 (k is exact; next() has moved past it)
+            const double base = __dmul_rn((double)(w.k0 + (float)w.g), P.period);
+            const double lo =
+                at_a ? __dsub_rn(__dadd_rn(base, P.cum[w.i - 2]), P.offset) : (double)w.sa;
+            const double hi =
+                at_b ? __dsub_rn(__dadd_rn(base, P.cum[w.i - 1]), P.offset) : (double)w.sb;
+            const float4 v[2] = {v0, v1};
+            float4 p[2];
+            piece64(lo, hi, (double)w.sa, (double)w.sb, v, p);
+            p0 = p[0];
+            p1 = p[1];
+            s0 = (float)lo;
+            s1 = (float)hi;
+          }
+          put_piece(D, op, p0, p1, s0, s1, tq, (int32_t)r);
         }
 #pragma unroll 1
         for (int end = 0; end < 2; ++end) {
@@ -377,10 +417,10 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
           DashCap C{0.f, 0.f, 0.f, 0.f};
           if (cap) C = make_cap(end ? p1 : p0, end == 0);
           const int64_t oc = end ? op + 2 : o0;
-          const float sv = (float)(end ? hi : lo);
+          const float sv = end ? s1 : s0;
           const bool shared = cap && J > 4;
           if (cap && !shared)
-            emit_cap(C, J, square, 0, 1, tq, sv, (int32_t)r, oc, out_rib, out_s, out_tag, out_src);
+            emit_cap(C, J, square, 0, 1, tq, sv, (int32_t)r, oc, D.rib, D.s, D.tag, D.src);
           for (unsigned m = __ballot_sync(0xffffffffu, shared); m; m &= m - 1u) {
             const int from = __ffs(m) - 1;
             DashCap B;
@@ -391,17 +431,12 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
             emit_cap(B, __shfl_sync(0xffffffffu, J, from), false, lane, 32,
                      __shfl_sync(0xffffffffu, tq, from), __shfl_sync(0xffffffffu, sv, from),
                      __shfl_sync(0xffffffffu, (int32_t)r, from),
-                     __shfl_sync(0xffffffffu, oc, from), out_rib, out_s, out_tag, out_src);
+                     __shfl_sync(0xffffffffu, oc, from), D.rib, D.s, D.tag, D.src);
           }
         }
       }
     }
-    if (tile == n_tiles - 1 && threadIdx.x == DASH_NT - 1) {
-      long long tot = s_prefix + total;
-      *n_out = tot;
-      if (tot > out_cap) ps_record_error(status, PS_ERR_CAPACITY);
-    }
-    __syncthreads();
+    __syncwarp();
   }
 }
 
@@ -421,19 +456,7 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
     return PS_ERR_INVALID;
   if (n_pattern < 1 || n_pattern > 32 || !(offset == offset)) return PS_ERR_INVALID;
   DashPattern P;
-  P.m2 = (n_pattern % 2) ? 2 * n_pattern : n_pattern;
-  P.cum[0] = 0.0;
-  for (int i = 0; i < P.m2; ++i) {
-    double d = (double)h_pattern[i % n_pattern];
-    if (!(d >= 0.0)) return PS_ERR_INVALID;
-    P.cum[i + 1] = P.cum[i] + d;
-  }
-  P.period = P.cum[P.m2];
-  P.offset = (double)offset;
-  for (int i = 0; i <= P.m2; ++i) P.cum_f[i] = (float)P.cum[i];
-  P.period_f = (float)P.period;
-  P.period_lo = (float)(P.period - (double)P.period_f);
-  P.offset_f = offset;
+  if (!dash_pattern(P, h_pattern, n_pattern, offset)) return PS_ERR_INVALID;
   P.path_cap = d_path_cap;
   P.n_path = d_path_cap ? n_path : 0;
   P.j_round = 0;
@@ -444,7 +467,6 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
     int J = (int)ceil(x - 1e-4);
     P.j_round = J < 1 ? 1 : J;
   }
-  if (!(P.period > 0.0)) return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
   ctx->last_stream = stream;
   int64_t n_tiles = (capacity + DASH_TILE - 1) / DASH_TILE + 1;
@@ -452,13 +474,23 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
   if (rc != PS_OK) return rc;
   cudaMemsetAsync(ctx->d_tile_flag, 0, sizeof(uint32_t) * (n_tiles + 1), st);
   cudaMemsetAsync(ctx->d_counters, 0, sizeof(int32_t) * 16, st);
-  int grid = ps_persistent_grid(ctx, (const void*)k_dash, DASH_NT, 0);
+  if ((rc = ps_ensure_quad_hits(ctx, capacity)) != PS_OK) return rc;  // 8 bytes per quad
+  unsigned long long* word = reinterpret_cast<unsigned long long*>(ctx->d_quad_hits);
+  const DashOut D{reinterpret_cast<float4*>(d_out_rib), d_out_s, d_out_tag, d_out_src, out_capacity};
+  // no more CTAs than there can be tiles or rounds
+  const int64_t most0 = (capacity + DASH_TILE - 1) / DASH_TILE;
+  const int64_t most1 = (capacity + DASH_NT / 32 * EMIT_WQ - 1) / (DASH_NT / 32 * EMIT_WQ);
+  int64_t grid0 = ps_persistent_grid(ctx, (const void*)k_dash_count, DASH_NT, 0);
+  int64_t grid1 = ps_persistent_grid(ctx, (const void*)k_dash, DASH_NT, 0);
+  if (grid0 > most0) grid0 = most0 > 0 ? most0 : 1;
+  if (grid1 > most1) grid1 = most1 > 0 ? most1 : 1;
   ProfScope ps_(ctx, PK_DASH, st);
-  k_dash<<<grid, DASH_NT, 0, st>>>(reinterpret_cast<const float4*>(d_rib), d_s, d_tag, d_n_rib,
-                                    capacity, P, reinterpret_cast<float4*>(d_out_rib), d_out_s,
-                                    d_out_tag, d_out_src, d_n_out, out_capacity, ctx->d_tile_flag,
-                                    ctx->d_tile_agg, ctx->d_tile_incl, ctx->d_counters,
-                                    ctx->d_status);
+  k_dash_count<<<(unsigned)grid0, DASH_NT, 0, st>>>(d_s, d_tag, d_n_rib, capacity, P, word, d_n_out,
+                                                    out_capacity, ctx->d_tile_flag, ctx->d_tile_agg,
+                                                    ctx->d_tile_incl, ctx->d_counters,
+                                                    ctx->d_status);
+  k_dash<<<(unsigned)grid1, DASH_NT, 0, st>>>(reinterpret_cast<const float4*>(d_rib), d_s, d_tag,
+                                              d_n_rib, capacity, P, word, D, ctx->d_status);
   return ps_cuda_check(cudaGetLastError());
 }
 
