@@ -20,11 +20,9 @@ int ps_ensure_tiles(ps_context* ctx, int64_t n) {
   if (n <= ctx->tile_cap) return PS_OK;
   int64_t cap = n + n / 4 + 64;
   int rc;
-  if ((rc = grow((void**)&ctx->d_tile_flag, sizeof(uint32_t) * cap)) != PS_OK) return rc;
-  if ((rc = grow((void**)&ctx->d_tile_agg, sizeof(long long) * cap)) != PS_OK) return rc;
-  if ((rc = grow((void**)&ctx->d_tile_incl, sizeof(long long) * cap)) != PS_OK) return rc;
-  if ((rc = grow((void**)&ctx->d_tile_aggd, sizeof(double) * cap)) != PS_OK) return rc;
-  if ((rc = grow((void**)&ctx->d_tile_incld, sizeof(double) * cap)) != PS_OK) return rc;
+  // the ticket counters (64 bytes), then the states
+  if ((rc = grow((void**)&ctx->d_counters, 64 + sizeof(TileState) * cap)) != PS_OK) return rc;
+  ctx->d_tile_state = reinterpret_cast<TileState*>(ctx->d_counters + 16);
   ctx->tile_cap = cap;
   return PS_OK;
 }
@@ -85,13 +83,12 @@ extern "C" int ps_create(ps_context** out) {
   cudaDeviceGetAttribute(&ctx->num_sms, cudaDevAttrMultiProcessorCount, ctx->device);
   if (ctx->num_sms <= 0) ctx->num_sms = 1;
   if (cudaMalloc((void**)&ctx->d_status, 64) != cudaSuccess ||
-      cudaMalloc((void**)&ctx->d_counters, sizeof(int32_t) * 16) != cudaSuccess ||
-      cudaMalloc((void**)&ctx->d_scratch64, sizeof(int64_t) * 16) != cudaSuccess) {
+      cudaMalloc((void**)&ctx->d_scratch64, sizeof(int64_t) * 16) != cudaSuccess ||
+      ps_ensure_tiles(ctx, 1) != PS_OK) {
     ps_destroy(ctx);
     return PS_ERR_CUDA;
   }
   cudaMemset(ctx->d_status, 0, 64);
-  cudaMemset(ctx->d_counters, 0, sizeof(int32_t) * 16);
   ctx->tune[PS_TUNE_EMIT_SLABS] = 32;
   ctx->tune[PS_TUNE_SETUP_LINKS] = 2;
   ctx->tune[PS_TUNE_BIN_BLOCKS] = 0;
@@ -141,8 +138,7 @@ extern "C" int ps_get_pixel_tolerance(ps_context* ctx, float* tau) {
 extern "C" void ps_destroy(ps_context* ctx) {
   if (!ctx) return;
   if (ctx->prof_on) ps_profile_enable(ctx, 0);
-  void* ptrs[] = {ctx->d_status, ctx->d_tile_flag, ctx->d_tile_agg, ctx->d_tile_incl,
-                  ctx->d_tile_aggd, ctx->d_tile_incld, ctx->d_counters, ctx->d_recs,
+  void* ptrs[] = {ctx->d_status, ctx->d_counters, ctx->d_recs,
                   ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor, ctx->d_bin,
                   ctx->d_scratch64, ctx->d_mask_scratch, ctx->d_adj, ctx->d_quad_hits,
                   ctx->d_tile_list};
@@ -190,28 +186,23 @@ extern "C" int ps_get_status(ps_context* ctx, int* h_status) {
 // One warp takes the part of tile 1 of a look-back whose tile 0 never
 // publishes: its wait runs to the poll limit, records PS_ERR_TIMEOUT and ends.
 // It touches tiles 0 and 1 only.
-__global__ void k_wait_check(uint32_t* flag, long long* agg, long long* incl, double* aggd,
-                             double* incld, int which, int32_t* status) {
+__global__ void k_wait_check(TileState* state, int which, int32_t* status) {
   if (which == 0)
-    lookback_sum_warp(flag, agg, incl, 1, 1, status);
+    lookback_sum_warp(state, 1, 1, status);
   else
-    lookback_segsum_df(flag, reinterpret_cast<unsigned long long*>(aggd),
-                       reinterpret_cast<unsigned long long*>(incld), ps::DF{1.f, 0.f}, false, 1,
-                       status);
+    lookback_segsum_df(state, ps::DF{1.f, 0.f}, false, 1, status);
 }
 
 extern "C" int ps_check_wait_timeout(ps_context* ctx, int which, void* stream) {
   if (!ctx || (which != 0 && which != 1)) return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  // flags at 0, int64 values at 64 and 96, doubles at 128 and 160 (2 tiles each)
+  // the states of two tiles
   char* buf = nullptr;
   int rc = ps_cuda_check(cudaMalloc((void**)&buf, 256));
   if (rc != PS_OK) return rc;
   rc = ps_cuda_check(cudaMemsetAsync(buf, 0, 256, st));
   if (rc == PS_OK) {
-    k_wait_check<<<1, 32, 0, st>>>((uint32_t*)buf, (long long*)(buf + 64),
-                                   (long long*)(buf + 96), (double*)(buf + 128),
-                                   (double*)(buf + 160), which, ctx->d_status);
+    k_wait_check<<<1, 32, 0, st>>>((TileState*)buf, which, ctx->d_status);
     rc = ps_cuda_check(cudaGetLastError());
   }
   if (rc == PS_OK) rc = ps_cuda_check(cudaStreamSynchronize(st));

@@ -196,7 +196,7 @@ __global__ void __launch_bounds__(DASH_NT, 5) k_dash_count(
     const float* __restrict__ s, const uint32_t* __restrict__ tag,
     const int64_t* __restrict__ n_rib, int64_t capacity, const __grid_constant__ DashPattern P,
     unsigned long long* __restrict__ word, int64_t* __restrict__ n_out, int64_t out_cap,
-    uint32_t* tflag, long long* tagg, long long* tincl, int32_t* counters, int32_t* status) {
+    TileState* state, int32_t* counters, int32_t* status) {
   constexpr int WQ = 32 * DASH_QPT;  // quads per warp
   // two copies, used by alternate tiles: a warp may be a tile ahead of another
   __shared__ long long s_total[2][DASH_NT / 32];
@@ -281,7 +281,7 @@ __global__ void __launch_bounds__(DASH_NT, 5) k_dash_count(
       total += s_total[par][w];
     }
     if (wid == 0) {
-      long long pre = lookback_sum_warp(tflag, tagg, tincl, total, tile, status);
+      long long pre = lookback_sum_warp(state, total, tile, status);
       if (lane == 0) {
         s_prefix[par] = pre;
         s_next[par] = atomicAdd(&counters[3], 1);  // the tile's prefix is published
@@ -472,8 +472,7 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
   int64_t n_tiles = (capacity + DASH_TILE - 1) / DASH_TILE + 1;
   int rc = ps_ensure_tiles(ctx, n_tiles + 1);
   if (rc != PS_OK) return rc;
-  cudaMemsetAsync(ctx->d_tile_flag, 0, sizeof(uint32_t) * (n_tiles + 1), st);
-  cudaMemsetAsync(ctx->d_counters, 0, sizeof(int32_t) * 16, st);
+  cudaMemsetAsync(ctx->d_counters, 0, 64 + sizeof(TileState) * (n_tiles + 1), st);
   if ((rc = ps_ensure_quad_hits(ctx, capacity)) != PS_OK) return rc;  // 8 bytes per quad
   unsigned long long* word = reinterpret_cast<unsigned long long*>(ctx->d_quad_hits);
   const DashOut D{reinterpret_cast<float4*>(d_out_rib), d_out_s, d_out_tag, d_out_src, out_capacity};
@@ -486,8 +485,7 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
   if (grid1 > most1) grid1 = most1 > 0 ? most1 : 1;
   ProfScope ps_(ctx, PK_DASH, st);
   k_dash_count<<<(unsigned)grid0, DASH_NT, 0, st>>>(d_s, d_tag, d_n_rib, capacity, P, word, d_n_out,
-                                                    out_capacity, ctx->d_tile_flag, ctx->d_tile_agg,
-                                                    ctx->d_tile_incl, ctx->d_counters,
+                                                    out_capacity, ctx->d_tile_state, ctx->d_counters,
                                                     ctx->d_status);
   k_dash<<<(unsigned)grid1, DASH_NT, 0, st>>>(reinterpret_cast<const float4*>(d_rib), d_s, d_tag,
                                               d_n_rib, capacity, P, word, D, ctx->d_status);

@@ -62,6 +62,11 @@ enum {
 };
 static_assert(PK_COUNT == PS_PROF_SLOTS, "profile slots");
 
+// State of one tile of a single-pass scan (see below).
+struct __align__(16) TileState {
+  unsigned long long v, flag;
+};
+
 // Host-side context.
 struct ps_context {
   int prof_on;
@@ -73,13 +78,9 @@ struct ps_context {
   int32_t* d_status;        // first error recorded by a kernel
   // scan tile states (shared by the passes of one call; calls on one context
   // are serialized on the stream they are issued to)
-  uint32_t* d_tile_flag;
-  long long* d_tile_agg;
-  long long* d_tile_incl;
-  double* d_tile_aggd;
-  double* d_tile_incld;
+  TileState* d_tile_state;  // [tile_cap]
   int64_t tile_cap;
-  int32_t* d_counters;      // ticket counters, 16 ints
+  int32_t* d_counters;      // ticket counters, 16 ints, right before d_tile_state (one memset)
   LinkRec* d_recs;
   int64_t rec_cap;
   // raster workspace
@@ -110,134 +111,80 @@ __device__ __forceinline__ void ps_record_error(int32_t* status, int code) {
   if (status && *(volatile int32_t*)status == 0) atomicCAS(status, 0, code);
 }
 
-// ---- release / acquire ------------------------------------------------------
-__device__ __forceinline__ void st_release_u32(uint32_t* p, uint32_t v) {
-  asm volatile("st.release.gpu.global.u32 [%0], %1;" ::"l"(p), "r"(v) : "memory");
+// ---- single-pass scans --------------------------------------------------------
+// Tile states (decoupled look-back, Merrill & Garland 2016): a value and a flag, 0 = not
+// ready, TF_AGG = the tile's aggregate, TF_INCL = its inclusive prefix.  The two are read and
+// written as one 128-bit word, so that a reader needs no ordering between them
+// and pays one memory latency per round.
+#define TF_AGG 1ull
+#define TF_INCL 2ull
+
+__device__ __forceinline__ void st_state(TileState* p, unsigned long long v,
+                                         unsigned long long flag) {
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\tmov.b128 t, {%1, %2};\n\tst.relaxed.gpu.global.b128 [%0], t;\n\t}" ::"l"(p),
+      "l"(v), "l"(flag)
+      : "memory");
 }
-__device__ __forceinline__ uint32_t ld_acquire_u32(const uint32_t* p) {
-  uint32_t v;
-  asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_relaxed_s64(long long* p, long long v) {
-  asm volatile("st.relaxed.gpu.global.s64 [%0], %1;" ::"l"(p), "l"(v) : "memory");
-}
-__device__ __forceinline__ long long ld_relaxed_s64(const long long* p) {
-  long long v;
-  asm volatile("ld.relaxed.gpu.global.s64 %0, [%1];" : "=l"(v) : "l"(p) : "memory");
-  return v;
-}
-__device__ __forceinline__ void st_relaxed_f64(double* p, double v) {
-  asm volatile("st.relaxed.gpu.global.f64 [%0], %1;" ::"l"(p), "d"(v) : "memory");
-}
-__device__ __forceinline__ double ld_relaxed_f64(const double* p) {
-  double v;
-  asm volatile("ld.relaxed.gpu.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
-  return v;
+__device__ __forceinline__ TileState ld_state(const TileState* p) {
+  TileState s;
+  asm volatile(
+      "{\n\t.reg .b128 t;\n\tld.relaxed.gpu.global.b128 t, [%2];\n\tmov.b128 {%0, %1}, t;\n\t}"
+      : "=l"(s.v), "=l"(s.flag)
+      : "l"(p)
+      : "memory");
+  return s;
 }
 
-// Tile flags of the single-pass scans (decoupled look-back, Merrill & Garland
-// 2016): 0 = not ready, 1 = aggregate published, 2 = inclusive prefix published.
-// Bit 2 marks a segment head (segmented scans).
-#define TF_AGG 1u
-#define TF_INCL 2u
-#define TF_HEAD 4u
+// Sums of a look-back: int64, or a double-float pair in the state's 64 bits.
+struct SumI64 {
+  typedef long long T;
+  static __device__ __forceinline__ T zero() { return 0; }
+  static __device__ __forceinline__ T add(T a, T b) { return a + b; }
+  static __device__ __forceinline__ T shfl(T a, int lane) { return __shfl_sync(0xffffffffu, a, lane); }
+  static __device__ __forceinline__ T shfl_xor(T a, int o) { return __shfl_xor_sync(0xffffffffu, a, o); }
+  static __device__ __forceinline__ unsigned long long bits(T a) { return (unsigned long long)a; }
+  static __device__ __forceinline__ T of(unsigned long long w) { return (T)w; }
+};
+struct SumDF {
+  typedef ps::DF T;
+  static __device__ __forceinline__ T zero() { return ps::DF{0.f, 0.f}; }
+  static __device__ __forceinline__ T add(T a, T b) { return ps::df_add(a, b); }
+  static __device__ __forceinline__ T shfl(T a, int lane) {
+    return ps::DF{__shfl_sync(0xffffffffu, a.hi, lane), __shfl_sync(0xffffffffu, a.lo, lane)};
+  }
+  static __device__ __forceinline__ T shfl_xor(T a, int o) {
+    return ps::DF{__shfl_xor_sync(0xffffffffu, a.hi, o), __shfl_xor_sync(0xffffffffu, a.lo, o)};
+  }
+  static __device__ __forceinline__ unsigned long long bits(T a) {
+    return ((unsigned long long)__float_as_uint(a.lo) << 32) | (unsigned long long)__float_as_uint(a.hi);
+  }
+  static __device__ __forceinline__ T of(unsigned long long w) {
+    return ps::DF{__uint_as_float((uint32_t)w), __uint_as_float((uint32_t)(w >> 32))};
+  }
+};
 
-// Exclusive prefix of tile t for an int64 sum, with the walk spread over one
-// warp (all 32 lanes call it): lane k reads the state of tile i - k, so one
-// round covers 32 predecessors.  The walk ends at the nearest tile with an
-// inclusive prefix; that tile and every nearer one must have published before
-// the round is summed, else the round is read again (bounded by
-// PS_SPIN_LIMIT).
-__device__ __forceinline__ long long lookback_sum_warp(uint32_t* flag, long long* agg,
-                                                       long long* incl, long long tile_agg,
-                                                       int64_t t, int32_t* status) {
+// Sum of the tiles before tile t, the walk spread over one warp (all 32 lanes
+// call it): lane k reads the state of the k-th nearest tile, so one round covers 32
+// predecessors.  The walk ends at the nearest tile with an inclusive prefix; that
+// tile and every nearer one must have published before the round is summed,
+// else the round is read again (bounded by PS_SPIN_LIMIT; PS_ERR_TIMEOUT after it).  The
+// lanes add up their own terms and reduce them once at the end.  (With flags
+// and values in separate words, read one after the other, the arc-length scan
+// took 235 us on 43 M ribs and 997 us on 211 M, and 168 and 731 us with the
+// 128-bit states; reading two, four or eight windows of 32 a round cost registers and won
+// nothing: 173, 225 and 227 us.)
+template <class S>
+__device__ __forceinline__ typename S::T lookback_walk(const TileState* state, int64_t t,
+                                                       int32_t* status) {
   const int lane = threadIdx.x & 31;
-  if (lane == 0) {
-    if (t == 0) {
-      st_relaxed_s64(&incl[0], tile_agg);
-      st_release_u32(&flag[0], TF_INCL);
-    } else {
-      st_relaxed_s64(&agg[t], tile_agg);
-      st_release_u32(&flag[t], TF_AGG);
-    }
-  }
-  if (t == 0) return 0;
-  long long prefix = 0;
-  int64_t i = t - 1;
+  typename S::T mine = S::zero();
   int spins = 0;
-  for (;;) {
-    int64_t j = i - lane;
-    uint32_t f = j >= 0 ? ld_acquire_u32(&flag[j]) : TF_INCL;  // before tile 0: zero
-    unsigned stop_m = __ballot_sync(0xffffffffu, (f & TF_INCL) != 0u);
-    unsigned unready = __ballot_sync(0xffffffffu, (f & (TF_INCL | TF_AGG)) == 0u);
-    int first = stop_m ? __ffs(stop_m) - 1 : 31;
-    unsigned need = first == 31 ? 0xffffffffu : ((2u << first) - 1u);
-    if (unready & need) {
-      if (++spins > PS_SPIN_LIMIT) {
-        if (lane == 0) ps_record_error(status, PS_ERR_TIMEOUT);
-        break;
-      }
-      __nanosleep(32);
-      continue;
-    }
-    long long v = 0;
-    if (lane <= first && j >= 0) v = (f & TF_INCL) ? ld_relaxed_s64(&incl[j]) : ld_relaxed_s64(&agg[j]);
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
-    prefix += v;
-    if (stop_m) break;
-    i -= 32;
-  }
-  if (lane == 0) {
-    st_relaxed_s64(&incl[t], prefix + tile_agg);
-    st_release_u32(&flag[t], TF_INCL);
-  }
-  return prefix;
-}
-
-// Tile states of the arc-length look-backs: a double-float pair packed in 64
-// bits (hi in the low word), stored and loaded relaxed.
-__device__ __forceinline__ void st_relaxed_df(unsigned long long* p, ps::DF v) {
-  const unsigned long long w =
-      ((unsigned long long)__float_as_uint(v.lo) << 32) | (unsigned long long)__float_as_uint(v.hi);
-  asm volatile("st.relaxed.gpu.global.u64 [%0], %1;" ::"l"(p), "l"(w) : "memory");
-}
-__device__ __forceinline__ ps::DF ld_relaxed_df(const unsigned long long* p) {
-  unsigned long long w;
-  asm volatile("ld.relaxed.gpu.global.u64 %0, [%1];" : "=l"(w) : "l"(p) : "memory");
-  return ps::DF{__uint_as_float((uint32_t)w), __uint_as_float((uint32_t)(w >> 32))};
-}
-
-// Segmented (by path) sum of the tiles (chunks) before tile t: the carry into
-// the tile's elements that precede its first segment head (path start).  A chunk that holds a path
-// start publishes its inclusive value at once (it does not depend on the
-// carry); the walk, one warp reading 32 predecessors per round, ends at the
-// nearest chunk with an inclusive value or a path start, once that chunk and
-// every nearer one have published (bounded by PS_SPIN_LIMIT; PS_ERR_TIMEOUT
-// after it).  Sums are double-float pairs.
-__device__ __forceinline__ ps::DF lookback_segsum_df(uint32_t* flag, unsigned long long* agg,
-                                                 unsigned long long* incl, ps::DF tile_agg,
-                                                 bool tile_head, int64_t t, int32_t* status) {
-  const int lane = threadIdx.x & 31;
-  if (lane == 0) {
-    if (t == 0 || tile_head) {
-      st_relaxed_df(&incl[t], tile_agg);
-      st_release_u32(&flag[t], TF_INCL | (tile_head ? TF_HEAD : 0u));
-    } else {
-      st_relaxed_df(&agg[t], tile_agg);
-      st_release_u32(&flag[t], TF_AGG);
-    }
-  }
-  ps::DF carry{0.f, 0.f};
-  if (t == 0) return carry;
-  int64_t i = t - 1;
-  int spins = 0;
-  for (;;) {
+  for (int64_t i = t - 1;;) {
     const int64_t j = i - lane;
-    const uint32_t f = j >= 0 ? ld_acquire_u32(&flag[j]) : TF_INCL;  // before chunk 0: zero
-    const unsigned stop_m = __ballot_sync(0xffffffffu, (f & TF_INCL) != 0u);
-    const unsigned unready = __ballot_sync(0xffffffffu, (f & (TF_INCL | TF_AGG)) == 0u);
+    const TileState w = j >= 0 ? ld_state(state + j) : TileState{S::bits(S::zero()), TF_INCL};
+    const unsigned stop_m = __ballot_sync(0xffffffffu, w.flag == TF_INCL);
+    const unsigned unready = __ballot_sync(0xffffffffu, w.flag == 0ull);
     const int first = stop_m ? __ffs(stop_m) - 1 : 31;
     const unsigned need = first == 31 ? 0xffffffffu : ((2u << first) - 1u);
     if (unready & need) {
@@ -248,24 +195,42 @@ __device__ __forceinline__ ps::DF lookback_segsum_df(uint32_t* flag, unsigned lo
       __nanosleep(32);
       continue;
     }
-    ps::DF v{0.f, 0.f};
-    if (lane <= first && j >= 0) v = (f & TF_INCL) ? ld_relaxed_df(&incl[j]) : ld_relaxed_df(&agg[j]);
-    if (first == 0) {  // the nearest predecessor holds the prefix: no reduction
-      v = ps::DF{__shfl_sync(0xffffffffu, v.hi, 0), __shfl_sync(0xffffffffu, v.lo, 0)};
-    } else {
-#pragma unroll
-      for (int o = 16; o > 0; o >>= 1)
-        v = ps::df_add(v, ps::DF{__shfl_xor_sync(0xffffffffu, v.hi, o),
-                                 __shfl_xor_sync(0xffffffffu, v.lo, o)});
-    }
-    carry = ps::df_add(carry, v);
+    // the nearest predecessor holds the whole prefix: nothing to sum
+    if (first == 0 && i == t - 1) return S::shfl(S::of(w.v), 0);
+    if (lane <= first) mine = S::add(mine, S::of(w.v));
     if (stop_m) break;
     i -= 32;
   }
-  if (lane == 0 && !tile_head) {
-    st_relaxed_df(&incl[t], ps::df_add(carry, tile_agg));
-    st_release_u32(&flag[t], TF_INCL);
-  }
+#pragma unroll
+  for (int o = 16; o > 0; o >>= 1) mine = S::add(mine, S::shfl_xor(mine, o));
+  return mine;
+}
+
+// Exclusive prefix of tile t for an int64 sum; publishes the tile's own states.
+__device__ __forceinline__ long long lookback_sum_warp(TileState* state, long long tile_agg,
+                                                       int64_t t, int32_t* status) {
+  const int lane = threadIdx.x & 31;
+  if (lane == 0) st_state(&state[t], (unsigned long long)tile_agg, t == 0 ? TF_INCL : TF_AGG);
+  if (t == 0) return 0;
+  const long long prefix = lookback_walk<SumI64>(state, t, status);
+  if (lane == 0) st_state(&state[t], (unsigned long long)(prefix + tile_agg), TF_INCL);
+  return prefix;
+}
+
+// Segmented (by path) sum of the tiles (chunks) before tile t: the carry into
+// the tile's elements that precede its first segment head (path start).  A chunk that holds a path
+// start publishes its inclusive value at once (it does not depend on the
+// carry), so the walk ends at the nearest such chunk.  Sums are double-float
+// pairs.
+__device__ __forceinline__ ps::DF lookback_segsum_df(TileState* state, ps::DF tile_agg,
+                                                     bool tile_head, int64_t t, int32_t* status) {
+  const int lane = threadIdx.x & 31;
+  if (lane == 0)
+    st_state(&state[t], SumDF::bits(tile_agg), t == 0 || tile_head ? TF_INCL : TF_AGG);
+  if (t == 0) return ps::DF{0.f, 0.f};
+  const ps::DF carry = lookback_walk<SumDF>(state, t, status);
+  if (lane == 0 && !tile_head)
+    st_state(&state[t], SumDF::bits(ps::df_add(carry, tile_agg)), TF_INCL);
   return carry;
 }
 

@@ -401,8 +401,7 @@ __global__ void __launch_bounds__(TS_NT) k_tile_scan(const int32_t* __restrict__
                                                      int32_t* __restrict__ off,
                                                      int32_t* __restrict__ cursor,
                                                      int32_t* __restrict__ list, int n_tile,
-                                                     int64_t pair_cap, uint32_t* tflag,
-                                                     long long* tagg, long long* tincl,
+                                                     int64_t pair_cap, TileState* state,
                                                      int32_t* status) {
   __shared__ long long sm[TS_NT / 32];
   __shared__ long long s_pre;
@@ -437,7 +436,7 @@ __global__ void __launch_bounds__(TS_NT) k_tile_scan(const int32_t* __restrict__
     total += sm[w];
   }
   if (wid == 0) {
-    long long pre = lookback_sum_warp(tflag, tagg, tincl, total, blockIdx.x, status);
+    long long pre = lookback_sum_warp(state, total, blockIdx.x, status);
     if (lane == 0) s_pre = pre;
   }
   __syncthreads();
@@ -1630,8 +1629,7 @@ static int rasterize(ps_context* ctx, const float* d_rib, const uint32_t* d_tag,
   int grid_cov = ps_persistent_grid(ctx, kcov, CV_NT, cov_smem);
   ctx->last_n_tile = n_tile;
   cudaMemsetAsync(ctx->d_tile_count, 0, sizeof(int32_t) * (n_tile + 1), st);
-  cudaMemsetAsync(ctx->d_tile_flag, 0, sizeof(uint32_t) * ((n_tile + TS_TILE - 1) / TS_TILE + 1), st);
-  cudaMemsetAsync(ctx->d_counters, 0, sizeof(int32_t) * 16, st);
+  cudaMemsetAsync(ctx->d_counters, 0, 64 + sizeof(TileState) * ((n_tile + TS_TILE - 1) / TS_TILE + 1), st);
   cudaMemsetAsync(d_covered, 0, sizeof(uint64_t) * (size_t)n_path, st);
   // tiles without entries are never visited by the coverage kernel
   cudaMemsetAsync(d_canvas, 0, sizeof(uint16_t) * (size_t)width * (size_t)height, st);
@@ -1654,8 +1652,7 @@ static int rasterize(ps_context* ctx, const float* d_rib, const uint32_t* d_tag,
   const int ts_grid = (int)((n_tile + TS_TILE - 1) / TS_TILE);
   k_tile_scan<<<ts_grid, TS_NT, 0, st>>>(ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,
                                          ctx->d_tile_list, (int)n_tile, ctx->pair_cap,
-                                         ctx->d_tile_flag, ctx->d_tile_agg, ctx->d_tile_incl,
-                                         ctx->d_status); }
+                                         ctx->d_tile_state, ctx->d_status); }
   { ProfScope ps_(ctx, PK_BIN_SCATTER, st);
   k_bin<1><<<grid_bin1, BIN_NT, 0, st>>>(rib, d_tag, d_n_rib, capacity, width, height, y0, tiles_x,
                                       ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,

@@ -1247,8 +1247,7 @@ __global__ void __launch_bounds__(SETUP_NT, 2) k_link_setup(
     const float* __restrict__ miter, const uint8_t* __restrict__ closed, int n_path,
     int64_t n_link, float q, float tau, LinkRec* __restrict__ recs, int32_t* __restrict__ link_off,
     int32_t* __restrict__ path_off, int64_t* __restrict__ n_rib_out, int64_t capacity,
-    uint32_t* tflag, long long* tagg, long long* tincl, int32_t* counters, int32_t* status,
-    int64_t n_tiles, int64_t l_begin) {
+    TileState* state, int32_t* counters, int32_t* status, int64_t n_tiles, int64_t l_begin) {
   __shared__ long long sm[SETUP_NT / 32 + 1];
   __shared__ long long s_prefix;
   __shared__ int s_tile;
@@ -1328,7 +1327,7 @@ __global__ void __launch_bounds__(SETUP_NT, 2) k_link_setup(
   long long total;
   long long excl = block_excl_sum<SETUP_NT>(local, total, sm);
   if (threadIdx.x < 32) {
-    long long pre = lookback_sum_warp(tflag, tagg, tincl, total, tile, status);
+    long long pre = lookback_sum_warp(state, total, tile, status);
     if (threadIdx.x == 0) s_prefix = pre;
   }
   __syncthreads();
@@ -1664,8 +1663,8 @@ constexpr int SCAN_TILE = SCAN_NT * SCAN_IPT;
 template <bool VEC>
 __global__ void __launch_bounds__(SCAN_NT) k_arclen_scan(
     const float* chord_in, const uint32_t* __restrict__ tag, const int64_t* __restrict__ n_rib,
-    int64_t capacity, float* s_out, float* __restrict__ path_len, uint32_t* tflag,
-    unsigned long long* tagg, unsigned long long* tincl, int32_t* counters, int32_t* status) {
+    int64_t capacity, float* s_out, float* __restrict__ path_len, TileState* state,
+    int32_t* counters, int32_t* status) {
   __shared__ float sv[SCAN_NT / 32];
   __shared__ int sh[SCAN_NT / 32];
   __shared__ float s_carry[2];
@@ -1752,7 +1751,7 @@ __global__ void __launch_bounds__(SCAN_NT) k_arclen_scan(
         tile_v = df_add_f(tile_v, sv[w]);
         if (sh[w]) { tile_h = 1; break; }
       }
-      DF carry = lookback_segsum_df(tflag, tagg, tincl, tile_v, tile_h != 0, tile, status);
+      DF carry = lookback_segsum_df(state, tile_v, tile_h != 0, tile, status);
       if (lane == 0) {
         s_carry[0] = carry.hi;
         s_carry[1] = carry.lo;
@@ -1802,21 +1801,18 @@ __global__ void __launch_bounds__(SCAN_NT) k_arclen_scan(
 // Launch of k_arclen_scan with the vector form when every array allows it.
 static void launch_arclen_scan(ps_context* ctx, int grid_override, cudaStream_t st,
                                const float* chord, const uint32_t* tag, const int64_t* n_rib,
-                               int64_t capacity, float* s_out, float* path_len, uint32_t* flag,
-                               double* aggd, double* incld, int32_t* counters, int32_t* status) {
-  // the tile states' 8-byte words hold double-float pairs
-  unsigned long long* agg = reinterpret_cast<unsigned long long*>(aggd);
-  unsigned long long* incl = reinterpret_cast<unsigned long long*>(incld);
+                               int64_t capacity, float* s_out, float* path_len,
+                               TileState* state, int32_t* counters, int32_t* status) {
   const bool vec = ((reinterpret_cast<uintptr_t>(chord) | reinterpret_cast<uintptr_t>(tag) |
                      reinterpret_cast<uintptr_t>(s_out)) & 15u) == 0;
   const void* fn = vec ? (const void*)k_arclen_scan<true> : (const void*)k_arclen_scan<false>;
   int g = grid_override > 0 ? grid_override : ps_persistent_grid(ctx, fn, SCAN_NT, 0);
   if (vec)
-    k_arclen_scan<true><<<g, SCAN_NT, 0, st>>>(chord, tag, n_rib, capacity, s_out, path_len, flag,
-                                               agg, incl, counters, status);
+    k_arclen_scan<true><<<g, SCAN_NT, 0, st>>>(chord, tag, n_rib, capacity, s_out, path_len,
+                                               state, counters, status);
   else
     k_arclen_scan<false><<<g, SCAN_NT, 0, st>>>(chord, tag, n_rib, capacity, s_out, path_len,
-                                                flag, agg, incl, counters, status);
+                                                state, counters, status);
 }
 
 // Chords from rib midpoints (standalone arc length of any rib stream).
@@ -1862,8 +1858,11 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
   if ((rc = ps_ensure_recs(ctx, L)) != PS_OK) return rc;
   // link path indices live after the records
   int32_t* link_path = reinterpret_cast<int32_t*>(ctx->d_recs + ctx->rec_cap);
-  cudaMemsetAsync(ctx->d_tile_flag, 0, sizeof(uint32_t) * n_tiles, st);
-  cudaMemsetAsync(ctx->d_counters, 0, sizeof(int32_t) * 16, st);
+  // counters, set-up tiles and scan tiles
+  const int64_t scan_tiles = (out->capacity + SCAN_TILE - 1) / SCAN_TILE;
+  const bool arc = !(flags & PS_TESS_COUNT_ONLY) && (flags & PS_TESS_ARCLENGTH) && out->d_s;
+  cudaMemsetAsync(ctx->d_counters, 0,
+                  64 + sizeof(TileState) * (n_tiles + (arc ? scan_tiles + 2 : 0)), st);
   // a count-only call has no rib buffers to overflow
   int64_t count_cap = (flags & PS_TESS_COUNT_ONLY) ? INT64_MAX : out->capacity;
   { ProfScope ps_(ctx, PK_LINK_PATH, st);
@@ -1873,8 +1872,8 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
 #define PS_SETUP_ARGS                                                                          \
   seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,         \
       paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs, \
-      out->d_link_rib_off, out->d_path_rib_off, out->d_n_rib, count_cap, ctx->d_tile_flag,    \
-      ctx->d_tile_agg, ctx->d_tile_incl, ctx->d_counters, ctx->d_status, n_tiles, l0
+      out->d_link_rib_off, out->d_path_rib_off, out->d_n_rib, count_cap, ctx->d_tile_state,   \
+      ctx->d_counters, ctx->d_status, n_tiles, l0
   const unsigned g = (unsigned)n_tiles;
   const bool mx = precision == PS_PREC_MIXED;
   if (ctx->pixel_tol > 0.f) {
@@ -1895,7 +1894,6 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
   if ((rc = ps_cuda_check(cudaGetLastError())) != PS_OK) return rc;
   if (flags & PS_TESS_COUNT_ONLY) return PS_OK;
 
-  bool arc = (flags & PS_TESS_ARCLENGTH) && out->d_s;
   const void* fn = precision == PS_PREC_MIXED ? (const void*)k_emit<true> : (const void*)k_emit<false>;
   int grid = ps_persistent_grid(ctx, fn, EMIT_NT, 0);
   {
@@ -1912,14 +1910,11 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
   if (arc) {
     // the emitter wrote each rib's chord into s; the segmented scan turns them
     // into cumulative arc length in place
-    int64_t scan_tiles = (out->capacity + SCAN_TILE - 1) / SCAN_TILE;
-    cudaMemsetAsync(ctx->d_tile_flag + n_tiles + 1, 0, sizeof(uint32_t) * (scan_tiles + 1), st);
     if (out->d_path_len) cudaMemsetAsync(out->d_path_len, 0, sizeof(float) * P, st);
     ProfScope ps_(ctx, PK_ARCLEN, st);
     launch_arclen_scan(ctx, 0, st, out->d_s, out->d_tag, out->d_n_rib, out->capacity, out->d_s,
-                       out->d_path_len, ctx->d_tile_flag + n_tiles + 1,
-                       ctx->d_tile_aggd + n_tiles + 1, ctx->d_tile_incld + n_tiles + 1,
-                       ctx->d_counters, ctx->d_status);
+                       out->d_path_len, ctx->d_tile_state + n_tiles + 1, ctx->d_counters,
+                       ctx->d_status);
     if ((rc = ps_cuda_check(cudaGetLastError())) != PS_OK) return rc;
   }
   return PS_OK;
@@ -2048,16 +2043,15 @@ extern "C" int ps_arclength_scan(ps_context* ctx, const float* d_rib, const uint
   int64_t scan_tiles = (capacity + SCAN_TILE - 1) / SCAN_TILE;
   int rc = ps_ensure_tiles(ctx, scan_tiles + 2);
   if (rc != PS_OK) return rc;
-  cudaMemsetAsync(ctx->d_tile_flag, 0, sizeof(uint32_t) * (scan_tiles + 1), st);
-  cudaMemsetAsync(ctx->d_counters, 0, sizeof(int32_t) * 16, st);
+  cudaMemsetAsync(ctx->d_counters, 0, 64 + sizeof(TileState) * (scan_tiles + 1), st);
   if (d_path_len && n_path > 0) cudaMemsetAsync(d_path_len, 0, sizeof(float) * n_path, st);
   int g = ps_persistent_grid(ctx, (const void*)k_midpoint_chords, 256, 0);
   { ProfScope ps_(ctx, PK_MIDCHORD, st);
   k_midpoint_chords<<<g, 256, 0, st>>>(reinterpret_cast<const float4*>(d_rib), d_tag, d_n_rib,
                                        capacity, d_s); }
   ProfScope ps_(ctx, PK_ARCLEN, st);
-  launch_arclen_scan(ctx, 0, st, d_s, d_tag, d_n_rib, capacity, d_s, d_path_len, ctx->d_tile_flag,
-                     ctx->d_tile_aggd, ctx->d_tile_incld, ctx->d_counters, ctx->d_status);
+  launch_arclen_scan(ctx, 0, st, d_s, d_tag, d_n_rib, capacity, d_s, d_path_len, ctx->d_tile_state,
+                     ctx->d_counters, ctx->d_status);
   return ps_cuda_check(cudaGetLastError());
 }
 
@@ -2081,13 +2075,9 @@ constexpr int64_t NOALLOC_TILES = NOALLOC_SETUP_TILES + 1 + NOALLOC_SCAN_TILES +
 constexpr size_t al256(size_t x) { return (x + 255) & ~(size_t)255; }
 constexpr size_t NA_RECS = 0;
 constexpr size_t NA_PATH = al256(NA_RECS + sizeof(LinkRec) * NOALLOC_MAX_LINKS);
-constexpr size_t NA_FLAG = al256(NA_PATH + sizeof(int32_t) * NOALLOC_MAX_LINKS);
-constexpr size_t NA_AGG = al256(NA_FLAG + sizeof(uint32_t) * NOALLOC_TILES);
-constexpr size_t NA_INCL = al256(NA_AGG + sizeof(long long) * NOALLOC_TILES);
-constexpr size_t NA_AGGD = al256(NA_INCL + sizeof(long long) * NOALLOC_TILES);
-constexpr size_t NA_INCLD = al256(NA_AGGD + sizeof(double) * NOALLOC_TILES);
-constexpr size_t NA_CNT = al256(NA_INCLD + sizeof(double) * NOALLOC_TILES);
-constexpr size_t NA_BYTES = al256(NA_CNT + sizeof(int32_t) * 16);
+constexpr size_t NA_CNT = al256(NA_PATH + sizeof(int32_t) * NOALLOC_MAX_LINKS);
+constexpr size_t NA_STATE = NA_CNT + 64;  // right after the 16 counters: one memset
+constexpr size_t NA_BYTES = al256(NA_STATE + sizeof(TileState) * NOALLOC_TILES);
 }  // namespace
 
 // The workspace: about 4.0 MB held by every device that loads the library until
@@ -2140,19 +2130,14 @@ extern "C" int ps_tessellate_strokes_noalloc(const ps_segments* seg, const ps_pa
   unsigned char* base = g_noalloc_ptr[dev];
   LinkRec* recs = reinterpret_cast<LinkRec*>(base + NA_RECS);
   int32_t* link_path = reinterpret_cast<int32_t*>(base + NA_PATH);
-  uint32_t* tflag = reinterpret_cast<uint32_t*>(base + NA_FLAG);
-  long long* tagg = reinterpret_cast<long long*>(base + NA_AGG);
-  long long* tincl = reinterpret_cast<long long*>(base + NA_INCL);
-  double* taggd = reinterpret_cast<double*>(base + NA_AGGD);
-  double* tincld = reinterpret_cast<double*>(base + NA_INCLD);
+  TileState* state = reinterpret_cast<TileState*>(base + NA_STATE);
   int32_t* counters = reinterpret_cast<int32_t*>(base + NA_CNT);
 
   cudaStream_t st = (cudaStream_t)stream;
   int P = paths->n_path;
   int64_t n_tiles = (L + SETUP_TILE - 1) / SETUP_TILE;
   // the array keeps the previous call's contents: reset what must start at zero
-  if (cudaMemsetAsync(tflag, 0, sizeof(uint32_t) * NOALLOC_TILES, st) != cudaSuccess ||
-      cudaMemsetAsync(counters, 0, sizeof(int32_t) * 16, st) != cudaSuccess)
+  if (cudaMemsetAsync(counters, 0, 64 + sizeof(TileState) * NOALLOC_TILES, st) != cudaSuccess)
     return PS_ERR_CUDA;
   int64_t count_cap = count_only ? INT64_MAX : out->capacity;
   k_link_path<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(paths->d_seg_off, P, L, link_path, (int64_t)0);
@@ -2160,13 +2145,13 @@ extern "C" int ps_tessellate_strokes_noalloc(const ps_segments* seg, const ps_pa
     k_link_setup<true, SETUP_IPT><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
         paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, 0.f, recs, out->d_link_rib_off,
-        out->d_path_rib_off, out->d_n_rib, count_cap, tflag, tagg, tincl, counters, d_status,
+        out->d_path_rib_off, out->d_n_rib, count_cap, state, counters, d_status,
         n_tiles, (int64_t)0);
   else
     k_link_setup<false, SETUP_IPT><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
         paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, 0.f, recs, out->d_link_rib_off,
-        out->d_path_rib_off, out->d_n_rib, count_cap, tflag, tagg, tincl, counters, d_status,
+        out->d_path_rib_off, out->d_n_rib, count_cap, state, counters, d_status,
         n_tiles, (int64_t)0);
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   if (count_only) return PS_OK;
@@ -2193,8 +2178,7 @@ extern "C" int ps_tessellate_strokes_noalloc(const ps_segments* seg, const ps_pa
     int g2 = g_noalloc_sms[dev] * (per_sm2 > 0 ? per_sm2 : 1);
     int64_t o = NOALLOC_SETUP_TILES + 1;
     launch_arclen_scan(nullptr, g2, st, out->d_s, out->d_tag, out->d_n_rib, out->capacity,
-                       out->d_s, out->d_path_len, tflag + o, taggd + o, tincld + o, counters,
-                       d_status);
+                       out->d_s, out->d_path_len, state + o, counters, d_status);
     if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   }
   return PS_OK;
@@ -2212,35 +2196,34 @@ int ps_run_link_setup(ps_context* ctx, const ps_segments* seg, const ps_paths* p
   if ((rc = ps_ensure_tiles(ctx, n_tiles + 2)) != PS_OK) return rc;
   if ((rc = ps_ensure_recs(ctx, L)) != PS_OK) return rc;
   int32_t* link_path = reinterpret_cast<int32_t*>(ctx->d_recs + ctx->rec_cap);
-  cudaMemsetAsync(ctx->d_tile_flag, 0, sizeof(uint32_t) * n_tiles, st);
-  cudaMemsetAsync(ctx->d_counters, 0, sizeof(int32_t) * 16, st);
+  cudaMemsetAsync(ctx->d_counters, 0, 64 + sizeof(TileState) * n_tiles, st);
   k_link_path<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(paths->d_seg_off, P, L, link_path, (int64_t)0);
   const bool px = ctx->pixel_tol > 0.f;
   if (precision == PS_PREC_MIXED && px)
     k_link_setup<true, SETUP_IPT, true><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
         paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs,
-        d_link_off, d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_flag, ctx->d_tile_agg,
-        ctx->d_tile_incl, ctx->d_counters, ctx->d_status, n_tiles, (int64_t)0);
+        d_link_off, d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
+        ctx->d_counters, ctx->d_status, n_tiles, (int64_t)0);
   else if (px)
     k_link_setup<false, SETUP_IPT, true><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
         paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs,
-        d_link_off, d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_flag, ctx->d_tile_agg,
-        ctx->d_tile_incl, ctx->d_counters, ctx->d_status, n_tiles, (int64_t)0);
+        d_link_off, d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
+        ctx->d_counters, ctx->d_status, n_tiles, (int64_t)0);
   else if (precision == PS_PREC_MIXED)
     k_link_setup<true, SETUP_IPT><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
         paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs,
         d_link_off,
-        d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_flag, ctx->d_tile_agg, ctx->d_tile_incl,
+        d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
         ctx->d_counters, ctx->d_status, n_tiles, (int64_t)0);
   else
     k_link_setup<false, SETUP_IPT><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
         paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs,
         d_link_off,
-        d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_flag, ctx->d_tile_agg, ctx->d_tile_incl,
+        d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
         ctx->d_counters, ctx->d_status, n_tiles, (int64_t)0);
   return ps_cuda_check(cudaGetLastError());
 }
@@ -2251,11 +2234,9 @@ int ps_run_segmented_prefix(ps_context* ctx, float* d_vals, const uint32_t* d_ta
   int64_t scan_tiles = (capacity + SCAN_TILE - 1) / SCAN_TILE;
   int rc = ps_ensure_tiles(ctx, scan_tiles + 2);
   if (rc != PS_OK) return rc;
-  cudaMemsetAsync(ctx->d_tile_flag, 0, sizeof(uint32_t) * (scan_tiles + 1), st);
-  cudaMemsetAsync(ctx->d_counters, 0, sizeof(int32_t) * 16, st);
+  cudaMemsetAsync(ctx->d_counters, 0, 64 + sizeof(TileState) * (scan_tiles + 1), st);
   if (d_path_tot && n_path > 0) cudaMemsetAsync(d_path_tot, 0, sizeof(float) * n_path, st);
   launch_arclen_scan(ctx, 0, st, d_vals, d_tag, d_n_rib, capacity, d_vals, d_path_tot,
-                     ctx->d_tile_flag, ctx->d_tile_aggd, ctx->d_tile_incld, ctx->d_counters,
-                     ctx->d_status);
+                     ctx->d_tile_state, ctx->d_counters, ctx->d_status);
   return ps_cuda_check(cudaGetLastError());
 }
