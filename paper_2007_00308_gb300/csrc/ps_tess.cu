@@ -1353,15 +1353,21 @@ __global__ void __launch_bounds__(SETUP_NT, 2) k_link_setup(
 }
 
 // ---------------------------------------------------------------------------
-// K2: ribs.  Each warp takes chunks of EMIT_CHUNK consecutive ribs and works
-// through them in slabs of 32, one rib per lane: the lane's link advances
-// monotonically from the chunk's first link (found by a 32-way search), the
-// rib's psi(j), t(j), g(t(j)) and n(j) are evaluated, and the rib, its tag and
-// the chord to the previous rib of the same link (the previous lane, the last
-// lane of the previous slab, or for the chunk's first rib a re-evaluation) are
-// written.  No block-wide synchronisation.
+// K2: ribs.  Each warp takes chunks of consecutive ribs and works through them in
+// slabs of 32, one rib per lane: the lane's link advances monotonically from the
+// chunk's first link (found by a 32-way search), the rib's psi(j), t(j), g(t(j)) and
+// n(j) are evaluated, and the rib, its tag and the chord to the previous rib of
+// the same link (the previous lane, or the last lane of the previous slab) are
+// written.  A chunk's first slab begins one rib early, at the rib that its first
+// chord starts from (an out-of-line re-evaluation of that rib was a second
+// copy of all the rib code).  No block-wide synchronisation.  The chunk length follows
+// the rib count: with 32 slabs whatever the count, 9,937 ribs kept ten warps of the chip
+// busy for 74 us, and 7.5 M ribs took three rounds over the warps and a sliver,
+// 414 us; 10 and 350 us this way, and 1.69 ms for 43 M ribs (1.74), 10.1 ms for the 211 M
+// of a million near-cusp cubics (12.2: their chunks' first ribs were often the
+// costly ones).
 constexpr int EMIT_NT = 256;
-constexpr int EMIT_K = 32;  // slabs of 32 ribs per chunk by default (tunable: 4, 8, 16, 32, 64)
+constexpr int EMIT_K = 32;  // most slabs of 32 ribs per chunk by default (tunable: 4, 8, 16, 32, 64)
 
 struct RibEval {
   float4 v;      // N.x N.y P.x P.y
@@ -1510,23 +1516,8 @@ __device__ __forceinline__ RibEval eval_rib(const LinkRec* __restrict__ L, int j
   else return eval_rib32(L, j);
 }
 
-// The same, out of line: the emitter's rare re-evaluation of a chunk's
-// preceding rib calls it, so the hot loop holds one copy of the rib code.
-template <bool MIXED>
-__device__ __noinline__ RibEval eval_rib_ool(const LinkRec* __restrict__ L, int j) {
-  return eval_rib<MIXED>(L, j);
-}
-
-__device__ __forceinline__ int64_t find_link(const int32_t* off, int64_t lo, int64_t hi, int64_t r) {
-  // last l in [lo, hi] with off[l] <= r  (off non-decreasing)
-  while (hi > lo) {
-    int64_t mid = (lo + hi + 1) >> 1;
-    if ((int64_t)__ldg(off + mid) <= r) lo = mid; else hi = mid - 1;
-  }
-  return lo;
-}
-
-// Warp-cooperative find_link over [0, n - 1] (off[0] <= r): 32 probes per round.
+// The last link l in [0, n - 1] with off[l] <= r (off non-decreasing, off[0] <= r): a
+// warp's 32 probes per round.
 __device__ __forceinline__ int64_t find_link_warp(const int32_t* off, int64_t n, int64_t r,
                                                   int lane) {
   int64_t lo = 0, hi = n - 1;  // off[lo] <= r, answer in [lo, hi]
@@ -1552,23 +1543,28 @@ __global__ void __launch_bounds__(EMIT_NT, MIXED ? 2 : 3) k_emit(
     const LinkRec* __restrict__ recs, const int32_t* __restrict__ link_off,
     const int32_t* __restrict__ link_path, int64_t n_link, const int64_t* __restrict__ n_rib,
     int64_t capacity, float4* __restrict__ rib, uint32_t* __restrict__ tag,
-    float* __restrict__ chord, float* __restrict__ tout, int emit_k) {
+    float* __restrict__ chord, float* __restrict__ tout, int most_slabs) {
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31;
-  const int64_t chunk = 32 * (int64_t)emit_k;
-  const int64_t n_chunks = (R + chunk - 1) / chunk;
-  const int64_t warp0 = ((int64_t)blockIdx.x * EMIT_NT + threadIdx.x) >> 5;
   const int64_t n_warps = ((int64_t)gridDim.x * EMIT_NT) >> 5;
-  for (int64_t c = warp0; c < n_chunks; c += n_warps) {
-    const int64_t r0 = c * chunk;
-    int64_t l = find_link_warp(link_off, n_link, r0, lane);
+  // slabs per chunk: as many as most_slabs, in as few rounds over the warps as
+  // that takes, evened out over the rounds
+  const int64_t most = n_warps * (32 * (int64_t)most_slabs - 1);
+  const int64_t rounds = (R + most - 1) / most;
+  const int slabs = rounds > 0 ? (int)(((R + n_warps * rounds - 1) / (n_warps * rounds) + 32) >> 5) : 1;
+  const int64_t chunk = 32 * (int64_t)slabs - 1;
+  const int64_t n_chunks = (R + chunk - 1) / chunk;
+  // consecutive chunks go to different CTAs, so that few chunks spread over the SMs
+  for (int64_t c = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x; c < n_chunks; c += n_warps) {
+    const int64_t r0 = c * chunk, r1 = r0 + chunk < R ? r0 + chunk : R;
+    int64_t l = find_link_warp(link_off, n_link, r0 > 0 ? r0 - 1 : 0, lane);
     float2 carry_g = mk(0.f, 0.f), carry_gl = mk(0.f, 0.f);
     float carry_t = 0.f, carry_tl = 0.f;
 #pragma unroll 1
-    for (int s = 0; s < emit_k; ++s) {
-      const int64_t r = r0 + (int64_t)s * 32 + lane;
-      const bool active = r < R;
+    for (int64_t rs = r0 - 1; rs < r1; rs += 32) {
+      const int64_t r = rs + lane;
+      const bool active = r >= 0 && r < r1, write = active && r >= r0;
       RibEval E;
       E.grel = mk(0.f, 0.f);
       E.glo = mk(0.f, 0.f);
@@ -1580,10 +1576,12 @@ __global__ void __launch_bounds__(EMIT_NT, MIXED ? 2 : 3) k_emit(
         while (l + 1 < n_link && (int64_t)__ldg(link_off + l + 1) <= r) ++l;
         j = (int)(r - __ldg(link_off + l));
         E = eval_rib<MIXED>(recs + l, j);
-        rib[r] = E.v;
-        uint32_t p = (uint32_t)__ldg(link_path + l);
-        tag[r] = (p << 2) | (E.seg ? PS_TAG_SEGMENT : 0u) | (j == 0 ? PS_TAG_LINK_START : 0u);
-        if (tout) tout[r] = E.t + E.tlo;
+        if (write) {
+          rib[r] = E.v;
+          uint32_t p = (uint32_t)__ldg(link_path + l);
+          tag[r] = (p << 2) | (E.seg ? PS_TAG_SEGMENT : 0u) | (j == 0 ? PS_TAG_LINK_START : 0u);
+          if (tout) tout[r] = E.t + E.tlo;
+        }
       }
       if (chord) {
         // rib r - 1 is in the same link iff j > 0
@@ -1610,23 +1608,14 @@ __global__ void __launch_bounds__(EMIT_NT, MIXED ? 2 : 3) k_emit(
         }
         carry_t = __shfl_sync(0xffffffffu, E.t, 31);
         if (MIXED) carry_tl = __shfl_sync(0xffffffffu, E.tlo, 31);
-        if (active) {
+        if (write) {
           float cl = 0.f;
-          if (E.seg && j > 0) {
-            if (lane == 0 && s == 0) {
-              RibEval Ep = eval_rib_ool<MIXED>(recs + l, j - 1);
-              pg = Ep.grel;
-              pgl = Ep.glo;
-              pt = Ep.t;
-              ptl = Ep.tlo;
-            }
-            // Sec. 7: a step whose t decreases adds no length.  The chord is
-            // differenced as pairs before rounding (MIXED).
-            if (E.t > pt || (E.t == pt && E.tlo >= ptl)) {
-              float dx = (E.grel.x - pg.x) + (E.glo.x - pgl.x);
-              float dy = (E.grel.y - pg.y) + (E.glo.y - pgl.y);
-              cl = sqrtf(dx * dx + dy * dy);
-            }
+          // Sec. 7: a step whose t decreases adds no length.  The chord is
+          // differenced as pairs before rounding (MIXED).
+          if (E.seg && j > 0 && (E.t > pt || (E.t == pt && E.tlo >= ptl))) {
+            float dx = (E.grel.x - pg.x) + (E.glo.x - pgl.x);
+            float dy = (E.grel.y - pg.y) + (E.glo.y - pgl.y);
+            cl = sqrtf(dx * dx + dy * dy);
           }
           chord[r] = cl;
         }
