@@ -65,10 +65,14 @@ int ps_ensure_quad_hits(ps_context* ctx, int64_t n_rib) {
 }
 
 int ps_persistent_grid(ps_context* ctx, const void* kernel, int block, size_t smem) {
+  for (int i = 0; i < ctx->n_occ; ++i)
+    if (ctx->occ[i].kernel == kernel) return ctx->num_sms * ctx->occ[i].per_sm;
   int per_sm = 0;
   if (cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, block, smem) != cudaSuccess ||
       per_sm < 1)
-    per_sm = 1;
+    return ctx->num_sms;
+  if (ctx->n_occ < (int)(sizeof(ctx->occ) / sizeof(ctx->occ[0])))
+    ctx->occ[ctx->n_occ++] = {kernel, per_sm};
   return ctx->num_sms * per_sm;
 }
 

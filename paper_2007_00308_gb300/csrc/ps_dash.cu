@@ -476,18 +476,15 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
   if ((rc = ps_ensure_quad_hits(ctx, capacity)) != PS_OK) return rc;  // 8 bytes per quad
   unsigned long long* word = reinterpret_cast<unsigned long long*>(ctx->d_quad_hits);
   const DashOut D{reinterpret_cast<float4*>(d_out_rib), d_out_s, d_out_tag, d_out_src, out_capacity};
-  // no more CTAs than there can be tiles or rounds
-  const int64_t most0 = (capacity + DASH_TILE - 1) / DASH_TILE;
-  const int64_t most1 = (capacity + DASH_NT / 32 * EMIT_WQ - 1) / (DASH_NT / 32 * EMIT_WQ);
-  int64_t grid0 = ps_persistent_grid(ctx, (const void*)k_dash_count, DASH_NT, 0);
-  int64_t grid1 = ps_persistent_grid(ctx, (const void*)k_dash, DASH_NT, 0);
-  if (grid0 > most0) grid0 = most0 > 0 ? most0 : 1;
-  if (grid1 > most1) grid1 = most1 > 0 ? most1 : 1;
+  const int grid0 =
+      ps_grid_for(ps_persistent_grid(ctx, (const void*)k_dash_count, DASH_NT, 0), capacity, DASH_TILE);
+  const int grid1 = ps_grid_for(ps_persistent_grid(ctx, (const void*)k_dash, DASH_NT, 0), capacity,
+                                DASH_NT / 32 * EMIT_WQ);
   ProfScope ps_(ctx, PK_DASH, st);
-  k_dash_count<<<(unsigned)grid0, DASH_NT, 0, st>>>(d_s, d_tag, d_n_rib, capacity, P, word, d_n_out,
+  k_dash_count<<<grid0, DASH_NT, 0, st>>>(d_s, d_tag, d_n_rib, capacity, P, word, d_n_out,
                                                     out_capacity, ctx->d_tile_state, ctx->d_counters,
                                                     ctx->d_status);
-  k_dash<<<(unsigned)grid1, DASH_NT, 0, st>>>(reinterpret_cast<const float4*>(d_rib), d_s, d_tag,
+  k_dash<<<grid1, DASH_NT, 0, st>>>(reinterpret_cast<const float4*>(d_rib), d_s, d_tag,
                                               d_n_rib, capacity, P, word, D, ctx->d_status);
   return ps_cuda_check(cudaGetLastError());
 }

@@ -73,6 +73,9 @@ struct ps_context {
   cudaEvent_t prof_ev[PK_COUNT][2];
   int prof_recorded[PK_COUNT];
   int device;
+  // CTAs per SM of the kernels launched so far (ps_persistent_grid)
+  struct { const void* kernel; int per_sm; } occ[24];
+  int n_occ;
   int cov_attr_done[2];  // coverage kernels' shared-memory attribute set on this device
   void* last_stream;
   int32_t* d_status;        // first error recorded by a kernel
@@ -93,7 +96,7 @@ struct ps_context {
   uint32_t* d_quad_hits;    // [2 quad_hits_cap] per-rib {hits, box} words of the binning passes
   int64_t quad_hits_cap;
   int64_t pair_cap;
-  int64_t* d_scratch64;     // 16 int64 of per-call scalars
+  int64_t* d_scratch64;     // 16 int64: the work counts of the last raster call
   int64_t last_n_tile;      // tiles of the most recent raster call
   uint32_t* d_mask_scratch; // per-CTA per-path tile masks beyond shared memory
   size_t d_scratch_words;
@@ -240,7 +243,14 @@ int ps_ensure_recs(ps_context* ctx, int64_t n_link);
 int ps_ensure_raster(ps_context* ctx, int64_t n_tile, int64_t n_pair);
 int ps_ensure_quad_hits(ps_context* ctx, int64_t n_rib);
 int ps_cuda_check(cudaError_t e);
+// A persistent kernel's CTAs: as many as the device holds at once.  The occupancy is asked for
+// once per context and kernel (a query costs about as much as a launch).
 int ps_persistent_grid(ps_context* ctx, const void* kernel, int block, size_t smem);
+// ... but no more than one per `per` of at most n items.
+static inline int ps_grid_for(int grid, int64_t n, int64_t per) {
+  const int64_t want = (n + per - 1) / per;
+  return want < grid ? (int)(want > 0 ? want : 1) : grid;
+}
 // Link setup (records in ctx->d_recs, link path indices after them) into the given
 // offset arrays; used by the adjoint to rebuild the forward's interval records.
 int ps_run_link_setup(ps_context* ctx, const ps_segments* seg, const ps_paths* paths, float dtheta,

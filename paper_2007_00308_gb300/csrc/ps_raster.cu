@@ -180,6 +180,34 @@ struct BinQuad {
 };
 constexpr int TALL_ROWS = 6;
 
+// What the count pass clears for the kernels after it (each a launch less than a memset of
+// its own): the canvas (tiles without entries are never visited by the coverage kernel), the
+// per-path counts, the tile scan's states, the tile tickets and the work counts.
+struct RasterClear {
+  uint16_t* canvas;
+  int64_t n_px;
+  unsigned long long* covered;
+  int n_path;
+  TileState* state;
+  int n_state;
+  int32_t* counters;           // 16
+  unsigned long long* stats;  // 7
+};
+__device__ __forceinline__ void raster_clear(const RasterClear& C) {
+  const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
+  const int64_t n = (int64_t)gridDim.x * blockDim.x;
+  // single pixels up to a 16-byte boundary, eight at a time, single ones again
+  const int64_t head = min(C.n_px, (int64_t)(((16 - (reinterpret_cast<uintptr_t>(C.canvas) & 15)) & 15) / 2));
+  const int64_t body = (C.n_px - head) / 8;
+  uint4* v = reinterpret_cast<uint4*>(C.canvas + head);
+  for (int64_t i = i0; i < body; i += n) v[i] = make_uint4(0u, 0u, 0u, 0u);
+  for (int64_t i = i0; i < C.n_px - 8 * body; i += n) C.canvas[i < head ? i : i + 8 * body] = 0;
+  for (int64_t i = i0; i < C.n_path; i += n) C.covered[i] = 0ull;
+  for (int64_t i = i0; i < C.n_state; i += n) C.state[i] = TileState{0ull, 0ull};
+  if (i0 < 16) C.counters[i0] = 0;
+  if (i0 < 7) C.stats[i0] = 0ull;
+}
+
 template <int PASS>
 __global__ void __launch_bounds__(BIN_NT) k_bin(const float4* __restrict__ rib,
                                                 const uint32_t* __restrict__ tag,
@@ -191,13 +219,14 @@ __global__ void __launch_bounds__(BIN_NT) k_bin(const float4* __restrict__ rib,
                                                 uint32_t* __restrict__ bin, int64_t pair_cap,
                                                 uint2* __restrict__ hits,
                                                 int32_t* __restrict__ back,  // short fill, from the end
-                                                int32_t* status) {
+                                                RasterClear clear, int32_t* status) {
   __shared__ BinQuad s_q[BIN_NT];
   __shared__ int s_pre[BIN_NT / 32][33];
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   BinQuad* wq = s_q + wid * 32;
+  if (PASS == 0) raster_clear(clear);
   int64_t stride = (int64_t)gridDim.x * BIN_NT;
   for (int64_t base = (int64_t)blockIdx.x * BIN_NT; base < R; base += stride) {
     const int64_t r = base + threadIdx.x;
@@ -1285,6 +1314,8 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
   __shared__ __align__(16) float4 s_pre_rib[CV_WARPS][2][32];
   __shared__ uint32_t s_pre_tag[CV_WARPS][32];
 
+  const int n_list = tile_list[n_tile];  // tiles with entries (the canvas is cleared)
+  if ((int)blockIdx.x >= n_list) return;  // the others' tickets reach every tile
   for (int i = threadIdx.x; i < SLOTS * MASK_WORDS; i += CV_NT) s_mask[i] = 0u;
   for (int i = threadIdx.x; i < MASK_WORDS; i += CV_NT) s_canvas[i] = 0u;
   if (EXACT)
@@ -1315,7 +1346,6 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
   // tile's last pass reaches its flush, and read when the tile ends, so its
   // latency hides behind the flush (claiming earlier would hold a tile back
   // from an idle CTA)
-  const int n_list = tile_list[n_tile];  // tiles with entries (the canvas is cleared)
   if (threadIdx.x == 0) s_tile = atomicAdd(&counters[2], 1);
   bool dirty = true;  // the path hash holds the previous tile's keys
   for (;;) {
@@ -1629,27 +1659,29 @@ static int rasterize(ps_context* ctx, const float* d_rib, const uint32_t* d_tag,
   int grid_cov = ps_persistent_grid(ctx, kcov, CV_NT, cov_smem);
   ctx->last_n_tile = n_tile;
   cudaMemsetAsync(ctx->d_tile_count, 0, sizeof(int32_t) * (n_tile + 1), st);
-  cudaMemsetAsync(ctx->d_counters, 0, 64 + sizeof(TileState) * ((n_tile + TS_TILE - 1) / TS_TILE + 1), st);
-  cudaMemsetAsync(d_covered, 0, sizeof(uint64_t) * (size_t)n_path, st);
-  // tiles without entries are never visited by the coverage kernel
-  cudaMemsetAsync(d_canvas, 0, sizeof(uint16_t) * (size_t)width * (size_t)height, st);
-  cudaMemsetAsync(ctx->d_scratch64, 0, 7 * sizeof(int64_t), st);
+  const int ts_grid = (int)((n_tile + TS_TILE - 1) / TS_TILE);
+  const RasterClear clear{d_canvas, (int64_t)width * height,
+                          reinterpret_cast<unsigned long long*>(d_covered), n_path,
+                          ctx->d_tile_state, ts_grid + 1, ctx->d_counters,
+                          reinterpret_cast<unsigned long long*>(ctx->d_scratch64)};
   // persistent grids, each pass at its own occupancy (the count pass holds more
   // registers)
+  // (the count pass has the canvas to clear as well)
   int grid_bin = ctx->tune[PS_TUNE_BIN_BLOCKS] > 0
                      ? ctx->num_sms * ctx->tune[PS_TUNE_BIN_BLOCKS]
-                     : ps_persistent_grid(ctx, (const void*)k_bin<0>, BIN_NT, 0);
+                     : ps_grid_for(ps_persistent_grid(ctx, (const void*)k_bin<0>, BIN_NT, 0),
+                                   capacity + clear.n_px / 16, BIN_NT);
   int grid_bin1 = ctx->tune[PS_TUNE_BIN_BLOCKS] > 0
                       ? grid_bin
-                      : ps_persistent_grid(ctx, (const void*)k_bin<1>, BIN_NT, 0);
+                      : ps_grid_for(ps_persistent_grid(ctx, (const void*)k_bin<1>, BIN_NT, 0),
+                                    capacity, BIN_NT);
   const float4* rib = reinterpret_cast<const float4*>(d_rib);
   { ProfScope ps_(ctx, PK_BIN_COUNT, st);
   k_bin<0><<<grid_bin, BIN_NT, 0, st>>>(rib, d_tag, d_n_rib, capacity, width, height, y0, tiles_x,
                                       ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,
                                       ctx->d_bin, ctx->pair_cap, reinterpret_cast<uint2*>(ctx->d_quad_hits), ctx->d_tile_cursor + n_tile + 1,
-                                      ctx->d_status); }
+                                      clear, ctx->d_status); }
   { ProfScope ps_(ctx, PK_TILE_SCAN, st);
-  const int ts_grid = (int)((n_tile + TS_TILE - 1) / TS_TILE);
   k_tile_scan<<<ts_grid, TS_NT, 0, st>>>(ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,
                                          ctx->d_tile_list, (int)n_tile, ctx->pair_cap,
                                          ctx->d_tile_state, ctx->d_status); }
@@ -1657,7 +1689,7 @@ static int rasterize(ps_context* ctx, const float* d_rib, const uint32_t* d_tag,
   k_bin<1><<<grid_bin1, BIN_NT, 0, st>>>(rib, d_tag, d_n_rib, capacity, width, height, y0, tiles_x,
                                       ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,
                                       ctx->d_bin, ctx->pair_cap, reinterpret_cast<uint2*>(ctx->d_quad_hits), ctx->d_tile_cursor + n_tile + 1,
-                                      ctx->d_status); }
+                                      clear, ctx->d_status); }
   { ProfScope ps_(ctx, PK_COVERAGE, st);
 #define PS_COV_ARGS                                                                              \
   rib, d_tag, ctx->d_tile_off, ctx->d_bin, ctx->pair_cap, width, height, y0, tiles_x, (int)n_tile, \

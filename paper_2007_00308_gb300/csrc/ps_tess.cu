@@ -1245,8 +1245,8 @@ __global__ void __launch_bounds__(SETUP_NT, 2) k_link_setup(
     const int32_t* __restrict__ seg_off, const float* __restrict__ width,
     const uint8_t* __restrict__ join, const uint8_t* __restrict__ cap,
     const float* __restrict__ miter, const uint8_t* __restrict__ closed, int n_path,
-    int64_t n_link, float q, float tau, LinkRec* __restrict__ recs, int32_t* __restrict__ link_off,
-    int32_t* __restrict__ path_off, int64_t* __restrict__ n_rib_out, int64_t capacity,
+    int64_t n_link, float q, float tau, LinkRec* __restrict__ recs, int32_t* __restrict__ link_path,
+    float* __restrict__ path_len, int32_t* __restrict__ link_off, int32_t* __restrict__ path_off, int64_t* __restrict__ n_rib_out, int64_t capacity,
     TileState* state, int32_t* counters, int32_t* status, int64_t n_tiles, int64_t l_begin) {
   __shared__ long long sm[SETUP_NT / 32 + 1];
   __shared__ long long s_prefix;
@@ -1339,7 +1339,11 @@ __global__ void __launch_bounds__(SETUP_NT, 2) k_link_setup(
       if (off > 0x7fffffffLL) ps_record_error(status, PS_ERR_CAPACITY);
       link_off[l] = (int32_t)off;
       const int p = s_pth[li], kk = s_kk[li];
-      if (kk == 0) path_off[p] = (int32_t)off;
+      link_path[l] = p;  // for the rib tags
+      if (kk == 0) {
+        path_off[p] = (int32_t)off;
+        if (path_len) path_len[p] = 0.f;  // for a path without ribs
+      }
       off += s_cnt[li];
       if (l == n_link - 1) {
         link_off[n_link] = (int32_t)off;
@@ -1624,14 +1628,6 @@ __global__ void __launch_bounds__(EMIT_NT, MIXED ? 2 : 3) k_emit(
   }
 }
 
-// Path index of every link (for the rib tags).
-__global__ void k_link_path(const int32_t* __restrict__ seg_off, int n_path, int64_t n_link,
-                            int32_t* __restrict__ link_path, int64_t l_begin) {
-  int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  if (l >= n_link) return;
-  link_path[l] = find_path(seg_off, n_path, l_begin + l);
-}
-
 // ---------------------------------------------------------------------------
 // K3: segmented inclusive scan of per-rib chords into cumulative arc length
 // (Eq. 18), restarting at every path's first rib.  The tessellation runs it in
@@ -1795,7 +1791,8 @@ static void launch_arclen_scan(ps_context* ctx, int grid_override, cudaStream_t 
   const bool vec = ((reinterpret_cast<uintptr_t>(chord) | reinterpret_cast<uintptr_t>(tag) |
                      reinterpret_cast<uintptr_t>(s_out)) & 15u) == 0;
   const void* fn = vec ? (const void*)k_arclen_scan<true> : (const void*)k_arclen_scan<false>;
-  int g = grid_override > 0 ? grid_override : ps_persistent_grid(ctx, fn, SCAN_NT, 0);
+  const int g = ps_grid_for(
+      grid_override > 0 ? grid_override : ps_persistent_grid(ctx, fn, SCAN_NT, 0), capacity, SCAN_TILE);
   if (vec)
     k_arclen_scan<true><<<g, SCAN_NT, 0, st>>>(chord, tag, n_rib, capacity, s_out, path_len,
                                                state, counters, status);
@@ -1852,15 +1849,18 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
   const bool arc = !(flags & PS_TESS_COUNT_ONLY) && (flags & PS_TESS_ARCLENGTH) && out->d_s;
   cudaMemsetAsync(ctx->d_counters, 0,
                   64 + sizeof(TileState) * (n_tiles + (arc ? scan_tiles + 2 : 0)), st);
+  // the set-up clears the lengths of the paths that begin in the range: all paths of a whole
+  // batch; a range call's others are cleared here
+  const bool set_len = arc && out->d_path_len, whole = l0 == 0 && L == 2 * seg->n_seg + P;
+  if (set_len && !whole) cudaMemsetAsync(out->d_path_len, 0, sizeof(float) * P, st);
   // a count-only call has no rib buffers to overflow
   int64_t count_cap = (flags & PS_TESS_COUNT_ONLY) ? INT64_MAX : out->capacity;
-  { ProfScope ps_(ctx, PK_LINK_PATH, st);
-  k_link_path<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(paths->d_seg_off, P, L, link_path, l0); }
   {
   ProfScope ps_(ctx, PK_LINK_SETUP, st);
 #define PS_SETUP_ARGS                                                                          \
   seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,         \
       paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs, \
+      link_path, set_len ? out->d_path_len : nullptr,                                          \
       out->d_link_rib_off, out->d_path_rib_off, out->d_n_rib, count_cap, ctx->d_tile_state,   \
       ctx->d_counters, ctx->d_status, n_tiles, l0
   const unsigned g = (unsigned)n_tiles;
@@ -1884,7 +1884,7 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
   if (flags & PS_TESS_COUNT_ONLY) return PS_OK;
 
   const void* fn = precision == PS_PREC_MIXED ? (const void*)k_emit<true> : (const void*)k_emit<false>;
-  int grid = ps_persistent_grid(ctx, fn, EMIT_NT, 0);
+  const int grid = ps_grid_for(ps_persistent_grid(ctx, fn, EMIT_NT, 0), out->capacity, 31);
   {
   ProfScope ps_(ctx, PK_EMIT, st);
 #define PS_EMIT_ARGS                                                                           \
@@ -1899,7 +1899,6 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
   if (arc) {
     // the emitter wrote each rib's chord into s; the segmented scan turns them
     // into cumulative arc length in place
-    if (out->d_path_len) cudaMemsetAsync(out->d_path_len, 0, sizeof(float) * P, st);
     ProfScope ps_(ctx, PK_ARCLEN, st);
     launch_arclen_scan(ctx, 0, st, out->d_s, out->d_tag, out->d_n_rib, out->capacity, out->d_s,
                        out->d_path_len, ctx->d_tile_state + n_tiles + 1, ctx->d_counters,
@@ -2129,17 +2128,18 @@ extern "C" int ps_tessellate_strokes_noalloc(const ps_segments* seg, const ps_pa
   if (cudaMemsetAsync(counters, 0, 64 + sizeof(TileState) * NOALLOC_TILES, st) != cudaSuccess)
     return PS_ERR_CUDA;
   int64_t count_cap = count_only ? INT64_MAX : out->capacity;
-  k_link_path<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(paths->d_seg_off, P, L, link_path, (int64_t)0);
   if (precision == PS_PREC_MIXED)
     k_link_setup<true, SETUP_IPT><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
-        paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, 0.f, recs, out->d_link_rib_off,
+        paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, 0.f, recs, link_path,
+        arc ? out->d_path_len : nullptr, out->d_link_rib_off,
         out->d_path_rib_off, out->d_n_rib, count_cap, state, counters, d_status,
         n_tiles, (int64_t)0);
   else
     k_link_setup<false, SETUP_IPT><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
-        paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, 0.f, recs, out->d_link_rib_off,
+        paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, 0.f, recs, link_path,
+        arc ? out->d_path_len : nullptr, out->d_link_rib_off,
         out->d_path_rib_off, out->d_n_rib, count_cap, state, counters, d_status,
         n_tiles, (int64_t)0);
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
@@ -2159,8 +2159,6 @@ extern "C" int ps_tessellate_strokes_noalloc(const ps_segments* seg, const ps_pa
                                             out->d_tag, arc ? out->d_s : nullptr, out->d_t, EMIT_K);
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   if (arc) {
-    if (out->d_path_len && cudaMemsetAsync(out->d_path_len, 0, sizeof(float) * P, st) != cudaSuccess)
-      return PS_ERR_CUDA;
     int per_sm2 = 1;
     cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm2, (const void*)k_arclen_scan<true>,
                                                   SCAN_NT, 0);
@@ -2186,33 +2184,30 @@ int ps_run_link_setup(ps_context* ctx, const ps_segments* seg, const ps_paths* p
   if ((rc = ps_ensure_recs(ctx, L)) != PS_OK) return rc;
   int32_t* link_path = reinterpret_cast<int32_t*>(ctx->d_recs + ctx->rec_cap);
   cudaMemsetAsync(ctx->d_counters, 0, 64 + sizeof(TileState) * n_tiles, st);
-  k_link_path<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(paths->d_seg_off, P, L, link_path, (int64_t)0);
   const bool px = ctx->pixel_tol > 0.f;
   if (precision == PS_PREC_MIXED && px)
     k_link_setup<true, SETUP_IPT, true><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
         paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs,
-        d_link_off, d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
+        link_path, nullptr, d_link_off, d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
         ctx->d_counters, ctx->d_status, n_tiles, (int64_t)0);
   else if (px)
     k_link_setup<false, SETUP_IPT, true><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
         paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs,
-        d_link_off, d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
+        link_path, nullptr, d_link_off, d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
         ctx->d_counters, ctx->d_status, n_tiles, (int64_t)0);
   else if (precision == PS_PREC_MIXED)
     k_link_setup<true, SETUP_IPT><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
         paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs,
-        d_link_off,
-        d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
+        link_path, nullptr, d_link_off, d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
         ctx->d_counters, ctx->d_status, n_tiles, (int64_t)0);
   else
     k_link_setup<false, SETUP_IPT><<<(unsigned)n_tiles, SETUP_NT, 0, st>>>(
         seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,
         paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs,
-        d_link_off,
-        d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
+        link_path, nullptr, d_link_off, d_path_off, d_n_rib, INT64_MAX, ctx->d_tile_state,
         ctx->d_counters, ctx->d_status, n_tiles, (int64_t)0);
   return ps_cuda_check(cudaGetLastError());
 }
