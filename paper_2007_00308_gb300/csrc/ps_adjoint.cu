@@ -180,14 +180,6 @@ __device__ __forceinline__ float2 dang(float2 v) {
   return l2 > 0.f ? mk(-v.y / l2, v.x / l2) : mk(0.f, 0.f);
 }
 
-__device__ __forceinline__ int find_link_a(const int32_t* off, int64_t lo, int64_t hi, int64_t r) {
-  while (hi > lo) {
-    int64_t mid = (lo + hi + 1) >> 1;
-    if ((int64_t)__ldg(off + mid) <= r) lo = mid; else hi = mid - 1;
-  }
-  return (int)lo;
-}
-
 __global__ void k_adj_links(const uint8_t* st, const float* sp, const float* sw,
                             const int32_t* seg_off, const uint8_t* closed, int n_path,
                             int64_t n_link, int4* src) {
@@ -199,48 +191,80 @@ __global__ void k_adj_links(const uint8_t* st, const float* sp, const float* sw,
   src[l] = make_int4(R.kind, a, b, R.path);
 }
 
-// Sum of v over the lanes from this one to the end of its run of equal keys
-// (runs of a key are contiguous); exact at the run's first lane.
-__device__ __forceinline__ float run_sum(float v, long long key) {
+// Runs of lanes that add to the same target (runs are contiguous).  heads: the lanes that
+// begin a run; end: the last lane of this lane's run.
+struct Runs {
+  uint32_t heads;
+  int end;
+};
+__device__ __forceinline__ Runs runs_of(bool differs_from_previous) {
+  const int lane = threadIdx.x & 31;
+  Runs R;
+  R.heads = __ballot_sync(0xffffffffu, lane == 0 || differs_from_previous);
+  const uint32_t later = lane < 31 ? R.heads >> (lane + 1) : 0u;
+  R.end = later ? lane + __ffs(later) - 1 : 31;
+  return R;
+}
+// Sum of v over the lanes from this one to the end of its run; exact at the run's first lane.
+__device__ __forceinline__ float run_sum(float v, const Runs& R) {
   const int lane = threadIdx.x & 31;
 #pragma unroll
   for (int o = 1; o < 32; o <<= 1) {
-    float y = __shfl_down_sync(0xffffffffu, v, o);
-    long long ky = __shfl_down_sync(0xffffffffu, key, o);
-    if (lane + o < 32 && ky == key) v += y;
+    const float y = __shfl_down_sync(0xffffffffu, v, o);
+    if (lane + o <= R.end) v += y;
   }
   return v;
 }
-
-__device__ __forceinline__ bool run_head(long long key) {
-  long long kp = __shfl_up_sync(0xffffffffu, key, 1);
-  return (threadIdx.x & 31) == 0 || kp != key;
+// Sums of 16 values over the whole warp, in halves: each step adds one half of the
+// values across the lanes and passes the other half on (16 shuffles instead of
+// 80).  Lane k returns the sum of value k >> 1.
+__device__ __forceinline__ float sum16(float* v) {
+  const int lane = threadIdx.x & 31;
+#pragma unroll
+  for (int h = 8; h >= 1; h >>= 1) {
+    const bool up = (lane & (2 * h)) != 0;
+#pragma unroll
+    for (int i = 0; i < h; ++i) {
+      const float give = up ? v[i] : v[i + h], keep = up ? v[i + h] : v[i];
+      v[i] = keep + __shfl_xor_sync(0xffffffffu, give, 2 * h);
+    }
+  }
+  return v[0] + __shfl_xor_sync(0xffffffffu, v[0], 1);
 }
 
 // Per rib: gradients of g(t_j), psi_j, r, for the control points, the link's
-// boundary-angle adjoints and the path width.  A warp takes 32 consecutive
-// ribs (mostly of one link), sums their contributions per target with
-// segmented shuffles, and the first lane of each run adds them atomically:
-// every rib of a segment adds to the same few words, so adding per rib would
-// serialize on them.
+// boundary-angle adjoints and the path width.  A warp takes chunks of consecutive
+// ribs in slabs of 32 (mostly of one link), sums their contributions per target
+// with shuffles, and adds them atomically: every rib of a segment adds to the
+// same few words, so adding per rib would serialize on them.  The chunk's first
+// link is searched once, by the warp.  A slab's lanes 0 and 31 are its neighbours, so that
+// the chords on either side come by shuffle.  (A binary search by one lane for
+// every 32 ribs, keys shuffled with every value of the sums, and the neighbours'
+// points evaluated again by the outer lanes took 1,272 us on 13.2 M ribs; 910 us
+// without the first two, 645 us without the third.)
+//   dL/ds enters as its reverse (suffix) sums over the path, total - prefix + own
+// value, formed here from the inclusive prefix.
 __global__ void __launch_bounds__(256) k_adj_ribs(
     const LinkRec* __restrict__ recs, const int4* __restrict__ src,
     const int32_t* __restrict__ link_off, int64_t n_link, const int64_t* __restrict__ n_rib,
-    int64_t capacity, const float4* __restrict__ rib, const float* __restrict__ tf,
-    const float4* __restrict__ grib, const float* __restrict__ suffix,
-    const uint8_t* __restrict__ stype, float* __restrict__ gpts, float* __restrict__ adj_psi,
-    float* __restrict__ gwidth) {
+    int64_t capacity, const float* __restrict__ tf, const float4* __restrict__ grib,
+    const float* __restrict__ gs, const float* __restrict__ pre, const float* __restrict__ tot,
+    float* __restrict__ gpts, float* __restrict__ adj_psi, float* __restrict__ gwidth) {
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31;
-  for (int64_t base = blockIdx.x * (int64_t)blockDim.x + (threadIdx.x & ~31); base < R;
-       base += (int64_t)gridDim.x * blockDim.x) {
+  const int64_t n_warps = ((int64_t)gridDim.x * blockDim.x) >> 5;
+  constexpr int USE = 30;  // lanes 1 .. 30 of a slab are its ribs, 0 and 31 their neighbours
+  const int64_t slabs = (R + USE - 1) / USE;
+  const int64_t per = (slabs + n_warps - 1) / n_warps;  // one chunk per warp
+  const int64_t c = (int64_t)(threadIdx.x >> 5) * gridDim.x + blockIdx.x;
+  const int64_t first = c * per * USE, last = first + per * USE < R ? first + per * USE : R;
+  if (first >= last) return;
+  int l = (int)find_link_warp(link_off, n_link, first > 0 ? first - 1 : 0, lane);
+  for (int64_t base = first - 1; base < last - 1; base += USE) {
     const int64_t r = base + lane;
-    const bool act = r < R;
-    // link of rib r: one search for the warp's first rib, then a short walk
-    int l = 0;
-    if (lane == 0) l = find_link_a(link_off, 0, n_link - 1, base);
-    l = __shfl_sync(0xffffffffu, l, 0);
+    const bool act = r >= 0 && r < R;
+    const bool use = act && lane >= 1 && lane <= USE && r < last;
     if (act)
       while (l + 1 < n_link && (int64_t)__ldg(link_off + l + 1) <= r) ++l;
     // this rib's contributions: point gradients of segment seg_t (slots 0..3),
@@ -252,14 +276,16 @@ __global__ void __launch_bounds__(256) k_adj_ribs(
     const uint32_t meta = act ? __ldg(&L->meta) : 0u;
     const int kind = META_KIND(meta);
     const int j = act ? (int)(r - __ldg(link_off + l)) : 0;
-    const int nr = act ? __ldg(link_off + l + 1) - __ldg(link_off + l) : 0;
-    // The chords of Eq. 18 beside this rib: their directions from the
-    // centreline points g(t) - A in double-float, differenced before rounding
-    // (a short chord between points far from A keeps its direction); the
-    // neighbours' points come from the neighbouring lanes of the same link.
+    // The chord of Eq. 18 from the previous rib of the link: its direction from
+    // the centreline points g(t) - A in double-float, differenced before
+    // rounding (a short chord between points far from A keeps its direction),
+    // times dL/ds of the ribs from r on.  The neighbours' points and chords come
+    // from the neighbouring lanes.
     Seg g;
     float t = 0.f;
     DF2 gc{{0.f, 0.f}, {0.f, 0.f}};
+    int4 sc = make_int4(0, -1, -1, 0);
+    if (act) sc = __ldg(src + l);
     if (kind == LK_SEG) {
       const float4 p01 = __ldg(reinterpret_cast<const float4*>(L->P));
       const float4 p23 = __ldg(reinterpret_cast<const float4*>(L->P) + 1);
@@ -269,21 +295,26 @@ __global__ void __launch_bounds__(256) k_adj_ribs(
       t = __ldg(tf + r);
       gc = g_rel_comp_df(g, t);
     }
-    DF2 gprev, gnext;
-    gprev.x.hi = __shfl_up_sync(0xffffffffu, gc.x.hi, 1);
-    gprev.x.lo = __shfl_up_sync(0xffffffffu, gc.x.lo, 1);
-    gprev.y.hi = __shfl_up_sync(0xffffffffu, gc.y.hi, 1);
-    gprev.y.lo = __shfl_up_sync(0xffffffffu, gc.y.lo, 1);
-    gnext.x.hi = __shfl_down_sync(0xffffffffu, gc.x.hi, 1);
-    gnext.x.lo = __shfl_down_sync(0xffffffffu, gc.x.lo, 1);
-    gnext.y.hi = __shfl_down_sync(0xffffffffu, gc.y.hi, 1);
-    gnext.y.lo = __shfl_down_sync(0xffffffffu, gc.y.lo, 1);
-    if (kind == LK_SEG) {
-      if (lane == 0 && j > 0) gprev = g_rel_comp_df(g, __ldg(tf + r - 1));
-      if (lane == 31 && j + 1 < nr) gnext = g_rel_comp_df(g, __ldg(tf + r + 1));
+    float2 chord = mk(0.f, 0.f);
+    if (gs) {
+      DF2 gprev;
+      gprev.x.hi = __shfl_up_sync(0xffffffffu, gc.x.hi, 1);
+      gprev.x.lo = __shfl_up_sync(0xffffffffu, gc.x.lo, 1);
+      gprev.y.hi = __shfl_up_sync(0xffffffffu, gc.y.hi, 1);
+      gprev.y.lo = __shfl_up_sync(0xffffffffu, gc.y.lo, 1);
+      const float tprev = __shfl_up_sync(0xffffffffu, t, 1);
+      // (a step with decreasing t adds no length)
+      if (kind == LK_SEG && lane > 0 && j > 0 && t >= tprev) {
+        const float2 d = mk(df_f(df_sub(gc.x, gprev.x)), df_f(df_sub(gc.y, gprev.y)));
+        const float len = sqrtf(dot2(d, d));
+        const float suffix = __ldg(tot + sc.w) - __ldg(pre + r) + __ldg(gs + r);
+        if (len > 0.f) chord = d * (suffix / len);
+      }
     }
-    if (act) {
-    int4 sc = __ldg(src + l);
+    // the next rib's chord, when it is of the same link (else it is 0: its j is 0)
+    const float2 chord_n = mk(__shfl_down_sync(0xffffffffu, chord.x, 1),
+                              __shfl_down_sync(0xffffffffu, chord.y, 1));
+    if (use) {
     float4 G = __ldg(grib + r);
     float2 GN = mk(G.x, G.y), GP = mk(G.z, G.w);
     float rN = __ldg(&L->rN), rP = __ldg(&L->rP);
@@ -304,18 +335,8 @@ __global__ void __launch_bounds__(256) k_adj_ribs(
       sincosf(psi, &sn, &cs);
       float2 n = mk(-sn, cs), T = mk(cs, sn);
       // upstream on the centreline point: both vertices, and the chords to the
-      // neighbouring ribs of this link (Eq. 18; a step with decreasing t adds 0)
-      float2 Gg = GN + GP;
-      if (j > 0 && t >= __ldg(tf + r - 1)) {
-        float2 d = mk(df_f(df_sub(gc.x, gprev.x)), df_f(df_sub(gc.y, gprev.y)));
-        float len = sqrtf(dot2(d, d));
-        if (len > 0.f) Gg = Gg + d * (__ldg(suffix + r) / len);
-      }
-      if (j + 1 < nr && __ldg(tf + r + 1) >= t) {
-        float2 d = mk(df_f(df_sub(gnext.x, gc.x)), df_f(df_sub(gnext.y, gc.y)));
-        float len = sqrtf(dot2(d, d));
-        if (len > 0.f) Gg = Gg - d * (__ldg(suffix + r + 1) / len);
-      }
+      // neighbouring ribs of this link
+      const float2 Gg = GN + GP + chord - chord_n;
       // N = g - rN n, P = g + rP n: dN/dpsi = rN T, dP/dpsi = -rP T
       float Gpsi = rN * dot2(T, GN) - rP * dot2(T, GP);
       float Gr = -dot2(n, GN) + dot2(n, GP);  // rN = rP = w/2 on segment links
@@ -411,23 +432,47 @@ __global__ void __launch_bounds__(256) k_adj_ribs(
         }
       }
     }
-    }  // act
+    }  // use
     // sums per link (points, width) and per (link, interval) (angles)
-    const long long key1 = act ? (long long)l : -1 - (long long)lane;
-    const long long key2 = act ? 8 * (long long)l + kslot : -1 - (long long)lane;
-    const bool h1 = run_head(key1), h2 = run_head(key2);
+    // (the neighbours' lanes add zeros to whatever run they fall in)
+    const int lp = __shfl_up_sync(0xffffffffu, l, 1), kp = __shfl_up_sync(0xffffffffu, kslot, 1);
+    const bool new1 = use && lane > 1 && l != lp, new2 = new1 || (use && lane > 1 && kslot != kp);
+    const Runs r2 = runs_of(new2);
+    if (r2.heads == 1u) {  // all of one interval: lane 1 speaks for them
+      const int seg_1 = __shfl_sync(0xffffffffu, seg_t, 1), path_1 = __shfl_sync(0xffffffffu, path_t, 1);
+      const int64_t slot_1 = 8 * (int64_t)__shfl_sync(0xffffffffu, l, 1) +
+                             __shfl_sync(0xffffffffu, kslot, 1);
+      float v[16] = {P8[0], P8[1], P8[2], P8[3], P8[4], P8[5], P8[6], P8[7],
+                     gw, psA, psB, 0.f, 0.f, 0.f, 0.f, 0.f};
+      const float sum = sum16(v);
+      const int i = lane >> 1;
+      if (!(lane & 1) && sum != 0.f) {
+        if (i < 8) {
+          if (seg_1 >= 0) atomicAdd(gpts + 8 * (int64_t)seg_1 + i, sum);
+        } else if (i == 8) {
+          if (path_1 >= 0) atomicAdd(gwidth + path_1, sum);
+        } else {
+          atomicAdd(adj_psi + slot_1 + (i - 9), sum);
+        }
+      }
+      continue;
+    }
+    const Runs r1 = runs_of(new1);
+    // (the first run begins at lane 0, whose values are 0, and is added by lane 1)
+    const bool h1 = use && (lane == 1 || ((r1.heads >> lane) & 1u));
+    const bool h2 = use && (lane == 1 || ((r2.heads >> lane) & 1u));
 #pragma unroll
     for (int i = 0; i < 8; ++i) {
-      float v = run_sum(P8[i], key1);
+      float v = run_sum(P8[i], r1);
       if (h1 && seg_t >= 0 && v != 0.f) atomicAdd(gpts + 8 * (int64_t)seg_t + i, v);
     }
     {
-      float v = run_sum(gw, key1);
+      float v = run_sum(gw, r1);
       if (h1 && path_t >= 0 && v != 0.f) atomicAdd(gwidth + path_t, v);
     }
     {
-      float a = run_sum(psA, key2), b = run_sum(psB, key2);
-      if (h2 && act) {
+      float a = run_sum(psA, r2), b = run_sum(psB, r2);
+      if (h2) {
         if (a != 0.f) atomicAdd(adj_psi + 8 * (int64_t)l + kslot, a);
         if (b != 0.f) atomicAdd(adj_psi + 8 * (int64_t)l + kslot + 1, b);
       }
@@ -493,16 +538,6 @@ __global__ void k_adj_finalize(const LinkRec* __restrict__ recs, const int4* __r
   }
 }
 
-// suffix[r] = sum of dL/ds over ribs >= r of r's path = total - prefix + own
-__global__ void k_adj_suffix(float* suf, const float* g, const float* tot, const uint32_t* tag,
-                             const int64_t* n_rib, int64_t cap) {
-  int64_t R = *n_rib;
-  if (R > cap) R = cap;
-  for (int64_t r = blockIdx.x * (int64_t)blockDim.x + threadIdx.x; r < R;
-       r += (int64_t)gridDim.x * blockDim.x)
-    suf[r] = tot[tag[r] >> 2] - suf[r] + g[r];
-}
-
 }  // namespace
 
 extern "C" int ps_tessellate_backward(ps_context* ctx, const ps_segments* seg,
@@ -552,25 +587,19 @@ extern "C" int ps_tessellate_backward(ps_context* ctx, const ps_segments* seg,
   k_adj_links<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(seg->d_type, seg->d_pts, seg->d_w,
                                                           paths->d_seg_off, paths->d_closed, P, L,
                                                           src);
-  // suffix sums of dL/ds within each path: total - inclusive prefix + own value
-  cudaMemsetAsync(suf, 0, sizeof(float) * (cap + 1), st);
-  if (d_grad_s) {
-    cudaMemcpyAsync(suf, d_grad_s, sizeof(float) * cap, cudaMemcpyDeviceToDevice, st);
-    if ((rc = ps_run_segmented_prefix(ctx, suf, fwd->d_tag, fwd->d_n_rib, cap, tot, P, st)) != PS_OK)
-      return rc;
-  }
+  // prefix sums of dL/ds within each path, and their totals
+  if (d_grad_s &&
+      (rc = ps_run_segmented_prefix(ctx, d_grad_s, suf, fwd->d_tag, fwd->d_n_rib, cap, tot, P, st)) !=
+          PS_OK)
+    return rc;
   cudaMemsetAsync(adj, 0, sizeof(float) * 8 * L, st);
   cudaMemsetAsync(d_grad_pts, 0, sizeof(float) * 8 * S, st);
   cudaMemsetAsync(d_grad_width, 0, sizeof(float) * P, st);
-  // convert prefix -> suffix in place
-  if (d_grad_s)
-    k_adj_suffix<<<ctx->num_sms * 8, 256, 0, st>>>(suf, d_grad_s, tot, fwd->d_tag, fwd->d_n_rib,
-                                                  cap);
-  int grid = ctx->num_sms * 8;
+  const int grid =
+      ps_grid_for(ps_persistent_grid(ctx, (const void*)k_adj_ribs, 256, 0), cap, 32);
   k_adj_ribs<<<grid, 256, 0, st>>>(ctx->d_recs, src, fwd->d_link_rib_off, L, fwd->d_n_rib, cap,
-                                   reinterpret_cast<const float4*>(fwd->d_rib), fwd->d_t,
-                                   reinterpret_cast<const float4*>(d_grad_rib), suf, seg->d_type,
-                                   d_grad_pts, adj, d_grad_width);
+                                   fwd->d_t, reinterpret_cast<const float4*>(d_grad_rib), d_grad_s,
+                                   suf, tot, d_grad_pts, adj, d_grad_width);
   k_adj_finalize<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(ctx->d_recs, src, L, seg->d_type,
                                                               seg->d_pts, seg->d_w, adj,
                                                               d_grad_pts);

@@ -237,6 +237,28 @@ __device__ __forceinline__ ps::DF lookback_segsum_df(TileState* state, ps::DF ti
   return carry;
 }
 
+// The last link l in [0, n - 1] with off[l] <= r (off non-decreasing, off[0] <= r): a
+// warp's 32 probes per round.
+__device__ __forceinline__ int64_t find_link_warp(const int32_t* off, int64_t n, int64_t r,
+                                                  int lane) {
+  int64_t lo = 0, hi = n - 1;  // off[lo] <= r, answer in [lo, hi]
+  while (hi - lo > 31) {
+    int64_t step = (hi - lo + 31) / 32;
+    int64_t cand = lo + lane * step;
+    bool ok = cand <= hi && (int64_t)__ldg(off + cand) <= r;
+    uint32_t b = __ballot_sync(0xffffffffu, ok);
+    int m = __popc(b);  // lanes 0 .. m-1 ok (lane 0 always)
+    int64_t nlo = lo + (int64_t)(m - 1) * step;
+    int64_t nhi = m < 32 ? lo + (int64_t)m * step - 1 : hi;
+    lo = nlo;
+    hi = nhi < hi ? nhi : hi;
+  }
+  int64_t cand = lo + lane;
+  bool ok = cand <= hi && (int64_t)__ldg(off + cand) <= r;
+  uint32_t b = __ballot_sync(0xffffffffu, ok);
+  return lo + __popc(b) - 1;
+}
+
 // ---- host helpers -------------------------------------------------------------
 int ps_ensure_tiles(ps_context* ctx, int64_t n_tile);
 int ps_ensure_recs(ps_context* ctx, int64_t n_link);
@@ -256,8 +278,8 @@ static inline int ps_grid_for(int grid, int64_t n, int64_t per) {
 int ps_run_link_setup(ps_context* ctx, const ps_segments* seg, const ps_paths* paths, float dtheta,
                       int precision, int32_t* d_link_off, int32_t* d_path_off, int64_t* d_n_rib,
                       cudaStream_t st);
-// Segmented (by path) inclusive prefix of per-rib values, in place, with per-path totals.
-int ps_run_segmented_prefix(ps_context* ctx, float* d_vals, const uint32_t* d_tag,
+// Segmented (by path) inclusive prefix of per-rib values, with per-path totals.
+int ps_run_segmented_prefix(ps_context* ctx, const float* d_vals, float* d_prefix, const uint32_t* d_tag,
                             const int64_t* d_n_rib, int64_t capacity, float* d_path_tot,
                             int32_t n_path, cudaStream_t st);
 void ps_prof_mark(ps_context* ctx, int slot, int end, cudaStream_t st);

@@ -1520,28 +1520,6 @@ __device__ __forceinline__ RibEval eval_rib(const LinkRec* __restrict__ L, int j
   else return eval_rib32(L, j);
 }
 
-// The last link l in [0, n - 1] with off[l] <= r (off non-decreasing, off[0] <= r): a
-// warp's 32 probes per round.
-__device__ __forceinline__ int64_t find_link_warp(const int32_t* off, int64_t n, int64_t r,
-                                                  int lane) {
-  int64_t lo = 0, hi = n - 1;  // off[lo] <= r, answer in [lo, hi]
-  while (hi - lo > 31) {
-    int64_t step = (hi - lo + 31) / 32;
-    int64_t cand = lo + lane * step;
-    bool ok = cand <= hi && (int64_t)__ldg(off + cand) <= r;
-    uint32_t b = __ballot_sync(0xffffffffu, ok);
-    int m = __popc(b);  // lanes 0 .. m-1 ok (lane 0 always)
-    int64_t nlo = lo + (int64_t)(m - 1) * step;
-    int64_t nhi = m < 32 ? lo + (int64_t)m * step - 1 : hi;
-    lo = nlo;
-    hi = nhi < hi ? nhi : hi;
-  }
-  int64_t cand = lo + lane;
-  bool ok = cand <= hi && (int64_t)__ldg(off + cand) <= r;
-  uint32_t b = __ballot_sync(0xffffffffu, ok);
-  return lo + __popc(b) - 1;
-}
-
 template <bool MIXED>
 __global__ void __launch_bounds__(EMIT_NT, MIXED ? 2 : 3) k_emit(
     const LinkRec* __restrict__ recs, const int32_t* __restrict__ link_off,
@@ -2212,7 +2190,7 @@ int ps_run_link_setup(ps_context* ctx, const ps_segments* seg, const ps_paths* p
   return ps_cuda_check(cudaGetLastError());
 }
 
-int ps_run_segmented_prefix(ps_context* ctx, float* d_vals, const uint32_t* d_tag,
+int ps_run_segmented_prefix(ps_context* ctx, const float* d_vals, float* d_prefix, const uint32_t* d_tag,
                             const int64_t* d_n_rib, int64_t capacity, float* d_path_tot,
                             int32_t n_path, cudaStream_t st) {
   int64_t scan_tiles = (capacity + SCAN_TILE - 1) / SCAN_TILE;
@@ -2220,7 +2198,7 @@ int ps_run_segmented_prefix(ps_context* ctx, float* d_vals, const uint32_t* d_ta
   if (rc != PS_OK) return rc;
   cudaMemsetAsync(ctx->d_counters, 0, 64 + sizeof(TileState) * (scan_tiles + 1), st);
   if (d_path_tot && n_path > 0) cudaMemsetAsync(d_path_tot, 0, sizeof(float) * n_path, st);
-  launch_arclen_scan(ctx, 0, st, d_vals, d_tag, d_n_rib, capacity, d_vals, d_path_tot,
+  launch_arclen_scan(ctx, 0, st, d_vals, d_tag, d_n_rib, capacity, d_prefix, d_path_tot,
                      ctx->d_tile_state, ctx->d_counters, ctx->d_status);
   return ps_cuda_check(cudaGetLastError());
 }
