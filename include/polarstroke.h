@@ -274,6 +274,33 @@ int ps_count_ribs_sync(ps_context* ctx, const ps_segments* seg, const ps_paths* 
                        float dtheta, int precision, ps_tess_out* out, void* stream,
                        int64_t* h_n_rib);
 
+/* The tessellation in two calls over the links' interval records, for callers
+ * that size their rib buffers exactly, or that differentiate: the links are set up
+ * once, where ps_count_ribs_sync, ps_tessellate_strokes and
+ * ps_tessellate_backward would each set them up again.  d_records is caller-owned
+ * device memory of ps_record_bytes(n_link) bytes, 16-byte aligned, n_link = 2
+ * n_seg + n_path; its layout is private, and it belongs to the inputs, dtheta,
+ * precision and pixel tolerance that it was made with.
+ *   ps_link_records_sync  writes the records, out->d_link_rib_off,
+ *                         out->d_path_rib_off and *out->d_n_rib, and returns R on
+ *                         the host.  SYNCHRONIZES.
+ *   ps_emit_records       ribs, tags, t and arc length (flags as
+ *                         ps_tessellate_strokes, without PS_TESS_COUNT_ONLY) from
+ *                         the records and the offsets of that call.
+ *   ps_backward_records   ps_tessellate_backward from the records.
+ * n_path must be positive; other arguments and errors as in the calls they
+ * stand for. */
+int64_t ps_record_bytes(int64_t n_link);
+int ps_link_records_sync(ps_context* ctx, const ps_segments* seg, const ps_paths* paths,
+                         float dtheta, int precision, ps_tess_out* out, void* d_records,
+                         void* stream, int64_t* h_n_rib);
+int ps_emit_records(ps_context* ctx, const ps_segments* seg, const ps_paths* paths, int precision,
+                    uint32_t flags, ps_tess_out* out, const void* d_records, void* stream);
+int ps_backward_records(ps_context* ctx, const ps_segments* seg, const ps_paths* paths,
+                        int precision, const ps_tess_out* fwd, const void* d_records,
+                        const float* d_grad_rib, const float* d_grad_s, float* d_grad_pts,
+                        float* d_grad_width, void* stream);
+
 /* Cumulative arc length of an existing rib stream (Eq. 18): the centreline
  * point of a segment rib is its midpoint (N + P)/2 (exact when r_N = r_P, as in
  * segment links); joins and caps add 0; s restarts at 0 at every path's first

@@ -28,7 +28,8 @@ EXPORTS = ["ps_create", "ps_destroy", "ps_reserve", "ps_max_ribs", "ps_get_statu
            "ps_uniform_tessellate", "ps_facet_stats", "ps_dash_capped",
            "ps_rasterize_coverage_exact", "ps_set_pixel_tolerance", "ps_get_pixel_tolerance",
            "ps_check_wait_timeout", "ps_tessellate_links", "ps_add_s_carry",
-           "ps_rasterize_coverage_rows", "ps_route_quads"]
+           "ps_rasterize_coverage_rows", "ps_route_quads", "ps_record_bytes",
+           "ps_link_records_sync", "ps_emit_records", "ps_backward_records"]
 PS_PROF_SLOTS = 10
 PS_TUNE_EMIT_SLABS, PS_TUNE_SETUP_LINKS, PS_TUNE_BIN_BLOCKS = 0, 1, 2
 TUNE_CANDIDATES = {PS_TUNE_EMIT_SLABS: (4, 8, 16, 32, 64), PS_TUNE_SETUP_LINKS: (1, 2, 4),
@@ -122,6 +123,15 @@ def lib():
         L.ps_rasterize_coverage_rows.argtypes = [P, P, P, P, I64, I32, ctypes.c_int, ctypes.c_int,
                                                  ctypes.c_int, ctypes.c_int, P, P, ctypes.c_int, P]
         L.ps_route_quads.argtypes = [P, P, P, P, I64, I32, I32, I32, P, P, P, I64, P, P, P]
+        L.ps_record_bytes.argtypes = [I64]
+        L.ps_record_bytes.restype = I64
+        L.ps_link_records_sync.argtypes = [P, ctypes.POINTER(_Segments), ctypes.POINTER(_Paths),
+                                           ctypes.c_float, ctypes.c_int, ctypes.POINTER(_TessOut), P,
+                                           P, ctypes.POINTER(I64)]
+        L.ps_emit_records.argtypes = [P, ctypes.POINTER(_Segments), ctypes.POINTER(_Paths),
+                                      ctypes.c_int, ctypes.c_uint32, ctypes.POINTER(_TessOut), P, P]
+        L.ps_backward_records.argtypes = [P, ctypes.POINTER(_Segments), ctypes.POINTER(_Paths),
+                                          ctypes.c_int, ctypes.POINTER(_TessOut), P, P, P, P, P, P]
         L.ps_tessellate_strokes_noalloc.argtypes = [ctypes.POINTER(_Segments),
                                                     ctypes.POINTER(_Paths), ctypes.c_float,
                                                     ctypes.c_int, ctypes.c_uint32,
@@ -209,20 +219,38 @@ class Context:
 
 
 class DeviceBatch:
-    """A stroke batch's input arrays on the GPU (torch tensors)."""
+    """A stroke batch's input arrays on the GPU (torch tensors).
 
-    def __init__(self, batch, device="cuda"):
+    The arrays go over as one buffer: a copy from pinned memory instead of nine
+    from pageable memory, each waited for.  ``seg_pts`` and ``path_width``, when
+    given, are tensors on the device that stand in for the batch's own.
+    ``wait=False`` leaves the copy to the current stream's order; otherwise it is
+    done when the constructor returns."""
+
+    _ARRAYS = (("seg_pts", np.float32), ("seg_w", np.float32), ("path_seg_off", np.int32),
+               ("path_width", np.float32), ("path_miter", np.float32), ("seg_type", np.uint8),
+               ("path_join", np.uint8), ("path_cap", np.uint8), ("path_closed", np.uint8))
+
+    def __init__(self, batch, device="cuda", seg_pts=None, path_width=None, wait=True):
         import torch
-        t = lambda a, dt: torch.from_numpy(np.array(a, dtype=dt, order="C")).to(device)
-        self.seg_type = t(batch.seg_type, np.uint8)
-        self.seg_pts = t(np.asarray(batch.seg_pts, np.float32).reshape(-1), np.float32)
-        self.seg_w = t(batch.seg_w, np.float32)
-        self.path_seg_off = t(batch.path_seg_off, np.int32)
-        self.path_width = t(batch.path_width, np.float32)
-        self.path_join = t(batch.path_join, np.uint8)
-        self.path_cap = t(batch.path_cap, np.uint8)
-        self.path_miter = t(batch.path_miter, np.float32)
-        self.path_closed = t(batch.path_closed, np.uint8)
+        device = torch.device(device)
+        given = {"seg_pts": seg_pts, "path_width": path_width}
+        parts, size = [], 0
+        for name, dt in self._ARRAYS:
+            if given.get(name) is None:
+                a = np.asarray(getattr(batch, name), dt).reshape(-1)
+                parts.append((name, a, size))
+                size += -(-a.nbytes // 256) * 256
+        stage = torch.empty(size, dtype=torch.uint8, pin_memory=device.type == "cuda")
+        host = stage.numpy()
+        for _, a, at in parts:
+            host[at:at + a.nbytes].view(a.dtype)[:] = a
+        buf = stage.to(device, non_blocking=not wait)
+        for name, a, at in parts:
+            setattr(self, name, buf[at:at + a.nbytes].view(getattr(torch, a.dtype.name)))
+        for name, t in given.items():
+            if t is not None:
+                setattr(self, name, t)
         self.n_seg = int(batch.seg_type.shape[0])
         self.n_path = int(batch.path_width.shape[0])
         self.dtheta = float(np.float32(batch.dtheta))
@@ -245,15 +273,19 @@ class TessOutput:
 
     def __init__(self, n_link, n_path, capacity, arclength=True, want_t=False, device="cuda"):
         import torch
+        self._allocate(capacity, arclength, want_t, device)
+        self.link_rib_off = torch.empty(n_link + 1, dtype=torch.int32, device=device)
+        self.path_rib_off = torch.empty(n_path + 1, dtype=torch.int32, device=device)
+        self.path_len = torch.empty(n_path, dtype=torch.float32, device=device) if arclength else None
+        self.n_rib = torch.zeros(1, dtype=torch.int64, device=device)
+
+    def _allocate(self, capacity, arclength, want_t, device):
+        import torch
         self.capacity = int(capacity)
         self.rib = torch.empty((self.capacity, 4), dtype=torch.float32, device=device)
         self.tag = torch.empty(self.capacity, dtype=torch.int32, device=device)
         self.s = torch.empty(self.capacity, dtype=torch.float32, device=device) if arclength else None
         self.t = torch.empty(self.capacity, dtype=torch.float32, device=device) if want_t else None
-        self.link_rib_off = torch.empty(n_link + 1, dtype=torch.int32, device=device)
-        self.path_rib_off = torch.empty(n_path + 1, dtype=torch.int32, device=device)
-        self.path_len = torch.empty(n_path, dtype=torch.float32, device=device) if arclength else None
-        self.n_rib = torch.zeros(1, dtype=torch.int64, device=device)
 
     def _struct(self):
         p = lambda x: None if x is None else x.data_ptr()
@@ -452,13 +484,47 @@ def ps_route_quads(ctx: Context, rib, tag, n_rib, capacity, width, height, row_b
     _check(rc, "ps_route_quads")
 
 
+def _tessellate_exact(ctx: Context, db: DeviceBatch, precision, arclength=True, want_t=False,
+                      stream=None):
+    """Outputs of exactly the batch's ribs (one host sync for the count), the links'
+    records, and the rib count."""
+    import torch
+    out = TessOutput(db.n_link, db.n_path, 0, arclength=arclength)
+    records = torch.empty(lib().ps_record_bytes(db.n_link), dtype=torch.uint8, device="cuda")
+    if stream is not None:  # freed, or used by the adjoint, after work on that stream
+        records.record_stream(stream)
+    seg, paths = db._structs()
+    o = out._struct()
+    n = ctypes.c_int64(0)
+    _check(lib().ps_link_records_sync(ctx.handle, ctypes.byref(seg), ctypes.byref(paths), db.dtheta,
+                                      int(precision), ctypes.byref(o), _ptr(records),
+                                      _stream(stream), ctypes.byref(n)), "ps_count_ribs_sync")
+    out._allocate(max(n.value, 1), arclength, want_t, "cuda")
+    o = out._struct()
+    _check(lib().ps_emit_records(ctx.handle, ctypes.byref(seg), ctypes.byref(paths), int(precision),
+                                 PS_TESS_ARCLENGTH if arclength else 0, ctypes.byref(o),
+                                 _ptr(records), _stream(stream)), "ps_tessellate_strokes")
+    return out, records, n.value
+
+
+def _backward_records(ctx: Context, db: DeviceBatch, fwd: TessOutput, records, grad_rib, grad_s,
+                      grad_pts, grad_width, precision):
+    """Adjoint of a forward call from its links' records."""
+    seg, paths = db._structs()
+    o = fwd._struct()
+    _check(lib().ps_backward_records(ctx.handle, ctypes.byref(seg), ctypes.byref(paths),
+                                     int(precision), ctypes.byref(o), _ptr(records),
+                                     _ptr(grad_rib), _ptr(grad_s), _ptr(grad_pts),
+                                     _ptr(grad_width), _stream(None)), "ps_tessellate_backward")
+
+
 def tessellate(ctx: Context, db: DeviceBatch, precision=PS_PREC_FP32, arclength=True,
                want_t=False, capacity=None, stream=None) -> TessOutput:
     """Allocate exact-size outputs (one host sync for the count) and tessellate."""
-    if capacity is None:
-        probe = TessOutput(db.n_link, db.n_path, 0, arclength=False)
-        capacity = ps_count_ribs_sync(ctx, db, probe, precision, stream=stream)
-    out = TessOutput(db.n_link, db.n_path, max(int(capacity), 1), arclength=arclength, want_t=want_t)
+    if capacity is None and db.n_path > 0:
+        return _tessellate_exact(ctx, db, precision, arclength, want_t, stream)[0]
+    out = TessOutput(db.n_link, db.n_path, max(int(capacity or 0), 1), arclength=arclength,
+                     want_t=want_t)
     ps_tessellate_strokes(ctx, db, out, precision,
                           PS_TESS_ARCLENGTH if arclength else 0, stream=stream)
     return out

@@ -540,11 +540,11 @@ __global__ void k_adj_finalize(const LinkRec* __restrict__ recs, const int4* __r
 
 }  // namespace
 
-extern "C" int ps_tessellate_backward(ps_context* ctx, const ps_segments* seg,
-                                      const ps_paths* paths, float dtheta, int precision,
-                                      const ps_tess_out* fwd, const float* d_grad_rib,
-                                      const float* d_grad_s, float* d_grad_pts,
-                                      float* d_grad_width, void* stream) {
+// d_records: the forward's records, or NULL to set the links up again.
+static int backward(ps_context* ctx, const ps_segments* seg, const ps_paths* paths, float dtheta,
+                    int precision, const ps_tess_out* fwd, const LinkRec* recs,
+                    const float* d_grad_rib, const float* d_grad_s, float* d_grad_pts,
+                    float* d_grad_width, void* stream) {
   if (!ctx || !seg || !paths || !fwd) return PS_ERR_INVALID;
   // an empty batch has no gradients to write
   if (paths->n_path == 0 && seg->n_seg == 0) return PS_OK;
@@ -582,8 +582,12 @@ extern "C" int ps_tessellate_backward(ps_context* ctx, const ps_segments* seg,
   float* suf = (float*)(w + o_suf);
   float* tot = (float*)(w + o_tot);
   int64_t* nr = (int64_t*)(w + o_nr);
-  int rc = ps_run_link_setup(ctx, seg, paths, dtheta, precision, loff, poff, nr, st);
-  if (rc != PS_OK) return rc;
+  int rc;
+  if (!recs) {
+    if ((rc = ps_run_link_setup(ctx, seg, paths, dtheta, precision, loff, poff, nr, st)) != PS_OK)
+      return rc;
+    recs = ctx->d_recs;
+  }
   k_adj_links<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(seg->d_type, seg->d_pts, seg->d_w,
                                                           paths->d_seg_off, paths->d_closed, P, L,
                                                           src);
@@ -597,11 +601,29 @@ extern "C" int ps_tessellate_backward(ps_context* ctx, const ps_segments* seg,
   cudaMemsetAsync(d_grad_width, 0, sizeof(float) * P, st);
   const int grid =
       ps_grid_for(ps_persistent_grid(ctx, (const void*)k_adj_ribs, 256, 0), cap, 32);
-  k_adj_ribs<<<grid, 256, 0, st>>>(ctx->d_recs, src, fwd->d_link_rib_off, L, fwd->d_n_rib, cap,
+  k_adj_ribs<<<grid, 256, 0, st>>>(recs, src, fwd->d_link_rib_off, L, fwd->d_n_rib, cap,
                                    fwd->d_t, reinterpret_cast<const float4*>(d_grad_rib), d_grad_s,
                                    suf, tot, d_grad_pts, adj, d_grad_width);
-  k_adj_finalize<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(ctx->d_recs, src, L, seg->d_type,
+  k_adj_finalize<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(recs, src, L, seg->d_type,
                                                               seg->d_pts, seg->d_w, adj,
                                                               d_grad_pts);
   return ps_cuda_check(cudaGetLastError());
+}
+
+extern "C" int ps_tessellate_backward(ps_context* ctx, const ps_segments* seg,
+                                      const ps_paths* paths, float dtheta, int precision,
+                                      const ps_tess_out* fwd, const float* d_grad_rib,
+                                      const float* d_grad_s, float* d_grad_pts,
+                                      float* d_grad_width, void* stream) {
+  return backward(ctx, seg, paths, dtheta, precision, fwd, nullptr, d_grad_rib, d_grad_s, d_grad_pts,
+                  d_grad_width, stream);
+}
+
+extern "C" int ps_backward_records(ps_context* ctx, const ps_segments* seg, const ps_paths* paths,
+                                   int precision, const ps_tess_out* fwd, const void* d_records,
+                                   const float* d_grad_rib, const float* d_grad_s,
+                                   float* d_grad_pts, float* d_grad_width, void* stream) {
+  if (!d_records || (reinterpret_cast<uintptr_t>(d_records) & 15u)) return PS_ERR_INVALID;
+  return backward(ctx, seg, paths, 0.f, precision, fwd, static_cast<const LinkRec*>(d_records),
+                  d_grad_rib, d_grad_s, d_grad_pts, d_grad_width, stream);
 }

@@ -1806,9 +1806,13 @@ using namespace ps;
 // host entry points
 // Tessellation of the links [l0, l0 + L) of the batch (all of them when called
 // for the whole batch): offsets and ribs are local to the range.
+// The two phases, link set-up (records, offsets, rib count) and ribs, run together, or
+// apart over records in a caller's buffer.
+enum { PH_SETUP = 1, PH_RIBS = 2 };
 static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_paths* paths,
                              float dtheta, int precision, uint32_t flags, ps_tess_out* out,
-                             cudaStream_t st, int64_t l0, int64_t L) {
+                             cudaStream_t st, int64_t l0, int64_t L, int phases = PH_SETUP | PH_RIBS,
+                             LinkRec* recs = nullptr) {
   int P = paths->n_path;
   if (P <= 0) return PS_ERR_INVALID;
   // links per thread: the tuned value, or the default for the boosted kernel
@@ -1819,9 +1823,13 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
   // the arc-length scan's tiles follow the set-up tiles in the tile states
   if ((rc = ps_ensure_tiles(ctx, n_tiles + (out->capacity + SCAN_TILE - 1) / SCAN_TILE + 2)) != PS_OK)
     return rc;
-  if ((rc = ps_ensure_recs(ctx, L)) != PS_OK) return rc;
   // link path indices live after the records
-  int32_t* link_path = reinterpret_cast<int32_t*>(ctx->d_recs + ctx->rec_cap);
+  int32_t* link_path = reinterpret_cast<int32_t*>(recs + L);
+  if (!recs) {
+    if ((rc = ps_ensure_recs(ctx, L)) != PS_OK) return rc;
+    recs = ctx->d_recs;
+    link_path = reinterpret_cast<int32_t*>(ctx->d_recs + ctx->rec_cap);
+  }
   // counters, set-up tiles and scan tiles
   const int64_t scan_tiles = (out->capacity + SCAN_TILE - 1) / SCAN_TILE;
   const bool arc = !(flags & PS_TESS_COUNT_ONLY) && (flags & PS_TESS_ARCLENGTH) && out->d_s;
@@ -1830,14 +1838,15 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
   // the set-up clears the lengths of the paths that begin in the range: all paths of a whole
   // batch; a range call's others are cleared here
   const bool set_len = arc && out->d_path_len, whole = l0 == 0 && L == 2 * seg->n_seg + P;
-  if (set_len && !whole) cudaMemsetAsync(out->d_path_len, 0, sizeof(float) * P, st);
+  if (set_len && !(whole && (phases & PH_SETUP)))
+    cudaMemsetAsync(out->d_path_len, 0, sizeof(float) * P, st);
   // a count-only call has no rib buffers to overflow
   int64_t count_cap = (flags & PS_TESS_COUNT_ONLY) ? INT64_MAX : out->capacity;
-  {
+  if (phases & PH_SETUP) {
   ProfScope ps_(ctx, PK_LINK_SETUP, st);
 #define PS_SETUP_ARGS                                                                          \
   seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off, paths->d_width, paths->d_join,         \
-      paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, ctx->d_recs, \
+      paths->d_cap, paths->d_miter, paths->d_closed, P, L, dtheta, ctx->pixel_tol, recs,        \
       link_path, set_len ? out->d_path_len : nullptr,                                          \
       out->d_link_rib_off, out->d_path_rib_off, out->d_n_rib, count_cap, ctx->d_tile_state,   \
       ctx->d_counters, ctx->d_status, n_tiles, l0
@@ -1859,14 +1868,14 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
 #undef PS_SETUP_ARGS
   }
   if ((rc = ps_cuda_check(cudaGetLastError())) != PS_OK) return rc;
-  if (flags & PS_TESS_COUNT_ONLY) return PS_OK;
+  if ((flags & PS_TESS_COUNT_ONLY) || !(phases & PH_RIBS)) return PS_OK;
 
   const void* fn = precision == PS_PREC_MIXED ? (const void*)k_emit<true> : (const void*)k_emit<false>;
   const int grid = ps_grid_for(ps_persistent_grid(ctx, fn, EMIT_NT, 0), out->capacity, 31);
   {
   ProfScope ps_(ctx, PK_EMIT, st);
 #define PS_EMIT_ARGS                                                                           \
-  ctx->d_recs, out->d_link_rib_off, link_path, L, out->d_n_rib, out->capacity,                 \
+  recs, out->d_link_rib_off, link_path, L, out->d_n_rib, out->capacity,                        \
       reinterpret_cast<float4*>(out->d_rib), out->d_tag, arc ? out->d_s : nullptr, out->d_t,   \
       ctx->tune[PS_TUNE_EMIT_SLABS]
   if (precision == PS_PREC_MIXED) k_emit<true><<<grid, EMIT_NT, 0, st>>>(PS_EMIT_ARGS);
@@ -1921,6 +1930,54 @@ extern "C" int ps_tessellate_strokes(ps_context* ctx, const ps_segments* seg,
   ctx->last_stream = stream;
   return launch_tessellate(ctx, seg, paths, dtheta, precision, flags, out, st, 0,
                            2 * seg->n_seg + paths->n_path);
+}
+
+extern "C" int64_t ps_record_bytes(int64_t n_link) {
+  return n_link < 0 ? PS_ERR_INVALID : (int64_t)(sizeof(LinkRec) + sizeof(int32_t)) * n_link;
+}
+
+// The arguments of the calls over a caller's records.
+static bool records_ok(const ps_context* ctx, const ps_segments* seg, const ps_paths* paths,
+                       int precision, const ps_tess_out* out, const void* d_records) {
+  return ctx && seg && paths && out && d_records &&
+         (reinterpret_cast<uintptr_t>(d_records) & 15u) == 0 &&
+         (precision == PS_PREC_FP32 || precision == PS_PREC_MIXED) && seg->n_seg >= 0 &&
+         seg->n_seg <= (int64_t)1 << 29 && paths->n_path > 0 && out->d_link_rib_off && out->d_n_rib;
+}
+
+extern "C" int ps_link_records_sync(ps_context* ctx, const ps_segments* seg, const ps_paths* paths,
+                                    float dtheta, int precision, ps_tess_out* out, void* d_records,
+                                    void* stream, int64_t* h_n_rib) {
+  if (!records_ok(ctx, seg, paths, precision, out, d_records) || !out->d_path_rib_off || !h_n_rib ||
+      !(dtheta >= 1e-4f && dtheta <= 3.14159265f))
+    return PS_ERR_INVALID;
+  if (seg->n_seg > 0 && (!seg->d_type || !seg->d_pts)) return PS_ERR_INVALID;
+  if (!paths->d_seg_off || !paths->d_width || !paths->d_join || !paths->d_cap ||
+      !paths->d_miter || !paths->d_closed)
+    return PS_ERR_INVALID;
+  cudaStream_t st = (cudaStream_t)stream;
+  ctx->last_stream = stream;
+  int rc = launch_tessellate(ctx, seg, paths, dtheta, precision, PS_TESS_COUNT_ONLY, out, st, 0,
+                             2 * seg->n_seg + paths->n_path, PH_SETUP,
+                             static_cast<LinkRec*>(d_records));
+  if (rc != PS_OK) return rc;
+  rc = ps_cuda_check(cudaMemcpyAsync(h_n_rib, out->d_n_rib, sizeof(int64_t),
+                                     cudaMemcpyDeviceToHost, st));
+  if (rc != PS_OK) return rc;
+  return ps_cuda_check(cudaStreamSynchronize(st));
+}
+
+extern "C" int ps_emit_records(ps_context* ctx, const ps_segments* seg, const ps_paths* paths,
+                               int precision, uint32_t flags, ps_tess_out* out,
+                               const void* d_records, void* stream) {
+  if (!records_ok(ctx, seg, paths, precision, out, d_records) || !out->d_rib || !out->d_tag ||
+      out->capacity < 0 || (flags & PS_TESS_COUNT_ONLY) ||
+      ((flags & PS_TESS_ARCLENGTH) && !out->d_s))
+    return PS_ERR_INVALID;
+  ctx->last_stream = stream;
+  return launch_tessellate(ctx, seg, paths, 1.f, precision, flags, out, (cudaStream_t)stream, 0,
+                           2 * seg->n_seg + paths->n_path, PH_RIBS,
+                           static_cast<LinkRec*>(const_cast<void*>(d_records)));
 }
 
 extern "C" int ps_count_ribs_sync(ps_context* ctx, const ps_segments* seg, const ps_paths* paths,
