@@ -144,7 +144,7 @@ extern "C" void ps_destroy(ps_context* ctx) {
   if (ctx->prof_on) ps_profile_enable(ctx, 0);
   void* ptrs[] = {ctx->d_status, ctx->d_counters, ctx->d_recs,
                   ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor, ctx->d_bin,
-                  ctx->d_scratch64, ctx->d_mask_scratch, ctx->d_adj, ctx->d_quad_hits,
+                  ctx->d_scratch64, ctx->d_mask_scratch, ctx->d_adj, ctx->d_cap_tasks, ctx->d_quad_hits,
                   ctx->d_tile_list};
   for (void* p : ptrs)
     if (p) cudaFree(p);

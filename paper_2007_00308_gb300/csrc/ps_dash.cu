@@ -68,6 +68,15 @@ __device__ __forceinline__ void emit_cap(const DashCap& c, int J, bool square, i
   }
 }
 
+// A round cap to be written by k_dash_caps.
+struct CapTask {
+  DashCap cap;
+  uint32_t tag;
+  float s;
+  int32_t src, pad;
+  int64_t o;
+};
+
 constexpr int DASH_NT = 256;
 constexpr int DASH_QPT = 4;  // quads per thread
 constexpr int DASH_TILE = DASH_NT * DASH_QPT;
@@ -301,18 +310,24 @@ __global__ void __launch_bounds__(DASH_NT, 5) k_dash_count(
   }
 }
 
-constexpr int EMIT_WQ = 256;  // quads per warp and round of the writing pass
+constexpr int EMIT_WQ = 256;  // quads per ticket of the writing pass
 __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
     const float4* __restrict__ rib, const float* __restrict__ s, const uint32_t* __restrict__ tag,
     const int64_t* __restrict__ n_rib, int64_t capacity, const __grid_constant__ DashPattern P,
     const unsigned long long* __restrict__ word, const __grid_constant__ DashOut D,
-    int32_t* status) {
+    CapTask* __restrict__ tasks, int32_t* counters, int32_t* status) {
   __shared__ uint8_t s_queue[DASH_NT / 32][EMIT_WQ];  // a warp's queued quads
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  const int64_t stride = (int64_t)gridDim.x * (DASH_NT / 32) * EMIT_WQ;
-  for (int64_t t0 = ((int64_t)blockIdx.x * (DASH_NT / 32) + wid) * EMIT_WQ; t0 < R; t0 += stride) {
+  // warps take the next quads by ticket, as their work differs (caps, long lines
+  // with many stretches); a warp's next ticket is drawn while it writes
+  int ticket = 0;
+  if (lane == 0) ticket = atomicAdd(&counters[7], 1);
+  for (;;) {
+    const int64_t t0 = (int64_t)__shfl_sync(0xffffffffu, ticket, 0) * EMIT_WQ;
+    if (t0 >= R) return;
+    if (lane == 0) ticket = atomicAdd(&counters[7], 1);
     int qtot = 0;
 #pragma unroll 4
     for (int q = 0; q < EMIT_WQ / 32; ++q) {
@@ -336,10 +351,12 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
       qtot += __popc(qm);
     }
     __syncwarp();
-    // queued quads: one per lane, each round one piece of each; long caps are
-    // written by the whole warp (a lane alone would write a round cap's 181 ribs
-    // at 1 degree in turn: 2.81 ms -> 1.18 ms for 1,000 paths with capped
-    // dashes, 24.4 M ribs out)
+    // queued quads: one per lane, each round one piece of each.  Round caps are left to
+    // k_dash_caps, or without its list written by the whole warp (a lane alone
+    // would write a cap's 181 ribs at 1 degree in turn: 2.81 ms for 1,000 paths with
+    // capped dashes, 24.4 M ribs out, and 1.18 ms by warps; but a line of 200 px
+    // has 50 caps, all written by one warp while others had none: 530 us for this
+    // kernel, and 290 us and 138 for k_dash_caps with the list)
     for (int i0 = 0; i0 < qtot; i0 += 32) {
       const int lq = i0 + lane < qtot ? s_queue[wid][i0 + lane] : 0;
       bool more = i0 + lane < qtot;
@@ -421,7 +438,17 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
           const bool shared = cap && J > 4;
           if (cap && !shared)
             emit_cap(C, J, square, 0, 1, tq, sv, (int32_t)r, oc, D.rib, D.s, D.tag, D.src);
-          for (unsigned m = __ballot_sync(0xffffffffu, shared); m; m &= m - 1u) {
+          const unsigned sm = __ballot_sync(0xffffffffu, shared);
+          if (tasks) {
+            if (!sm) continue;
+            const int lead = __ffs(sm) - 1;
+            int at = 0;
+            if (lane == lead) at = atomicAdd(&counters[8], __popc(sm));
+            at = __shfl_sync(0xffffffffu, at, lead) + __popc(sm & ((1u << lane) - 1u));
+            if (shared) tasks[at] = CapTask{C, tq, sv, (int32_t)r, 0, oc};
+            continue;
+          }
+          for (unsigned m = sm; m; m &= m - 1u) {
             const int from = __ffs(m) - 1;
             DashCap B;
             B.cx = __shfl_sync(0xffffffffu, C.cx, from);
@@ -437,6 +464,18 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
       }
     }
     __syncwarp();
+  }
+}
+
+// Round caps, a warp to each.
+__global__ void __launch_bounds__(DASH_NT) k_dash_caps(const CapTask* __restrict__ tasks, int J,
+                                                       const __grid_constant__ DashOut D,
+                                                       const int32_t* __restrict__ counters) {
+  const int n = counters[8], lane = threadIdx.x & 31;
+  const int stride = gridDim.x * (DASH_NT / 32);
+  for (int i = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; i < n; i += stride) {
+    const CapTask T = tasks[i];
+    emit_cap(T.cap, J, false, lane, 32, T.tag, T.s, T.src, T.o, D.rib, D.s, D.tag, D.src);
   }
 }
 
@@ -480,12 +519,35 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
       ps_grid_for(ps_persistent_grid(ctx, (const void*)k_dash_count, DASH_NT, 0), capacity, DASH_TILE);
   const int grid1 = ps_grid_for(ps_persistent_grid(ctx, (const void*)k_dash, DASH_NT, 0), capacity,
                                 DASH_NT / 32 * EMIT_WQ);
+  // Room for every round cap (each fills j_round + 1 ribs of the output).  Without it (no
+  // memory, or a capture under way and no room from an earlier call) the writing
+  // pass writes them itself.
+  CapTask* tasks = nullptr;
+  if (P.path_cap && P.j_round > 4) {
+    const size_t need = sizeof(CapTask) * (size_t)(out_capacity / (P.j_round + 1) + 1);
+    if (need > ctx->cap_bytes) {
+      cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+      if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
+        if (ctx->d_cap_tasks) cudaFree(ctx->d_cap_tasks);
+        ctx->d_cap_tasks = nullptr;
+        ctx->cap_bytes = 0;
+        if (cudaMalloc(&ctx->d_cap_tasks, need) == cudaSuccess) ctx->cap_bytes = need;
+        else cudaGetLastError();  // carry on without
+      }
+    }
+    if (need <= ctx->cap_bytes) tasks = static_cast<CapTask*>(ctx->d_cap_tasks);
+  }
+  const int grid2 = ps_grid_for(ps_persistent_grid(ctx, (const void*)k_dash_caps, DASH_NT, 0),
+                                out_capacity / (P.j_round + 1) + 1, 1);
   ProfScope ps_(ctx, PK_DASH, st);
   k_dash_count<<<grid0, DASH_NT, 0, st>>>(d_s, d_tag, d_n_rib, capacity, P, word, d_n_out,
                                                     out_capacity, ctx->d_tile_state, ctx->d_counters,
                                                     ctx->d_status);
   k_dash<<<grid1, DASH_NT, 0, st>>>(reinterpret_cast<const float4*>(d_rib), d_s, d_tag,
-                                              d_n_rib, capacity, P, word, D, ctx->d_status);
+                                              d_n_rib, capacity, P, word, D, tasks, ctx->d_counters,
+                                    ctx->d_status);
+  if (tasks)
+    k_dash_caps<<<grid2, DASH_NT, 0, st>>>(tasks, P.j_round, D, ctx->d_counters);
   return ps_cuda_check(cudaGetLastError());
 }
 

@@ -187,7 +187,9 @@ struct DashWalkDF {
     sa = sa_f;
     sb = sb_f;
     const float u = sa + P.offset_f;
-    k0 = floorf(u / P.period_f) - 1.f;  // one off at most: one period more or less before sa
+    // the period that holds sa, or the one before where FP32 does not tell them apart
+    k0 = floorf(u / P.period_f);
+    if (!(fmaf(-k0, P.period_f, u) > 4e-6f * P.period_f + 4e-7f * fabsf(u))) k0 -= 1.f;
     const float n = (sb - sa) / P.period_f;
     // (false for NaN; a period near FP32's range end has no exact products)
     sure = fabsf(k0) < 4194304.f && n < 1024.f && P.period_f > 1e-20f;

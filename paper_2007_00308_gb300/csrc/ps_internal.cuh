@@ -102,6 +102,8 @@ struct ps_context {
   size_t d_scratch_words;
   void* d_adj;              // adjoint workspace
   size_t adj_bytes;
+  void* d_cap_tasks;        // the dasher's round caps
+  size_t cap_bytes;
   int num_sms;
   int tune[PS_TUNE_COUNT];  // launch parameters (ps_set_tuning)
   float pixel_tol;          // pixel tolerance of the per-link step boost (0: off)
