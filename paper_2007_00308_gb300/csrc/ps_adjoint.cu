@@ -485,6 +485,7 @@ __global__ void k_adj_finalize(const LinkRec* __restrict__ recs, const int4* __r
                                int64_t n_link, const uint8_t* st, const float* sp, const float* sw,
                                const float* __restrict__ adj_psi, float* __restrict__ gpts) {
   int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
+  dep_wait();
   if (l >= n_link) return;
   int4 sc = src[l];
   const LinkRec* L = recs + l;
@@ -604,9 +605,8 @@ static int backward(ps_context* ctx, const ps_segments* seg, const ps_paths* pat
   k_adj_ribs<<<grid, 256, 0, st>>>(recs, src, fwd->d_link_rib_off, L, fwd->d_n_rib, cap,
                                    fwd->d_t, reinterpret_cast<const float4*>(d_grad_rib), d_grad_s,
                                    suf, tot, d_grad_pts, adj, d_grad_width);
-  k_adj_finalize<<<(unsigned)((L + 255) / 256), 256, 0, st>>>(recs, src, L, seg->d_type,
-                                                              seg->d_pts, seg->d_w, adj,
-                                                              d_grad_pts);
+  ps_launch_after(true, &k_adj_finalize, (int)((L + 255) / 256), 256, 0, st, recs, src, L, seg->d_type,
+                  seg->d_pts, seg->d_w, adj, d_grad_pts);
   return ps_cuda_check(cudaGetLastError());
 }
 

@@ -317,6 +317,7 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
     const unsigned long long* __restrict__ word, const __grid_constant__ DashOut D,
     CapTask* __restrict__ tasks, int32_t* counters, int32_t* status) {
   __shared__ uint8_t s_queue[DASH_NT / 32][EMIT_WQ];  // a warp's queued quads
+  dep_wait();
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -471,6 +472,7 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
 __global__ void __launch_bounds__(DASH_NT) k_dash_caps(const CapTask* __restrict__ tasks, int J,
                                                        const __grid_constant__ DashOut D,
                                                        const int32_t* __restrict__ counters) {
+  dep_wait();
   const int n = counters[8], lane = threadIdx.x & 31;
   const int stride = gridDim.x * (DASH_NT / 32);
   for (int i = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; i < n; i += stride) {
@@ -543,11 +545,11 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
   k_dash_count<<<grid0, DASH_NT, 0, st>>>(d_s, d_tag, d_n_rib, capacity, P, word, d_n_out,
                                                     out_capacity, ctx->d_tile_state, ctx->d_counters,
                                                     ctx->d_status);
-  k_dash<<<grid1, DASH_NT, 0, st>>>(reinterpret_cast<const float4*>(d_rib), d_s, d_tag,
-                                              d_n_rib, capacity, P, word, D, tasks, ctx->d_counters,
-                                    ctx->d_status);
+  // (one profile slot for all three: no event records in between)
+  ps_launch_after(true, &k_dash, grid1, DASH_NT, 0, st, reinterpret_cast<const float4*>(d_rib), d_s,
+                  d_tag, d_n_rib, capacity, P, word, D, tasks, ctx->d_counters, ctx->d_status);
   if (tasks)
-    k_dash_caps<<<grid2, DASH_NT, 0, st>>>(tasks, P.j_round, D, ctx->d_counters);
+    ps_launch_after(true, &k_dash_caps, grid2, DASH_NT, 0, st, tasks, P.j_round, D, ctx->d_counters);
   return ps_cuda_check(cudaGetLastError());
 }
 

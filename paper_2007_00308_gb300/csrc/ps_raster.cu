@@ -222,6 +222,7 @@ __global__ void __launch_bounds__(BIN_NT) k_bin(const float4* __restrict__ rib,
                                                 RasterClear clear, int32_t* status) {
   __shared__ BinQuad s_q[BIN_NT];
   __shared__ int s_pre[BIN_NT / 32][33];
+  if (PASS == 1) dep_wait();
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -436,6 +437,7 @@ __global__ void __launch_bounds__(TS_NT) k_tile_scan(const int32_t* __restrict__
   __shared__ long long s_pre;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long i0 = (long long)blockIdx.x * TS_TILE + (long long)threadIdx.x * TS_IPT;
+  dep_wait();
   int c[TS_IPT];
   if (i0 + TS_IPT <= n_tile) {
     const int4* cp = reinterpret_cast<const int4*>(count + i0);
@@ -1314,6 +1316,7 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
   __shared__ __align__(16) float4 s_pre_rib[CV_WARPS][2][32];
   __shared__ uint32_t s_pre_tag[CV_WARPS][32];
 
+  dep_wait();
   const int n_list = tile_list[n_tile];  // tiles with entries (the canvas is cleared)
   if ((int)blockIdx.x >= n_list) return;  // the others' tickets reach every tile
   for (int i = threadIdx.x; i < SLOTS * MASK_WORDS; i += CV_NT) s_mask[i] = 0u;
@@ -1700,24 +1703,22 @@ static int rasterize(ps_context* ctx, const float* d_rib, const uint32_t* d_tag,
                                       ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,
                                       ctx->d_bin, ctx->pair_cap, reinterpret_cast<uint2*>(ctx->d_quad_hits), ctx->d_tile_cursor + n_tile + 1,
                                       clear, ctx->d_status); }
+  const bool overlap = !ctx->prof_on;
   { ProfScope ps_(ctx, PK_TILE_SCAN, st);
-  k_tile_scan<<<ts_grid, TS_NT, 0, st>>>(ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,
-                                         ctx->d_tile_list, (int)n_tile, ctx->pair_cap,
-                                         ctx->d_tile_state, ctx->d_status); }
+  ps_launch_after(overlap, &k_tile_scan, ts_grid, TS_NT, 0, st, ctx->d_tile_count, ctx->d_tile_off,
+                  ctx->d_tile_cursor, ctx->d_tile_list, (int)n_tile, ctx->pair_cap,
+                  ctx->d_tile_state, ctx->d_status); }
   { ProfScope ps_(ctx, PK_BIN_SCATTER, st);
-  k_bin<1><<<grid_bin1, BIN_NT, 0, st>>>(rib, d_tag, d_n_rib, capacity, width, height, y0, tiles_x,
-                                      ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,
-                                      ctx->d_bin, ctx->pair_cap, reinterpret_cast<uint2*>(ctx->d_quad_hits), ctx->d_tile_cursor + n_tile + 1,
-                                      clear, ctx->d_status); }
+  ps_launch_after(overlap, &k_bin<1>, grid_bin1, BIN_NT, 0, st, rib, d_tag, d_n_rib, capacity, width,
+                  height, y0, tiles_x, ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,
+                  ctx->d_bin, ctx->pair_cap, reinterpret_cast<uint2*>(ctx->d_quad_hits),
+                  ctx->d_tile_cursor + n_tile + 1, clear, ctx->d_status); }
   { ProfScope ps_(ctx, PK_COVERAGE, st);
-#define PS_COV_ARGS                                                                              \
-  rib, d_tag, ctx->d_tile_off, ctx->d_bin, ctx->pair_cap, width, height, y0, tiles_x, (int)n_tile, \
-      ctx->d_tile_list, d_canvas, reinterpret_cast<unsigned long long*>(d_covered), n_path, ctx->d_counters,      \
-      ctx->d_status, reinterpret_cast<unsigned long long*>(ctx->d_scratch64)
-  if (exact) k_coverage<true><<<grid_cov, CV_NT, cov_smem, st>>>(PS_COV_ARGS);
-  else k_coverage<false><<<grid_cov, CV_NT, cov_smem, st>>>(PS_COV_ARGS);
-#undef PS_COV_ARGS
-  }
+  ps_launch_after(overlap, exact ? &k_coverage<true> : &k_coverage<false>, grid_cov, CV_NT, cov_smem, st,
+                  rib, d_tag, ctx->d_tile_off, ctx->d_bin, ctx->pair_cap, width, height, y0, tiles_x,
+                  (int)n_tile, ctx->d_tile_list, d_canvas,
+                  reinterpret_cast<unsigned long long*>(d_covered), n_path, ctx->d_counters,
+                  ctx->d_status, reinterpret_cast<unsigned long long*>(ctx->d_scratch64)); }
   return ps_cuda_check(cudaGetLastError());
 }
 

@@ -1526,6 +1526,7 @@ __global__ void __launch_bounds__(EMIT_NT, MIXED ? 2 : 3) k_emit(
     const int32_t* __restrict__ link_path, int64_t n_link, const int64_t* __restrict__ n_rib,
     int64_t capacity, float4* __restrict__ rib, uint32_t* __restrict__ tag,
     float* __restrict__ chord, float* __restrict__ tout, int most_slabs) {
+  dep_wait();
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31;
@@ -1633,6 +1634,7 @@ __global__ void __launch_bounds__(SCAN_NT) k_arclen_scan(
   __shared__ float s_carry[2];
   __shared__ int64_t s_tile;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
+  dep_wait();
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int64_t n_tiles = (R + SCAN_TILE - 1) / SCAN_TILE;
@@ -1762,7 +1764,7 @@ __global__ void __launch_bounds__(SCAN_NT) k_arclen_scan(
 }
 
 // Launch of k_arclen_scan with the vector form when every array allows it.
-static void launch_arclen_scan(ps_context* ctx, int grid_override, cudaStream_t st,
+static void launch_arclen_scan(ps_context* ctx, int grid_override, bool overlap, cudaStream_t st,
                                const float* chord, const uint32_t* tag, const int64_t* n_rib,
                                int64_t capacity, float* s_out, float* path_len,
                                TileState* state, int32_t* counters, int32_t* status) {
@@ -1771,12 +1773,8 @@ static void launch_arclen_scan(ps_context* ctx, int grid_override, cudaStream_t 
   const void* fn = vec ? (const void*)k_arclen_scan<true> : (const void*)k_arclen_scan<false>;
   const int g = ps_grid_for(
       grid_override > 0 ? grid_override : ps_persistent_grid(ctx, fn, SCAN_NT, 0), capacity, SCAN_TILE);
-  if (vec)
-    k_arclen_scan<true><<<g, SCAN_NT, 0, st>>>(chord, tag, n_rib, capacity, s_out, path_len,
-                                               state, counters, status);
-  else
-    k_arclen_scan<false><<<g, SCAN_NT, 0, st>>>(chord, tag, n_rib, capacity, s_out, path_len,
-                                                state, counters, status);
+  ps_launch_after(overlap, vec ? &k_arclen_scan<true> : &k_arclen_scan<false>, g, SCAN_NT, 0, st, chord,
+                  tag, n_rib, capacity, s_out, path_len, state, counters, status);
 }
 
 // Chords from rib midpoints (standalone arc length of any rib stream).
@@ -1874,20 +1872,18 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
   const int grid = ps_grid_for(ps_persistent_grid(ctx, fn, EMIT_NT, 0), out->capacity, 31);
   {
   ProfScope ps_(ctx, PK_EMIT, st);
-#define PS_EMIT_ARGS                                                                           \
-  recs, out->d_link_rib_off, link_path, L, out->d_n_rib, out->capacity,                        \
-      reinterpret_cast<float4*>(out->d_rib), out->d_tag, arc ? out->d_s : nullptr, out->d_t,   \
-      ctx->tune[PS_TUNE_EMIT_SLABS]
-  if (precision == PS_PREC_MIXED) k_emit<true><<<grid, EMIT_NT, 0, st>>>(PS_EMIT_ARGS);
-  else k_emit<false><<<grid, EMIT_NT, 0, st>>>(PS_EMIT_ARGS);
-#undef PS_EMIT_ARGS
+  ps_launch_after(!ctx->prof_on && (phases & PH_SETUP),
+                  precision == PS_PREC_MIXED ? &k_emit<true> : &k_emit<false>, grid, EMIT_NT, 0, st,
+                  recs, out->d_link_rib_off, link_path, L, out->d_n_rib, out->capacity,
+                  reinterpret_cast<float4*>(out->d_rib), out->d_tag, arc ? out->d_s : nullptr,
+                  out->d_t, ctx->tune[PS_TUNE_EMIT_SLABS]);
   }
   if ((rc = ps_cuda_check(cudaGetLastError())) != PS_OK) return rc;
   if (arc) {
     // the emitter wrote each rib's chord into s; the segmented scan turns them
     // into cumulative arc length in place
     ProfScope ps_(ctx, PK_ARCLEN, st);
-    launch_arclen_scan(ctx, 0, st, out->d_s, out->d_tag, out->d_n_rib, out->capacity, out->d_s,
+    launch_arclen_scan(ctx, 0, !ctx->prof_on, st, out->d_s, out->d_tag, out->d_n_rib, out->capacity, out->d_s,
                        out->d_path_len, ctx->d_tile_state + n_tiles + 1, ctx->d_counters,
                        ctx->d_status);
     if ((rc = ps_cuda_check(cudaGetLastError())) != PS_OK) return rc;
@@ -2073,7 +2069,7 @@ extern "C" int ps_arclength_scan(ps_context* ctx, const float* d_rib, const uint
   k_midpoint_chords<<<g, 256, 0, st>>>(reinterpret_cast<const float4*>(d_rib), d_tag, d_n_rib,
                                        capacity, d_s); }
   ProfScope ps_(ctx, PK_ARCLEN, st);
-  launch_arclen_scan(ctx, 0, st, d_s, d_tag, d_n_rib, capacity, d_s, d_path_len, ctx->d_tile_state,
+  launch_arclen_scan(ctx, 0, false, st, d_s, d_tag, d_n_rib, capacity, d_s, d_path_len, ctx->d_tile_state,
                      ctx->d_counters, ctx->d_status);
   return ps_cuda_check(cudaGetLastError());
 }
@@ -2184,14 +2180,10 @@ extern "C" int ps_tessellate_strokes_noalloc(const ps_segments* seg, const ps_pa
       &per_sm, precision == PS_PREC_MIXED ? (const void*)k_emit<true> : (const void*)k_emit<false>,
       EMIT_NT, 0);
   int grid = g_noalloc_sms[dev] * (per_sm > 0 ? per_sm : 1);
-  if (precision == PS_PREC_MIXED)
-    k_emit<true><<<grid, EMIT_NT, 0, st>>>(recs, out->d_link_rib_off, link_path, L, out->d_n_rib,
-                                           out->capacity, reinterpret_cast<float4*>(out->d_rib),
-                                           out->d_tag, arc ? out->d_s : nullptr, out->d_t, EMIT_K);
-  else
-    k_emit<false><<<grid, EMIT_NT, 0, st>>>(recs, out->d_link_rib_off, link_path, L, out->d_n_rib,
-                                            out->capacity, reinterpret_cast<float4*>(out->d_rib),
-                                            out->d_tag, arc ? out->d_s : nullptr, out->d_t, EMIT_K);
+  ps_launch_after(true, precision == PS_PREC_MIXED ? &k_emit<true> : &k_emit<false>, grid, EMIT_NT, 0, st,
+                  recs, out->d_link_rib_off, link_path, L, out->d_n_rib, out->capacity,
+                  reinterpret_cast<float4*>(out->d_rib), out->d_tag, arc ? out->d_s : nullptr,
+                  out->d_t, EMIT_K);
   if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   if (arc) {
     int per_sm2 = 1;
@@ -2199,7 +2191,7 @@ extern "C" int ps_tessellate_strokes_noalloc(const ps_segments* seg, const ps_pa
                                                   SCAN_NT, 0);
     int g2 = g_noalloc_sms[dev] * (per_sm2 > 0 ? per_sm2 : 1);
     int64_t o = NOALLOC_SETUP_TILES + 1;
-    launch_arclen_scan(nullptr, g2, st, out->d_s, out->d_tag, out->d_n_rib, out->capacity,
+    launch_arclen_scan(nullptr, g2, true, st, out->d_s, out->d_tag, out->d_n_rib, out->capacity,
                        out->d_s, out->d_path_len, state + o, counters, d_status);
     if (cudaGetLastError() != cudaSuccess) return PS_ERR_CUDA;
   }
@@ -2255,7 +2247,7 @@ int ps_run_segmented_prefix(ps_context* ctx, const float* d_vals, float* d_prefi
   if (rc != PS_OK) return rc;
   cudaMemsetAsync(ctx->d_counters, 0, 64 + sizeof(TileState) * (scan_tiles + 1), st);
   if (d_path_tot && n_path > 0) cudaMemsetAsync(d_path_tot, 0, sizeof(float) * n_path, st);
-  launch_arclen_scan(ctx, 0, st, d_vals, d_tag, d_n_rib, capacity, d_prefix, d_path_tot,
+  launch_arclen_scan(ctx, 0, false, st, d_vals, d_tag, d_n_rib, capacity, d_prefix, d_path_tot,
                      ctx->d_tile_state, ctx->d_counters, ctx->d_status);
   return ps_cuda_check(cudaGetLastError());
 }
