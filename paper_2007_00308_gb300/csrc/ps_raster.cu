@@ -15,9 +15,10 @@ constexpr int TILE_PX = 16;                 // tile edge in pixels
 constexpr int TILE_UNITS = TILE_PX * 256;   // in 1/256 px
 constexpr int COORD_LIMIT = 1 << 29;        // |v * 256| < 2^29, i.e. |v| < 2^21 px
 
-// floor(a / 256) and ceil(a / 256) (arithmetic shifts round toward -inf)
-__device__ __forceinline__ int64_t floor256(int64_t a) { return a >> 8; }
-__device__ __forceinline__ int64_t ceil256(int64_t a) { return -((-a) >> 8); }
+// floor(a / 256) and ceil(a / 256) (arithmetic shifts round toward -inf); coordinates are
+// below 2^30 in magnitude here, so int32 holds every step
+__device__ __forceinline__ int floor256(int a) { return a >> 8; }
+__device__ __forceinline__ int ceil256(int a) { return -((-a) >> 8); }
 
 struct QuadFix {
   int x[4], y[4];  // N0 P0 N1 P1 in 1/256 px
@@ -41,11 +42,8 @@ __device__ __forceinline__ bool snap_quad(const float4 a, const float4 b, QuadFi
 
 // Pixel range whose sample window [256p + 8, 256p + 248] meets [lo, hi].
 __device__ __forceinline__ void pix_range(int lo, int hi, int n, int& p0, int& p1) {
-  int64_t a = ceil256((int64_t)lo - 248), b = floor256((int64_t)hi - 8);
-  if (a < 0) a = 0;
-  if (b > n - 1) b = n - 1;
-  p0 = (int)a;
-  p1 = (int)b;
+  p0 = max(ceil256(lo - 248), 0);
+  p1 = min(floor256(hi - 8), n - 1);
 }
 
 // Can triangle (x0,y0)-(x1,y1)-(x2,y2) cover a sample of the tile whose samples
@@ -208,8 +206,12 @@ __device__ __forceinline__ void raster_clear(const RasterClear& C) {
   if (i0 < 7) C.stats[i0] = 0ull;
 }
 
+// Five and six CTAs per SM (48 and 40 registers): the passes wait for memory and atomics as much
+// as they issue (count 1,028 -> 909 us, scatter 815 -> 782 us on 43 M ribs, of which 60 us of the
+// count by int32 pixel ranges and by staging only the quads of three tiles and more; six and
+// eight CTAs spill: 963 and 813 us).
 template <int PASS>
-__global__ void __launch_bounds__(BIN_NT) k_bin(const float4* __restrict__ rib,
+__global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 6) k_bin(const float4* __restrict__ rib,
                                                 const uint32_t* __restrict__ tag,
                                                 const int64_t* __restrict__ n_rib, int64_t capacity,
                                                 int W, int H, int y0, int tiles_x,
@@ -260,10 +262,11 @@ __global__ void __launch_bounds__(BIN_NT) k_bin(const float4* __restrict__ rib,
         pix_range(mny, mxy, H, py0, py1);
         if (px0 <= px1 && py0 <= py1) {
           int tx0 = px0 / TILE_PX, tx1 = px1 / TILE_PX, ty0 = py0 / TILE_PX, ty1 = py1 / TILE_PX;
-          for (int v = 0; v < 4; ++v) {
-            Q.x[v] = q.x[v];
-            Q.y[v] = q.y[v];
-          }
+          if ((tx1 - tx0 + 1) * (ty1 - ty0 + 1) > 2)
+            for (int v = 0; v < 4; ++v) {
+              Q.x[v] = q.x[v];
+              Q.y[v] = q.y[v];
+            }
           Q.tx0 = tx0;
           Q.ty0 = ty0;
           Q.tbase = ty0 * tiles_x + tx0;
@@ -346,17 +349,20 @@ __global__ void __launch_bounds__(BIN_NT) k_bin(const float4* __restrict__ rib,
       direct(tdir);
       if (__any_sync(0xffffffffu, tdir2 >= 0)) direct(tdir2);
     }
-    // warp scan of the pair counts
-    int x = cnt;
+    // warp scan of the pair counts, where some quad has more than two tiles
+    int total = 0;
+    if (__any_sync(0xffffffffu, cnt > 0)) {
+      int x = cnt;
 #pragma unroll
-    for (int o = 1; o < 32; o <<= 1) {
-      int y = __shfl_up_sync(0xffffffffu, x, o);
-      if (lane >= o) x += y;
+      for (int o = 1; o < 32; o <<= 1) {
+        int y = __shfl_up_sync(0xffffffffu, x, o);
+        if (lane >= o) x += y;
+      }
+      s_pre[wid][lane + 1] = x;
+      if (lane == 0) s_pre[wid][0] = 0;
+      total = __shfl_sync(0xffffffffu, x, 31);
+      __syncwarp();
     }
-    s_pre[wid][lane + 1] = x;
-    if (lane == 0) s_pre[wid][0] = 0;
-    const int total = __shfl_sync(0xffffffffu, x, 31);
-    __syncwarp();
     for (int it0 = 0; it0 < total; it0 += 32) {
       const int it = it0 + lane;
       int t = -1, e = 0, i = 0, tl = 0;
@@ -1305,7 +1311,7 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
   uint32_t* s_keys = reinterpret_cast<uint32_t*>(s_ent + CV_NT);                 // HKEYS
   uint16_t* s_slot_of = reinterpret_cast<uint16_t*>(s_keys + HKEYS);             // HKEYS
   uint32_t* s_slot_path = reinterpret_cast<uint32_t*>(s_slot_of + HKEYS);        // HKEYS
-  __shared__ int s_tile, s_nslot, s_next;
+  __shared__ int s_tile, s_b0, s_b1, s_nslot, s_next;  // the tile (-1: none left), its bin entries
   __shared__ uint8_t s_own[CV_WARPS][32];
   __shared__ uint8_t s_own2[CV_WARPS][32];
   __shared__ uint32_t s_canvas[MASK_WORDS];
@@ -1327,8 +1333,11 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
   int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   EntrySetup* my = s_ent + wid * 32;
   // work counters (items: per warp, the same in every lane; rows: per lane),
-  // added to the global ones at tile ends: one atomic per warp and tile
+  // added to the global ones at the kernel's end or every 200 batches, before a
+  // field fills (at every tile's end the 42 atomics on one line cost a scene of 11,174 tiles
+  // with 145 entries each 4 us of 293)
   unsigned long long st_items = 0, st_rows = 0;
+  unsigned st_passes = 0, st_paths = 0;  // thread 0: passes over tiles, distinct paths
   int st_batches = 0;
   auto flush_stats = [&]() {
     for (int o = 16; o > 0; o >>= 1) st_rows += __shfl_xor_sync(0xffffffffu, st_rows, o);
@@ -1341,15 +1350,32 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
       atomicAdd(stats + 3, f2);
       atomicAdd(stats + 6, st_rows);
     }
+    if (threadIdx.x == 0 && stats && st_passes) {
+      atomicAdd(stats + 4, (unsigned long long)st_paths);
+      atomicAdd(stats + 5, (unsigned long long)st_passes);
+    }
     st_items = 0;
     st_rows = 0;
     st_batches = 0;
+    st_passes = 0;
+    st_paths = 0;
   };
-  // tiles are claimed by ticket; the next ticket's atomic is issued when a
-  // tile's last pass reaches its flush, and read when the tile ends, so its
-  // latency hides behind the flush (claiming earlier would hold a tile back
-  // from an idle CTA)
-  if (threadIdx.x == 0) s_tile = atomicAdd(&counters[2], 1);
+  // Tiles are claimed by ticket.  The next tile is claimed, and its place in the list and
+  // its entries' range are read, by one thread of the last warp while the current tile's
+  // last pass is flushed: three dependent accesses that the next tile would
+  // otherwise begin with (claiming earlier would hold a tile back from an idle
+  // CTA).
+  auto claim = [&]() {
+    const int k = atomicAdd(&counters[2], 1);
+    int t = -1;
+    if (k < n_list) {
+      t = tile_list[k];
+      s_b0 = off[t];
+      s_b1 = off[t + 1];
+    }
+    s_tile = t;
+  };
+  if (threadIdx.x == CV_NT - 1) claim();
   bool dirty = true;  // the path hash holds the previous tile's keys
   for (;;) {
     if (dirty)
@@ -1359,21 +1385,21 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
       }
     if (threadIdx.x == 0) s_nslot = 0;
     __syncthreads();
-    const int ticket = s_tile;
-    int t_next = 0;
-    flush_stats();
-    if (ticket >= n_list) return;
-    const int t = tile_list[ticket];
+    const int t = s_tile;
+    if (t < 0) {
+      flush_stats();
+      return;
+    }
     int tx = t % tiles_x, ty = t / tiles_x;
     int ox = tx * TILE_UNITS, oy = ty * TILE_UNITS;
-    int64_t b0 = off[t], b1 = off[t + 1];
+    int64_t b0 = s_b0, b1 = s_b1;
     if (b1 > pair_cap) b1 = pair_cap;
     int n = (int)(b1 > b0 ? b1 - b0 : 0);
     int tw = min(TILE_PX, W - tx * TILE_PX), th = min(TILE_PX, H - ty * TILE_PX);
     dirty = n > 0;
     if (n == 0) {  // listed but its entries are beyond the bin capacity
-      if (threadIdx.x == 0) t_next = atomicAdd(&counters[2], 1);
       __syncthreads();  // every thread has read s_tile before it is rewritten
+      if (threadIdx.x == CV_NT - 1) claim();
     }
     for (int pass = 0; n > 0; ++pass) {
       int slot_lo = pass * SLOTS;
@@ -1589,29 +1615,31 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
       // warp per slot
       int nslot = min(s_nslot, HKEYS);
       int nhere = min(SLOTS, nslot - slot_lo);
-      if (threadIdx.x == 0 && slot_lo + SLOTS >= nslot) t_next = atomicAdd(&counters[2], 1);
+      if (threadIdx.x == CV_NT - 1 && slot_lo + SLOTS >= nslot) claim();
+      uint4 cw = make_uint4(0u, 0u, 0u, 0u);  // this lane's four canvas words over the warp's slots
       for (int s2 = wid; s2 < nhere; s2 += CV_WARPS) {
-        uint32_t* ms = s_mask + s2 * MASK_WORDS;
-        unsigned c = 0;
-#pragma unroll
-        for (int w = lane; w < MASK_WORDS; w += 32) {
-          const uint32_t v = ms[w];
-          ms[w] = 0u;
-          c += __popc(v);
-          if (v) atomicOr(&s_canvas[w], v);
-        }
-        for (int o = 16; o > 0; o >>= 1) c += __shfl_xor_sync(0xffffffffu, c, o);
+        uint4* ms = reinterpret_cast<uint4*>(s_mask + s2 * MASK_WORDS) + lane;
+        const uint4 v = *ms;
+        *ms = make_uint4(0u, 0u, 0u, 0u);
+        cw.x |= v.x;
+        cw.y |= v.y;
+        cw.z |= v.z;
+        cw.w |= v.w;
+        const unsigned c = __reduce_add_sync(
+            0xffffffffu, __popc(v.x) + __popc(v.y) + __popc(v.z) + __popc(v.w));
         if (lane == 0 && c) {
           uint32_t p = s_slot_path[slot_lo + s2];
           if ((int)p < n_path) atomicAdd(covered + p, (unsigned long long)c);
         }
       }
+      if (cw.x) atomicOr(&s_canvas[4 * lane], cw.x);
+      if (cw.y) atomicOr(&s_canvas[4 * lane + 1], cw.y);
+      if (cw.z) atomicOr(&s_canvas[4 * lane + 2], cw.z);
+      if (cw.w) atomicOr(&s_canvas[4 * lane + 3], cw.w);
       if (threadIdx.x == 0) {
         if (s_nslot > HKEYS) ps_record_error(status, PS_ERR_CAPACITY);
-        if (stats) {
-          atomicAdd(stats + 5, 1ull);
-          if (pass == 0) atomicAdd(stats + 4, (unsigned long long)nslot);
-        }
+        ++st_passes;
+        if (pass == 0) st_paths += nslot;
       }
       __syncthreads();
       for (int w = threadIdx.x; w < MASK_WORDS; w += CV_NT) {
@@ -1630,9 +1658,6 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
       }
       if (slot_lo + SLOTS >= nslot) break;
     }
-    // a non-empty tile's barriers already follow every read of s_tile and
-    // s_nslot
-    if (threadIdx.x == 0) s_tile = t_next;
   }
 }
 
