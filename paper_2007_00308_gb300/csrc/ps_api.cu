@@ -156,7 +156,7 @@ extern "C" int ps_reserve(ps_context* ctx, int64_t n_link, int64_t n_rib, int64_
   if (!ctx || n_link < 0 || n_rib < 0 || n_tile < 0 || n_pair < 0) return PS_ERR_INVALID;
   int rc;
   if (n_link && (rc = ps_ensure_recs(ctx, n_link)) != PS_OK) return rc;
-  int64_t tiles = (n_link + 511) / 512 + (n_rib + 2047) / 2048 + 4 + n_rib / 512;
+  int64_t tiles = (n_link + 255) / 256 + (n_rib + 2047) / 2048 + 4 + n_rib / 512;
   if ((rc = ps_ensure_tiles(ctx, tiles)) != PS_OK) return rc;
   // the dash's and the binning's words per rib
   if (n_rib && (rc = ps_ensure_quad_hits(ctx, n_rib)) != PS_OK) return rc;

@@ -1813,9 +1813,14 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
                              LinkRec* recs = nullptr) {
   int P = paths->n_path;
   if (P <= 0) return PS_ERR_INVALID;
-  // links per thread: the tuned value, or the default for the boosted kernel
+  // links per thread: at most the tuned value, or the default for the boosted kernel
   // (one instantiation only)
-  const int ipt = ctx->pixel_tol > 0.f ? SETUP_IPT : ctx->tune[PS_TUNE_SETUP_LINKS];
+  int ipt = ctx->pixel_tol > 0.f ? SETUP_IPT : ctx->tune[PS_TUNE_SETUP_LINKS];
+  // fewer where all CTAs still run at once (two per SM): a thread's links follow one
+  // another, and nothing is gained but latency (18,278 links: 44 us at two per thread, 33 at
+  // one; 60,922: 49 and 44; 133,120, more than one wave: 36 and 49)
+  if (ctx->pixel_tol == 0.f)
+    while (ipt > 1 && L <= (int64_t)SETUP_NT * (ipt / 2) * 2 * ctx->num_sms) ipt /= 2;
   int64_t n_tiles = (L + SETUP_NT * ipt - 1) / (SETUP_NT * ipt);
   int rc;
   // the arc-length scan's tiles follow the set-up tiles in the tile states
