@@ -157,34 +157,36 @@ __device__ __forceinline__ float2 g_rel(const Seg& g, float t) {
 // float t in double-float arithmetic (ps_df.cuh) -- the differences exact as
 // pairs, the weights as pairs, the products exact in their high parts and the
 // rounding errors gathered lazily; the conic's quotient by one residual step.
+__device__ __forceinline__ F2 f2_pt(float2 p) { return F2{p.x, p.y}; }
+__device__ __forceinline__ DF2 df2_of(F2 hi, F2 lo) { return DF2{DF{hi.x, lo.x}, DF{hi.y, lo.y}}; }
 __device__ __forceinline__ DF2 g_rel_comp_df(const Seg& g, float t) {
   const DF U = two_sum(1.f, -t);
-  const DF bx = two_sum(g.B.x, -g.A.x), by = two_sum(g.B.y, -g.A.y);
-  const DF dx = two_sum(g.D.x, -g.A.x), dy = two_sum(g.D.y, -g.A.y);
+  const F2 A = f2_pt(g.A);
+  const DFP b = two_diff2(f2_pt(g.B), A), d = two_diff2(f2_pt(g.D), A);
   switch (g.type) {
     case PS_CUBIC: {
-      const DF cx = two_sum(g.C.x, -g.A.x), cy = two_sum(g.C.y, -g.A.y);
+      const DFP c = two_diff2(f2_pt(g.C), A);
       const DF ut3 = df_mul_f(df_mul_f(U, t), 3.f);
       const DF wb = df_mul(ut3, U), wc = df_mul_f(ut3, t), wd = df_mul_f(two_prod(t, t), t);
-      Acc x = acc_first(bx, wb), y = acc_first(by, wb);
-      acc_prod(x, cx, wc); acc_prod(y, cy, wc);
-      acc_prod(x, dx, wd); acc_prod(y, dy, wd);
-      return DF2{acc_df(x), acc_df(y)};
+      Acc2 v = acc_first2(b, wb);
+      acc_prod2(v, c, wc);
+      acc_prod2(v, d, wd);
+      return df2_of(v.s, v.e);
     }
     case PS_QUAD: {
       const DF wb = df_mul_f(df_mul_f(U, t), 2.f), wd = two_prod(t, t);
-      Acc x = acc_first(bx, wb), y = acc_first(by, wb);
-      acc_prod(x, dx, wd); acc_prod(y, dy, wd);
-      return DF2{acc_df(x), acc_df(y)};
+      Acc2 v = acc_first2(b, wb);
+      acc_prod2(v, d, wd);
+      return df2_of(v.s, v.e);
     }
     case PS_CONIC: {
       const DF ut = df_mul_f(U, t);
       const DF wb = df_mul_f(ut, 2.f * g.w);  // 2w exact
       const DF wd = two_prod(t, t);
       const DF den = df_add(df_add(df_mul(U, U), wb), wd);
-      Acc ax = acc_first(bx, wb), ay = acc_first(by, wb);
-      acc_prod(ax, dx, wd); acc_prod(ay, dy, wd);
-      const DF x = fast_two_sum(ax.s, ax.e), y = fast_two_sum(ay.s, ay.e);
+      Acc2 v = acc_first2(b, wb);
+      acc_prod2(v, d, wd);
+      const DF x = fast_two_sum(v.s.x, v.e.x), y = fast_two_sum(v.s.y, v.e.y);
       // the quotient in double-float: q_hi, then the residual's quotient
       const float inv = 1.f / den.hi;
       const float qx = x.hi * inv, qy = y.hi * inv;
@@ -193,7 +195,7 @@ __device__ __forceinline__ DF2 g_rel_comp_df(const Seg& g, float t) {
       return DF2{fast_two_sum(qx, rx.hi * inv), fast_two_sum(qy, ry.hi * inv)};
     }
     default:
-      return DF2{df_mul_f(dx, t), df_mul_f(dy, t)};
+      return DF2{df_mul_f(DF{d.hi.x, d.lo.x}, t), df_mul_f(DF{d.hi.y, d.lo.y}, t)};
   }
 }
 __device__ __forceinline__ float2 g_rel_comp(const Seg& g, float t) {

@@ -187,45 +187,44 @@ __device__ __noinline__ bool solve_t64(const Seg& g, double sn, double cs, doubl
 // The power-form coefficients of solve_coeffs describe the same function.
 __device__ __forceinline__ float hn_resid(const Seg& g, float t, DF nx, DF ny) {
   const DF U = two_sum(1.f, -t);
-  DF2 d0, d1, d2;
+  auto vec = [](float2 b, float2 a) { return two_diff2(f2_pt(b), f2_pt(a)); };
+  DFP d0, d1, d2;
   DF w0, w1, w2;
   switch (g.type) {
     case PS_CUBIC:
-      d0 = df_vec(g.B, g.A); d1 = df_vec(g.C, g.B); d2 = df_vec(g.D, g.C);
+      d0 = vec(g.B, g.A); d1 = vec(g.C, g.B); d2 = vec(g.D, g.C);
       w0 = df_mul(U, U); w1 = df_mul_f(U, 2.f * t); w2 = two_prod(t, t);
       break;
     case PS_QUAD:
-      d0 = df_vec(g.B, g.A); d1 = df_vec(g.D, g.B); d2 = d1;
+      d0 = vec(g.B, g.A); d1 = vec(g.D, g.B); d2 = d1;
       w0 = U; w1 = DF{t, 0.f}; w2 = DF{0.f, 0.f};
       break;
     default:
-      d0 = df_vec(g.B, g.A); d1 = df_vec(g.D, g.A); d2 = df_vec(g.D, g.B);
+      d0 = vec(g.B, g.A); d1 = vec(g.D, g.A); d2 = vec(g.D, g.B);
       w0 = df_mul_f(df_mul(U, U), g.w); w1 = df_mul_f(U, t); w2 = df_mul_f(two_prod(t, t), g.w);
       break;
   }
-  Acc hx = acc_first(d0.x, w0), hy = acc_first(d0.y, w0);
-  acc_prod(hx, d1.x, w1); acc_prod(hy, d1.y, w1);
-  acc_prod(hx, d2.x, w2); acc_prod(hy, d2.y, w2);
-  Acc f = acc_first(acc_df(hx), nx);
-  acc_prod(f, acc_df(hy), ny);
+  Acc2 h = acc_first2(d0, w0);
+  acc_prod2(h, d1, w1);
+  acc_prod2(h, d2, w2);
+  Acc f = acc_first(DF{h.s.x, h.e.x}, nx);
+  acc_prod(f, DF{h.s.y, h.e.y}, ny);
   return acc_round(f);
 }
 
 // H(t).N as a power-form quadratic a + b t + c t^2 with double-float
 // coefficients (the differences exact as pairs, N a pair).
 __device__ __forceinline__ void hn_coeffs_df(const Seg& g, DF nx, DF ny, DF& a, DF& b, DF& c) {
-  DF2 d0, d1, d2;
-  switch (g.type) {
-    case PS_CUBIC: d0 = df_vec(g.B, g.A); d1 = df_vec(g.C, g.B); d2 = df_vec(g.D, g.C); break;
-    case PS_QUAD: d0 = df_vec(g.B, g.A); d1 = df_vec(g.D, g.B); d2 = d1; break;
-    default: d0 = df_vec(g.B, g.A); d1 = df_vec(g.D, g.A); d2 = df_vec(g.D, g.B); break;
-  }
-  auto dotn = [&](DF2 d) {
-    Acc A = acc_first(d.x, nx);
-    acc_prod(A, d.y, ny);
-    return fast_two_sum(A.s, A.e);
-  };
-  const DF e0 = dotn(d0), e1 = dotn(d1), e2 = dotn(d2);
+  // the differences' end points: d0 and d1 side by side, d2 in x and y
+  const float2 p1 = g.type == PS_CUBIC ? g.C : g.D, q1 = g.type == PS_CONIC ? g.A : g.B;
+  const float2 q2 = g.type == PS_CUBIC ? g.C : g.B;
+  Acc2 e = acc_first2(two_diff2(F2{g.B.x, p1.x}, F2{g.A.x, q1.x}), nx);
+  acc_prod2(e, two_diff2(F2{g.B.y, p1.y}, F2{g.A.y, q1.y}), ny);
+  const DFP e01 = fast_two_sum2(e.s, e.e);
+  const DFP d2 = two_diff2(f2_pt(g.D), f2_pt(q2));
+  Acc f = acc_first(DF{d2.hi.x, d2.lo.x}, nx);
+  acc_prod(f, DF{d2.hi.y, d2.lo.y}, ny);
+  const DF e0{e01.hi.x, e01.lo.x}, e1{e01.hi.y, e01.lo.y}, e2 = fast_two_sum(f.s, f.e);
   switch (g.type) {
     case PS_CUBIC:  // e0 u^2 + 2 e1 u t + e2 t^2
       a = e0;
@@ -1501,9 +1500,11 @@ __device__ __forceinline__ RibEval eval_rib_mx(const LinkRec* __restrict__ L, in
     rp = df_mul_f(df_sqrt2(), rP);
   }
   // N = A + g - rn n, P = A + g + rp n, n = (-sin psi, cos psi)
-  const DF sx = two_sum(ax, gx.hi), sy = two_sum(ay, gy.hi);
-  float4 v = make_float4(sum_prod_round(sx, gx.lo, sn, rn), sum_prod_round(sy, gy.lo, df_neg(cs), rn),
-                         sum_prod_round(sx, gx.lo, df_neg(sn), rp), sum_prod_round(sy, gy.lo, cs, rp));
+  const DFP s1 = two_sum2(F2{ax, ay}, F2{gx.hi, gy.hi});
+  const F2 gl{gx.lo, gy.lo};
+  const DFP n{F2{sn.hi, -cs.hi}, F2{sn.lo, -cs.lo}};  // -(-sin psi, cos psi)
+  const F2 vn = sum_prod_round2(s1, gl, n, rn), vp = sum_prod_round2(s1, gl, n, df_neg(rp));
+  float4 v = make_float4(vn.x, vn.y, vp.x, vp.y);
   if ((meta & META_FLAG_OVERRIDE) && (j == 1 || j == 2)) {
     const float4 vv = __ldg(reinterpret_cast<const float4*>(&L->v1));
     const float2 o = j == 1 ? mk(vv.x, vv.y) : mk(vv.z, vv.w);
