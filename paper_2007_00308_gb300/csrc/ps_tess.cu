@@ -113,24 +113,18 @@ __device__ __forceinline__ bool solve_t32(const Seg& g, float sn, float cs, floa
   float2 N = mk(-sn, cs), T = mk(cs, sn);
   solve_coeffs<float>(g, N, a, b, c);
   float disc = b * b - 4.f * a * c, scale = b * b + fabsf(4.f * a * c);
-  float r[2];
+  float r[2] = {0.f, 0.f};
   int n = FAST ? quad_roots_fast(a, b, c, disc, scale, 1e-5f, r)
                : quad_roots<float>(a, b, c, disc, scale, 1e-5f, r);
-  float best = 0.f, bestv = -3.0e38f;
-  bool found = false;
-  for (int i = 0; i < n; ++i) {
-    float t = r[i];
-    if (!(t >= pa - 1e-5f && t <= pb + 1e-5f)) continue;
-    t = fminf(fmaxf(t, pa), pb);
-    float v = dot2(hodo(g, t), T);
-    if (!found || v > bestv) {
-      bestv = v;
-      best = t;
-      found = true;
-    }
-  }
-  if (found) {
-    t_out = best;
+  auto in_range = [&](float t) { return t >= pa - 1e-5f && t <= pb + 1e-5f; };
+  const bool in0 = n > 0 && in_range(r[0]), in1 = n > 1 && in_range(r[1]);
+  if (in0 || in1) {
+    const float t1 = fminf(fmaxf(r[1], pa), pb);
+    t_out = in0 ? fminf(fmaxf(r[0], pa), pb) : t1;
+    // the tangents only where they decide: an interval turns by pi at most and seldom holds both
+    // roots (k_emit with the tangent taken at every root in range: 1,608 us against 1,544 on the
+    // 43 M ribs of the bench workload, 9.11 ms against 8.56 on 211 M ribs of near cusps)
+    if (in0 && in1 && dot2(hodo(g, t1), T) > dot2(hodo(g, t_out), T)) t_out = t1;
     return true;
   }
   float fa = fabsf(dot2(hodo(g, pa), N)), fb = fabsf(dot2(hodo(g, pb), N));
@@ -254,7 +248,7 @@ __device__ __noinline__ DF solve_t_quad_df(const Seg& g, DF sn, DF cs, DF pa, DF
   const DF nx = df_neg(sn);
   DF a, b, c;
   hn_coeffs_df(g, nx, cs, a, b, c);
-  DF r[2];
+  DF r[2] = {{0.f, 0.f}, {0.f, 0.f}};
   int n = 0;
   if (df_is0(c)) {
     if (!df_is0(b)) r[n++] = df_neg(df_div(a, b));
@@ -277,22 +271,16 @@ __device__ __noinline__ DF solve_t_quad_df(const Seg& g, DF sn, DF cs, DF pa, DF
   }
   const DF lo = df_add_f(pa, -1e-12f), hi = df_add_f(pb, 1e-12f);
   const float2 T = mk(cs.hi, sn.hi);
-  DF best = pa;
-  float bestv = -3.0e38f;
-  bool found = false;
-  for (int i = 0; i < n; ++i) {
-    DF t = r[i];
-    if (df_lt(t, lo) || df_lt(hi, t)) continue;
-    if (df_lt(t, pa)) t = pa;
-    if (df_lt(pb, t)) t = pb;
-    const float v = dot2(hodo(g, t.hi), T);
-    if (!found || v > bestv) {
-      bestv = v;
-      best = t;
-      found = true;
-    }
+  bool in[2];
+#pragma unroll
+  for (int i = 0; i < 2; ++i) {
+    in[i] = i < n && !(df_lt(r[i], lo) || df_lt(hi, r[i]));
+    if (df_lt(r[i], pa)) r[i] = pa;
+    if (df_lt(pb, r[i])) r[i] = pb;
   }
-  if (found) return best;
+  if (in[0] && in[1]) return dot2(hodo(g, r[1].hi), T) > dot2(hodo(g, r[0].hi), T) ? r[1] : r[0];
+  if (in[0]) return r[0];
+  if (in[1]) return r[1];
   const float2 N = mk(nx.hi, cs.hi);
   const float fa = fabsf(dot2(hodo(g, pa.hi), N)), fb = fabsf(dot2(hodo(g, pb.hi), N));
   return fa < fb ? pa : pb;
