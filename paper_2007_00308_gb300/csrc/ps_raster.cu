@@ -648,6 +648,7 @@ constexpr uint32_t EL_TRI1_NEG = 0xCu | 0xBu << 4 | 0x2u << 8;   // 0->3 3->2 2-
 // |A| + |B| < 2^17 (inside the fast form's 2^18), and the fast-form constant
 // A (8 - x) + B (8 - y) is formed in int64 (|8 - x| < 2^16 + 4104, as the quad
 // meets the tile) and clamped into int32.  One code path serves all classes.
+template <bool EXACT>
 __device__ __forceinline__ int setup_small(const QuadFix& q, int ymin, int ymax, int tw, int th,
                                            EntrySetup& E, int* __restrict__ sc) {
   const int X0 = q.x[0], Y0 = q.y[0], X1 = q.x[1], Y1 = q.y[1];  // N0 P0
@@ -707,7 +708,8 @@ __device__ __forceinline__ int setup_small(const QuadFix& q, int ymin, int ymax,
     long long c64 = (long long)A * (8 - xa) + (long long)B * (8 - ya);
     int lim = 4080 * S + 1;
     int c = (int)(c64 > lim ? lim : (c64 < -lim ? -lim : c64));
-    *reinterpret_cast<int4*>(&E.e[i]) = make_int4(A, B, c + 240 * A + 176 * B, 16 * A + 80 * B);
+    if (!EXACT)  // (the exact form keeps the polygon's edges, store_exact)
+      *reinterpret_cast<int4*>(&E.e[i]) = make_int4(A, B, c + 240 * A + 176 * B, 16 * A + 80 * B);
     float fa = (float)A;
     float k = __fdividef((float)-B, fa), u = __fdividef((float)-c, fa);
     float eps = 4.f + 1e-6f * (fabsf(u) + 4096.f * fabsf(k));
@@ -726,7 +728,7 @@ __device__ __forceinline__ int setup_small(const QuadFix& q, int ymin, int ymax,
     uh[i] = A < 0 ? hi_b : -INFINITY;
   }
   E.valid = cls | (a0 != 0 ? 1 : 0) | (a1 != 0 ? 2 : 0);
-  if (two) {
+  if (!EXACT && two) {
     // With F(p) = cross(P1 - N0, p - N0), triangle 0's diagonal edge is
     // -sgn(a0) F and triangle 1's is sgn(a1) F.  When a0 and a1 have the same
     // sign the triangles lie on opposite sides and triangle 1 needs e[0] <= 0,
@@ -976,7 +978,7 @@ __device__ __forceinline__ int setup_edges(const float4 ra, const float4 rb, int
     int mny = min(min(q.y[0], q.y[1]), min(q.y[2], q.y[3]));
     int mxy = max(max(q.y[0], q.y[1]), max(q.y[2], q.y[3]));
     if (mxx - mnx < (1 << 16) && mxy - mny < (1 << 16)) {
-      int tot = setup_small(q, mny, mxy, tw, th, E, sc);
+      int tot = setup_small<EXACT>(q, mny, mxy, tw, th, E, sc);
       if (EXACT && tot > 0) store_exact(q, E);
       return tot;
     }
