@@ -1354,9 +1354,9 @@ __global__ void __launch_bounds__(SETUP_NT, 2) k_link_setup(
 // copy of all the rib code).  No block-wide synchronisation.  The chunk length follows
 // the rib count: with 32 slabs whatever the count, 9,937 ribs kept ten warps of the chip
 // busy for 74 us, and 7.5 M ribs took three rounds over the warps and a sliver,
-// 414 us; 10 and 350 us this way, and 1.69 ms for 43 M ribs (1.74), 10.1 ms for the 211 M
-// of a million near-cusp cubics (12.2: their chunks' first ribs were often the
-// costly ones).
+// 414 us; 10 and 350 us this way, 43 M ribs 1.74 -> 1.69 ms and the 211 M of a million
+// near-cusp cubics 12.2 -> 10.1 ms (their chunks' first ribs were often the costly
+// ones), before the packed pairs and the tangents left out (1.54 and 8.56 ms since).
 constexpr int EMIT_NT = 256;
 constexpr int EMIT_K = 32;  // most slabs of 32 ribs per chunk by default (tunable: 4, 8, 16, 32, 64)
 
