@@ -392,15 +392,15 @@ def alu_peak_tests(sm_mhz, ops):
 
 # DRAM traffic of one k_coverage launch per bin entry, from an ncu capture of
 # the first 1,000 paths of the workload (dram__bytes_read.sum + write.sum =
-# 124.4 MB over 8,357,160 bin entries); scaled to the launch by its bin
+# 123.5 MB over 8,357,160 bin entries); scaled to the launch by its bin
 # entries.
-COVERAGE_TRAFFIC_PER_PAIR = (117.854208e6 + 6.578688e6) / 8357160
+COVERAGE_TRAFFIC_PER_PAIR = (117.552384e6 + 5.908224e6) / 8357160
 
 
 AUTOTUNE = True
 
 
-TESS_KERNELS = ("k_link_path", "k_link_setup", "k_emit", "k_arclen_scan")
+TESS_KERNELS = ("k_link_setup", "k_emit", "k_arclen_scan")
 
 
 def tessellation_only(kmean: dict, n_seg: int, world: int) -> dict:
