@@ -317,7 +317,7 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
     const unsigned long long* __restrict__ word, const __grid_constant__ DashOut D,
     CapTask* __restrict__ tasks, int32_t* counters, int32_t* status) {
   __shared__ uint8_t s_queue[DASH_NT / 32][EMIT_WQ];  // a warp's queued quads
-  dep_wait();
+  dep_wait(word);
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -472,7 +472,7 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
 __global__ void __launch_bounds__(DASH_NT) k_dash_caps(const CapTask* __restrict__ tasks, int J,
                                                        const __grid_constant__ DashOut D,
                                                        const int32_t* __restrict__ counters) {
-  dep_wait();
+  dep_wait(tasks, counters);
   const int n = counters[8], lane = threadIdx.x & 31;
   const int stride = gridDim.x * (DASH_NT / 32);
   for (int i = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; i < n; i += stride) {

@@ -224,7 +224,7 @@ __global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 6) k_bin(const float4*
                                                 RasterClear clear, int32_t* status) {
   __shared__ BinQuad s_q[BIN_NT];
   __shared__ int s_pre[BIN_NT / 32][33];
-  if (PASS == 1) dep_wait();
+  if (PASS == 1) dep_wait(off, hits);
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -234,7 +234,7 @@ __global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 6) k_bin(const float4*
   for (int64_t base = (int64_t)blockIdx.x * BIN_NT; base < R; base += stride) {
     const int64_t r = base + threadIdx.x;
     const bool in = r >= 1 && r < R;
-    const uint2 hb = PASS == 1 && in ? __ldg(hits + r) : make_uint2(0u, 0u);
+    const uint2 hb = PASS == 1 && in ? hits[r] : make_uint2(0u, 0u);
     const uint32_t h = hb.x;
     const bool direct1 = PASS == 1 && (h & HITS_DIRECT) && h != HITS_RETEST;
     const bool boxed1 = PASS == 1 && h != 0u && !direct1 && h != HITS_RETEST;
@@ -443,7 +443,7 @@ __global__ void __launch_bounds__(TS_NT) k_tile_scan(const int32_t* __restrict__
   __shared__ long long s_pre;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long i0 = (long long)blockIdx.x * TS_TILE + (long long)threadIdx.x * TS_IPT;
-  dep_wait();
+  dep_wait(count);
   int c[TS_IPT];
   if (i0 + TS_IPT <= n_tile) {
     const int4* cp = reinterpret_cast<const int4*>(count + i0);
@@ -1324,7 +1324,7 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
   __shared__ __align__(16) float4 s_pre_rib[CV_WARPS][2][32];
   __shared__ uint32_t s_pre_tag[CV_WARPS][32];
 
-  dep_wait();
+  dep_wait(off, bin, tile_list);
   const int n_list = tile_list[n_tile];  // tiles with entries (the canvas is cleared)
   if ((int)blockIdx.x >= n_list) return;  // the others' tickets reach every tile
   for (int i = threadIdx.x; i < SLOTS * MASK_WORDS; i += CV_NT) s_mask[i] = 0u;

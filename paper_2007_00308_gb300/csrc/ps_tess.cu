@@ -1369,34 +1369,34 @@ struct RibEval {
 };
 
 // One rib, FP32 (PS_PREC_FP32).
-__device__ __forceinline__ RibEval eval_rib32(const LinkRec* __restrict__ L, int j) {
+__device__ __forceinline__ RibEval eval_rib32(const LinkRec* L, int j) {
   // fields are read where needed (L1-cached) instead of copying the record
   RibEval R;
-  uint32_t meta = __ldg(&L->meta);
+  uint32_t meta = L->meta;
   int kind = META_KIND(meta);
   int M = META_M(meta);
-  float4 p01 = __ldg(reinterpret_cast<const float4*>(L->P));
-  float rN = __ldg(&L->rN), rP = __ldg(&L->rP);
+  float4 p01 = *reinterpret_cast<const float4*>(L->P);
+  float rN = L->rN, rP = L->rP;
   R.tlo = 0.f;
   R.glo = mk(0.f, 0.f);
   if (kind == LK_SEG) {
     Seg g;
-    float4 p23 = __ldg(reinterpret_cast<const float4*>(L->P) + 1);
+    float4 p23 = reinterpret_cast<const float4*>(L->P)[1];
     g.type = META_TYPE(meta);
     g.A = mk(p01.x, p01.y); g.B = mk(p01.z, p01.w); g.C = mk(p23.x, p23.y); g.D = mk(p23.z, p23.w);
-    g.w = __ldg(&L->w);
+    g.w = L->w;
     int k = 0;
-    while (k < M && j >= (int)__ldg(&L->dsum[k + 1])) ++k;
+    while (k < M && j >= (int)L->dsum[k + 1]) ++k;
     // k == M only for j == N; boundary when j == dsum[k]
     float t, psi;
-    int dk = (int)__ldg(&L->dsum[k]);
+    int dk = (int)L->dsum[k];
     bool bnd = j == dk;
-    psi = bnd ? __ldg(&L->psi[k]) : __ldg(&L->psi[k]) + __ldg(&L->step[k]) * (float)(j - dk);
+    psi = bnd ? L->psi[k] : L->psi[k] + L->step[k] * (float)(j - dk);
     float sn, cs;
     sincosf(psi, &sn, &cs);
-    float pa = __ldg(&L->p[k]);
+    float pa = L->p[k];
     if (bnd || META_PIVOT(meta, k)) t = pa;
-    else t = solve_t(g, sn, cs, pa, __ldg(&L->p[k + 1]));
+    else t = solve_t(g, sn, cs, pa, L->p[k + 1]);
     float2 n = mk(-sn, cs);
     float2 gr = g_rel(g, t);
     float2 Nv = gr - n * rN, Pv = gr + n * rP;
@@ -1405,8 +1405,8 @@ __device__ __forceinline__ RibEval eval_rib32(const LinkRec* __restrict__ L, int
     R.t = t;
     R.seg = true;
   } else {
-    int J = (int)__ldg(&L->dsum[1]);
-    float psi = (j == J) ? __ldg(&L->psi[1]) : __ldg(&L->psi[0]) + __ldg(&L->step[0]) * (float)j;
+    int J = (int)L->dsum[1];
+    float psi = (j == J) ? L->psi[1] : L->psi[0] + L->step[0] * (float)j;
     float sn, cs;
     sincosf(psi, &sn, &cs);
     float2 n = mk(-sn, cs);
@@ -1418,7 +1418,7 @@ __device__ __forceinline__ RibEval eval_rib32(const LinkRec* __restrict__ L, int
     float2 at = mk(p01.x, p01.y);
     float2 Nv = at - n * rn, Pv = at + n * rp;
     if ((meta & META_FLAG_OVERRIDE) && (j == 1 || j == 2)) {
-      float4 vv = __ldg(reinterpret_cast<const float4*>(&L->v1));
+      float4 vv = *reinterpret_cast<const float4*>(&L->v1);
       float2 v = j == 1 ? mk(vv.x, vv.y) : mk(vv.z, vv.w);
       if (rN > 0.f) Nv = v; else Pv = v;
     }
@@ -1430,28 +1430,28 @@ __device__ __forceinline__ RibEval eval_rib32(const LinkRec* __restrict__ L, int
   return R;
 }
 
-__device__ __forceinline__ DF ld_pair(const float* hi, const float* lo) { return DF{__ldg(hi), __ldg(lo)}; }
+__device__ __forceinline__ DF ld_pair(const float* hi, const float* lo) { return DF{*hi, *lo}; }
 
 // One rib, PS_PREC_MIXED: psi(j) = Psi_k + step_k (j - Delta_Sigma(k)) as a
 // pair, its normal by the double-float sincos (one call for every kind of
 // link), t by the double-float solve, g(t) compensated, and each vertex
 // coordinate summed in double-float and rounded once (Eq. 14-17).
-__device__ __forceinline__ RibEval eval_rib_mx(const LinkRec* __restrict__ L, int j) {
+__device__ __forceinline__ RibEval eval_rib_mx(const LinkRec* L, int j) {
   RibEval R;
-  const uint32_t meta = __ldg(&L->meta);
+  const uint32_t meta = L->meta;
   const int kind = META_KIND(meta);
-  const float4 p01 = __ldg(reinterpret_cast<const float4*>(L->P));
-  const float rN = __ldg(&L->rN), rP = __ldg(&L->rP);
+  const float4 p01 = *reinterpret_cast<const float4*>(L->P);
+  const float rN = L->rN, rP = L->rP;
   const bool seg = kind == LK_SEG;
   // the rib's angle
   int k = 0, dk = 0;
   DF psi;
   if (seg) {
     const int M = META_M(meta);
-    while (k < M && j >= (int)__ldg(&L->dsum[k + 1])) ++k;
-    dk = (int)__ldg(&L->dsum[k]);
+    while (k < M && j >= (int)L->dsum[k + 1]) ++k;
+    dk = (int)L->dsum[k];
   } else {
-    dk = j == (int)__ldg(&L->dsum[1]) ? j : 0;  // the last pivot rib is Psi_1 itself
+    dk = j == (int)L->dsum[1] ? j : 0;  // the last pivot rib is Psi_1 itself
     k = dk ? 1 : 0;
   }
   psi = ld_pair(&L->psi[k], &L->psi_lo[k]);
@@ -1468,10 +1468,10 @@ __device__ __forceinline__ RibEval eval_rib_mx(const LinkRec* __restrict__ L, in
   R.tlo = 0.f;
   if (seg) {
     Seg g;
-    const float4 p23 = __ldg(reinterpret_cast<const float4*>(L->P) + 1);
+    const float4 p23 = reinterpret_cast<const float4*>(L->P)[1];
     g.type = META_TYPE(meta);
     g.A = mk(p01.x, p01.y); g.B = mk(p01.z, p01.w); g.C = mk(p23.x, p23.y); g.D = mk(p23.z, p23.w);
-    g.w = __ldg(&L->w);
+    g.w = L->w;
     const DF pa = ld_pair(&L->p[k], &L->p_lo[k]);
     DF t = pa;
     if (j != dk && !META_PIVOT(meta, k))
@@ -1494,7 +1494,7 @@ __device__ __forceinline__ RibEval eval_rib_mx(const LinkRec* __restrict__ L, in
   const F2 vn = sum_prod_round2(s1, gl, n, rn), vp = sum_prod_round2(s1, gl, n, df_neg(rp));
   float4 v = make_float4(vn.x, vn.y, vp.x, vp.y);
   if ((meta & META_FLAG_OVERRIDE) && (j == 1 || j == 2)) {
-    const float4 vv = __ldg(reinterpret_cast<const float4*>(&L->v1));
+    const float4 vv = *reinterpret_cast<const float4*>(&L->v1);
     const float2 o = j == 1 ? mk(vv.x, vv.y) : mk(vv.z, vv.w);
     if (rN > 0.f) { v.x = o.x; v.y = o.y; } else { v.z = o.x; v.w = o.y; }
   }
@@ -1504,7 +1504,7 @@ __device__ __forceinline__ RibEval eval_rib_mx(const LinkRec* __restrict__ L, in
 }
 
 template <bool MIXED>
-__device__ __forceinline__ RibEval eval_rib(const LinkRec* __restrict__ L, int j) {
+__device__ __forceinline__ RibEval eval_rib(const LinkRec* L, int j) {
   if constexpr (MIXED) return eval_rib_mx(L, j);
   else return eval_rib32(L, j);
 }
@@ -1515,7 +1515,7 @@ __global__ void __launch_bounds__(EMIT_NT, MIXED ? 2 : 3) k_emit(
     const int32_t* __restrict__ link_path, int64_t n_link, const int64_t* __restrict__ n_rib,
     int64_t capacity, float4* __restrict__ rib, uint32_t* __restrict__ tag,
     float* __restrict__ chord, float* __restrict__ tout, int most_slabs) {
-  dep_wait();
+  dep_wait(recs, link_off, link_path, n_rib);
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31;
@@ -1545,12 +1545,12 @@ __global__ void __launch_bounds__(EMIT_NT, MIXED ? 2 : 3) k_emit(
       E.seg = false;
       int j = 0;
       if (active) {
-        while (l + 1 < n_link && (int64_t)__ldg(link_off + l + 1) <= r) ++l;
-        j = (int)(r - __ldg(link_off + l));
+        while (l + 1 < n_link && (int64_t)link_off[l + 1] <= r) ++l;
+        j = (int)(r - link_off[l]);
         E = eval_rib<MIXED>(recs + l, j);
         if (write) {
           rib[r] = E.v;
-          uint32_t p = (uint32_t)__ldg(link_path + l);
+          uint32_t p = (uint32_t)link_path[l];
           tag[r] = (p << 2) | (E.seg ? PS_TAG_SEGMENT : 0u) | (j == 0 ? PS_TAG_LINK_START : 0u);
           if (tout) tout[r] = E.t + E.tlo;
         }
@@ -1613,8 +1613,9 @@ constexpr int SCAN_TILE = SCAN_NT * SCAN_IPT;
 // tile sums are FP32 (relative error ~1e-6 of s); the carry between tiles,
 // which runs over a whole path, is a double-float pair from a warp-wide
 // look-back.
+// (Three CTAs per SM for the form without vectors, which the compiler gives up otherwise.)
 template <bool VEC>
-__global__ void __launch_bounds__(SCAN_NT) k_arclen_scan(
+__global__ void __launch_bounds__(SCAN_NT, VEC ? 1 : 3) k_arclen_scan(
     const float* chord_in, const uint32_t* __restrict__ tag, const int64_t* __restrict__ n_rib,
     int64_t capacity, float* s_out, float* __restrict__ path_len, TileState* state,
     int32_t* counters, int32_t* status) {
@@ -1623,7 +1624,7 @@ __global__ void __launch_bounds__(SCAN_NT) k_arclen_scan(
   __shared__ float s_carry[2];
   __shared__ int64_t s_tile;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  dep_wait();
+  dep_wait(chord_in, tag, n_rib);
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int64_t n_tiles = (R + SCAN_TILE - 1) / SCAN_TILE;
@@ -1649,7 +1650,7 @@ __global__ void __launch_bounds__(SCAN_NT) k_arclen_scan(
 #pragma unroll
       for (int q = 0; q < SCAN_IPT / 4; ++q) {
         float4 a = cp[q];
-        uint4 b = __ldg(tp + q);
+        uint4 b = tp[q];
         c[4 * q] = a.x; c[4 * q + 1] = a.y; c[4 * q + 2] = a.z; c[4 * q + 3] = a.w;
         pth[4 * q] = b.x >> 2; pth[4 * q + 1] = b.y >> 2;
         pth[4 * q + 2] = b.z >> 2; pth[4 * q + 3] = b.w >> 2;
@@ -1659,12 +1660,12 @@ __global__ void __launch_bounds__(SCAN_NT) k_arclen_scan(
       for (int i = 0; i < SCAN_IPT; ++i) {
         int64_t r = base + i;
         c[i] = r < R ? chord_in[r] : 0.f;
-        pth[i] = r < R ? (__ldg(tag + r) >> 2) : 0xffffffffu;
+        pth[i] = r < R ? tag[r] >> 2 : 0xffffffffu;
       }
     }
     // path of the rib before this thread's first: the previous lane's last
     uint32_t prevp = __shfl_up_sync(0xffffffffu, pth[SCAN_IPT - 1], 1);
-    if (lane == 0) prevp = (base > 0 && base <= R) ? (__ldg(tag + base - 1) >> 2) : 0xffffffffu;
+    if (lane == 0) prevp = (base > 0 && base <= R) ? tag[base - 1] >> 2 : 0xffffffffu;
     uint32_t hm = 0;  // bit i: rib base + i starts a path
     float acc = 0.f;
 #pragma unroll
@@ -1721,7 +1722,7 @@ __global__ void __launch_bounds__(SCAN_NT) k_arclen_scan(
     }
     // path of the rib after this thread's last: the next lane's first
     uint32_t nextp = __shfl_down_sync(0xffffffffu, pth[0], 1);
-    if (lane == 31) nextp = base + SCAN_IPT < R ? (__ldg(tag + base + SCAN_IPT) >> 2) : 0xffffffffu;
+    if (lane == 31) nextp = base + SCAN_IPT < R ? tag[base + SCAN_IPT] >> 2 : 0xffffffffu;
     // ribs before this thread's first head continue the running total
     const DF tile_carry = (hprev || whead) ? DF{0.f, 0.f} : DF{s_carry[0], s_carry[1]};
     float run = hprev ? vprev : vprev + wcarry;
