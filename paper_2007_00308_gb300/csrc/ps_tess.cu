@@ -1547,10 +1547,10 @@ __global__ void __launch_bounds__(EMIT_NT, MIXED ? 2 : 3) k_emit(
       if (active) {
         while (l + 1 < n_link && (int64_t)link_off[l + 1] <= r) ++l;
         j = (int)(r - link_off[l]);
+        const uint32_t p = (uint32_t)link_path[l];  // (before the rib: its latency hides there)
         E = eval_rib<MIXED>(recs + l, j);
         if (write) {
           rib[r] = E.v;
-          uint32_t p = (uint32_t)link_path[l];
           tag[r] = (p << 2) | (E.seg ? PS_TAG_SEGMENT : 0u) | (j == 0 ? PS_TAG_LINK_START : 0u);
           if (tout) tout[r] = E.t + E.tlo;
         }
