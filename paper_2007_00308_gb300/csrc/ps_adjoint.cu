@@ -578,9 +578,8 @@ static int backward(ps_context* ctx, const ps_segments* seg, const ps_paths* pat
   size_t o_nr = (o_tot + sizeof(float) * (P + 1) + 15) & ~(size_t)15;
   size_t bytes = o_nr + 16;
   if (bytes > ctx->adj_bytes) {
-    if (ctx->d_adj) cudaFree(ctx->d_adj);
-    ctx->d_adj = nullptr;
-    if (cudaMalloc(&ctx->d_adj, bytes) != cudaSuccess) return PS_ERR_CUDA;
+    ctx->adj_bytes = 0;
+    if (ps_grow(&ctx->d_adj, bytes) != PS_OK) return PS_ERR_CUDA;
     ctx->adj_bytes = bytes;
   }
   char* w = (char*)ctx->d_adj;

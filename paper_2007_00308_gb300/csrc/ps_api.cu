@@ -9,19 +9,29 @@
 
 int ps_cuda_check(cudaError_t e) { return e == cudaSuccess ? PS_OK : PS_ERR_CUDA; }
 
-static int grow(void** p, size_t bytes) {
+// Replaces a block by a larger one.  The old one goes first, and with it whatever its
+// capacity promised: callers set the capacity to 0 before, and to its value once the
+// new block is there, so that a call after a failed one asks again.
+int ps_grow(void** p, size_t bytes) {
   if (*p) cudaFree(*p);
   *p = nullptr;
   if (bytes == 0) return PS_OK;
-  return ps_cuda_check(cudaMalloc(p, bytes));
+  const int rc = ps_cuda_check(cudaMalloc(p, bytes));
+  if (rc != PS_OK) {
+    *p = nullptr;
+    cudaGetLastError();  // returned here, not by the next launch's check
+  }
+  return rc;
 }
 
 int ps_ensure_tiles(ps_context* ctx, int64_t n) {
   if (n <= ctx->tile_cap) return PS_OK;
   int64_t cap = n + n / 4 + 64;
   int rc;
+  ctx->tile_cap = 0;
+  ctx->d_tile_state = nullptr;
   // the ticket counters (64 bytes), then the states
-  if ((rc = grow((void**)&ctx->d_counters, 64 + sizeof(TileState) * cap)) != PS_OK) return rc;
+  if ((rc = ps_grow((void**)&ctx->d_counters, 64 + sizeof(TileState) * cap)) != PS_OK) return rc;
   ctx->d_tile_state = reinterpret_cast<TileState*>(ctx->d_counters + 16);
   ctx->tile_cap = cap;
   return PS_OK;
@@ -30,8 +40,9 @@ int ps_ensure_tiles(ps_context* ctx, int64_t n) {
 int ps_ensure_recs(ps_context* ctx, int64_t n_link) {
   if (n_link <= ctx->rec_cap) return PS_OK;
   int64_t cap = n_link + n_link / 4 + 64;
+  ctx->rec_cap = 0;
   // records followed by one int32 path index per link
-  int rc = grow((void**)&ctx->d_recs, (sizeof(LinkRec) + sizeof(int32_t)) * cap);
+  int rc = ps_grow((void**)&ctx->d_recs, (sizeof(LinkRec) + sizeof(int32_t)) * cap);
   if (rc != PS_OK) return rc;
   ctx->rec_cap = cap;
   return PS_OK;
@@ -41,15 +52,17 @@ int ps_ensure_raster(ps_context* ctx, int64_t n_tile, int64_t n_pair) {
   int rc;
   if (n_tile > ctx->raster_tile_cap) {
     int64_t cap = n_tile + 64;
-    if ((rc = grow((void**)&ctx->d_tile_count, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
-    if ((rc = grow((void**)&ctx->d_tile_off, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
-    if ((rc = grow((void**)&ctx->d_tile_cursor, 2 * sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
-    if ((rc = grow((void**)&ctx->d_tile_list, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
+    ctx->raster_tile_cap = 0;
+    if ((rc = ps_grow((void**)&ctx->d_tile_count, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
+    if ((rc = ps_grow((void**)&ctx->d_tile_off, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
+    if ((rc = ps_grow((void**)&ctx->d_tile_cursor, 2 * sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
+    if ((rc = ps_grow((void**)&ctx->d_tile_list, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
     ctx->raster_tile_cap = cap;
   }
   if (n_pair > ctx->pair_cap) {
     int64_t cap = n_pair + n_pair / 8 + 1024;
-    if ((rc = grow((void**)&ctx->d_bin, sizeof(uint32_t) * cap)) != PS_OK) return rc;
+    ctx->pair_cap = 0;
+    if ((rc = ps_grow((void**)&ctx->d_bin, sizeof(uint32_t) * cap)) != PS_OK) return rc;
     ctx->pair_cap = cap;
   }
   return PS_OK;
@@ -58,7 +71,8 @@ int ps_ensure_raster(ps_context* ctx, int64_t n_tile, int64_t n_pair) {
 int ps_ensure_quad_hits(ps_context* ctx, int64_t n_rib) {
   if (n_rib <= ctx->quad_hits_cap) return PS_OK;
   int64_t cap = n_rib + n_rib / 8 + 1024;
-  int rc = grow((void**)&ctx->d_quad_hits, 2 * sizeof(uint32_t) * cap);
+  ctx->quad_hits_cap = 0;
+  int rc = ps_grow((void**)&ctx->d_quad_hits, 2 * sizeof(uint32_t) * cap);
   if (rc != PS_OK) return rc;
   ctx->quad_hits_cap = cap;
   return PS_OK;

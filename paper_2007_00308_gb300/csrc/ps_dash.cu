@@ -530,11 +530,8 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
     if (need > ctx->cap_bytes) {
       cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
       if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
-        if (ctx->d_cap_tasks) cudaFree(ctx->d_cap_tasks);
-        ctx->d_cap_tasks = nullptr;
         ctx->cap_bytes = 0;
-        if (cudaMalloc(&ctx->d_cap_tasks, need) == cudaSuccess) ctx->cap_bytes = need;
-        else cudaGetLastError();  // carry on without
+        if (ps_grow(&ctx->d_cap_tasks, need) == PS_OK) ctx->cap_bytes = need;  // else carry on without
       }
     }
     if (need <= ctx->cap_bytes) tasks = static_cast<CapTask*>(ctx->d_cap_tasks);

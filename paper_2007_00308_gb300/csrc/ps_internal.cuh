@@ -305,6 +305,7 @@ static inline void ps_launch_after(bool overlap, void (*kernel)(P...), int grid,
 }
 
 // ---- host helpers -------------------------------------------------------------
+int ps_grow(void** p, size_t bytes);
 int ps_ensure_tiles(ps_context* ctx, int64_t n_tile);
 int ps_ensure_recs(ps_context* ctx, int64_t n_link);
 int ps_ensure_raster(ps_context* ctx, int64_t n_tile, int64_t n_pair);
