@@ -27,7 +27,10 @@
  *   - Sizes that depend on the data (rib count, bin entries) live in device
  *     memory; kernels read them there, so a sequence of calls can be captured
  *     in a CUDA graph once the context's workspace has been reserved (the first
- *     call with given sizes may cudaMalloc; capture the second).
+ *     call with given sizes may cudaMalloc; capture the second).  From the first
+ *     captured call on, workspace that a later, larger call outgrows is kept until
+ *     ps_destroy, as the graph may use it (under twice the size of what replaced
+ *     it, in all); the graph must not be replayed after ps_destroy.
  *   - Return codes: PS_OK or a negative PS_ERR_* for argument errors detected on
  *     the host.  Errors found by kernels (capacity exceeded, a bounded wait that
  *     gave up, out-of-range coordinates) are recorded in the context's device

@@ -563,7 +563,7 @@ static int backward(ps_context* ctx, const ps_segments* seg, const ps_paths* pat
   if (precision != PS_PREC_FP32 && precision != PS_PREC_MIXED) return PS_ERR_INVALID;
   if (paths->n_path <= 0 || seg->n_seg < 0) return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   int64_t S = seg->n_seg;
   int P = paths->n_path;
   int64_t L = 2 * S + P;
@@ -578,9 +578,10 @@ static int backward(ps_context* ctx, const ps_segments* seg, const ps_paths* pat
   size_t o_nr = (o_tot + sizeof(float) * (P + 1) + 15) & ~(size_t)15;
   size_t bytes = o_nr + 16;
   if (bytes > ctx->adj_bytes) {
+    const size_t room = (size_t)ps_grown(ctx, (int64_t)ctx->adj_bytes, (int64_t)bytes);
     ctx->adj_bytes = 0;
-    if (ps_grow(&ctx->d_adj, bytes) != PS_OK) return PS_ERR_CUDA;
-    ctx->adj_bytes = bytes;
+    if (ps_grow(ctx, &ctx->d_adj, room) != PS_OK) return PS_ERR_CUDA;
+    ctx->adj_bytes = room;
   }
   char* w = (char*)ctx->d_adj;
   int32_t* loff = (int32_t*)(w + o_loff);

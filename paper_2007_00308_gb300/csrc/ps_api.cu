@@ -9,11 +9,34 @@
 
 int ps_cuda_check(cudaError_t e) { return e == cudaSuccess ? PS_OK : PS_ERR_CUDA; }
 
+void ps_on_stream(ps_context* ctx, void* stream) {
+  ctx->last_stream = stream;
+  if (ctx->captured) return;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  if (cudaStreamIsCapturing((cudaStream_t)stream, &cs) != cudaSuccess) cudaGetLastError();
+  else if (cs != cudaStreamCaptureStatusNone) ctx->captured = 1;
+}
+
+int64_t ps_grown(const ps_context* ctx, int64_t old, int64_t want) {
+  return ctx->captured && want < old + old / 2 ? old + old / 2 : want;
+}
+
 // Replaces a block by a larger one.  The old one goes first, and with it whatever its
 // capacity promised: callers set the capacity to 0 before, and to its value once the
 // new block is there, so that a call after a failed one asks again.
-int ps_grow(void** p, size_t bytes) {
-  if (*p) cudaFree(*p);
+int ps_grow(ps_context* ctx, void** p, size_t bytes) {
+  if (*p && ctx->captured) {
+    if (ctx->n_kept == ctx->kept_cap) {
+      const int cap = 2 * ctx->kept_cap + 16;
+      void** list = (void**)realloc(ctx->kept, sizeof(void*) * cap);
+      if (!list) return PS_ERR_CUDA;
+      ctx->kept = list;
+      ctx->kept_cap = cap;
+    }
+    ctx->kept[ctx->n_kept++] = *p;
+  } else if (*p) {
+    cudaFree(*p);
+  }
   *p = nullptr;
   if (bytes == 0) return PS_OK;
   const int rc = ps_cuda_check(cudaMalloc(p, bytes));
@@ -26,12 +49,12 @@ int ps_grow(void** p, size_t bytes) {
 
 int ps_ensure_tiles(ps_context* ctx, int64_t n) {
   if (n <= ctx->tile_cap) return PS_OK;
-  int64_t cap = n + n / 4 + 64;
+  int64_t cap = ps_grown(ctx, ctx->tile_cap, n + n / 4 + 64);
   int rc;
   ctx->tile_cap = 0;
   ctx->d_tile_state = nullptr;
   // the ticket counters (64 bytes), then the states
-  if ((rc = ps_grow((void**)&ctx->d_counters, 64 + sizeof(TileState) * cap)) != PS_OK) return rc;
+  if ((rc = ps_grow(ctx, (void**)&ctx->d_counters, 64 + sizeof(TileState) * cap)) != PS_OK) return rc;
   ctx->d_tile_state = reinterpret_cast<TileState*>(ctx->d_counters + 16);
   ctx->tile_cap = cap;
   return PS_OK;
@@ -39,10 +62,10 @@ int ps_ensure_tiles(ps_context* ctx, int64_t n) {
 
 int ps_ensure_recs(ps_context* ctx, int64_t n_link) {
   if (n_link <= ctx->rec_cap) return PS_OK;
-  int64_t cap = n_link + n_link / 4 + 64;
+  int64_t cap = ps_grown(ctx, ctx->rec_cap, n_link + n_link / 4 + 64);
   ctx->rec_cap = 0;
   // records followed by one int32 path index per link
-  int rc = ps_grow((void**)&ctx->d_recs, (sizeof(LinkRec) + sizeof(int32_t)) * cap);
+  int rc = ps_grow(ctx, (void**)&ctx->d_recs, (sizeof(LinkRec) + sizeof(int32_t)) * cap);
   if (rc != PS_OK) return rc;
   ctx->rec_cap = cap;
   return PS_OK;
@@ -51,18 +74,18 @@ int ps_ensure_recs(ps_context* ctx, int64_t n_link) {
 int ps_ensure_raster(ps_context* ctx, int64_t n_tile, int64_t n_pair) {
   int rc;
   if (n_tile > ctx->raster_tile_cap) {
-    int64_t cap = n_tile + 64;
+    int64_t cap = ps_grown(ctx, ctx->raster_tile_cap, n_tile + 64);
     ctx->raster_tile_cap = 0;
-    if ((rc = ps_grow((void**)&ctx->d_tile_count, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
-    if ((rc = ps_grow((void**)&ctx->d_tile_off, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
-    if ((rc = ps_grow((void**)&ctx->d_tile_cursor, 2 * sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
-    if ((rc = ps_grow((void**)&ctx->d_tile_list, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
+    if ((rc = ps_grow(ctx, (void**)&ctx->d_tile_count, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
+    if ((rc = ps_grow(ctx, (void**)&ctx->d_tile_off, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
+    if ((rc = ps_grow(ctx, (void**)&ctx->d_tile_cursor, 2 * sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
+    if ((rc = ps_grow(ctx, (void**)&ctx->d_tile_list, sizeof(int32_t) * (cap + 1))) != PS_OK) return rc;
     ctx->raster_tile_cap = cap;
   }
   if (n_pair > ctx->pair_cap) {
-    int64_t cap = n_pair + n_pair / 8 + 1024;
+    int64_t cap = ps_grown(ctx, ctx->pair_cap, n_pair + n_pair / 8 + 1024);
     ctx->pair_cap = 0;
-    if ((rc = ps_grow((void**)&ctx->d_bin, sizeof(uint32_t) * cap)) != PS_OK) return rc;
+    if ((rc = ps_grow(ctx, (void**)&ctx->d_bin, sizeof(uint32_t) * cap)) != PS_OK) return rc;
     ctx->pair_cap = cap;
   }
   return PS_OK;
@@ -70,9 +93,9 @@ int ps_ensure_raster(ps_context* ctx, int64_t n_tile, int64_t n_pair) {
 
 int ps_ensure_quad_hits(ps_context* ctx, int64_t n_rib) {
   if (n_rib <= ctx->quad_hits_cap) return PS_OK;
-  int64_t cap = n_rib + n_rib / 8 + 1024;
+  int64_t cap = ps_grown(ctx, ctx->quad_hits_cap, n_rib + n_rib / 8 + 1024);
   ctx->quad_hits_cap = 0;
-  int rc = ps_grow((void**)&ctx->d_quad_hits, 2 * sizeof(uint32_t) * cap);
+  int rc = ps_grow(ctx, (void**)&ctx->d_quad_hits, 2 * sizeof(uint32_t) * cap);
   if (rc != PS_OK) return rc;
   ctx->quad_hits_cap = cap;
   return PS_OK;
@@ -162,6 +185,8 @@ extern "C" void ps_destroy(ps_context* ctx) {
                   ctx->d_tile_list};
   for (void* p : ptrs)
     if (p) cudaFree(p);
+  for (int i = 0; i < ctx->n_kept; ++i) cudaFree(ctx->kept[i]);
+  free(ctx->kept);
   free(ctx);
 }
 
@@ -225,7 +250,7 @@ extern "C" int ps_check_wait_timeout(ps_context* ctx, int which, void* stream) {
   }
   if (rc == PS_OK) rc = ps_cuda_check(cudaStreamSynchronize(st));
   cudaFree(buf);
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   return rc;
 }
 

@@ -509,7 +509,7 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
     P.j_round = J < 1 ? 1 : J;
   }
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   int64_t n_tiles = (capacity + DASH_TILE - 1) / DASH_TILE + 1;
   int rc = ps_ensure_tiles(ctx, n_tiles + 1);
   if (rc != PS_OK) return rc;
@@ -530,8 +530,9 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
     if (need > ctx->cap_bytes) {
       cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
       if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
+        const size_t room = (size_t)ps_grown(ctx, (int64_t)ctx->cap_bytes, (int64_t)need);
         ctx->cap_bytes = 0;
-        if (ps_grow(&ctx->d_cap_tasks, need) == PS_OK) ctx->cap_bytes = need;  // else carry on without
+        if (ps_grow(ctx, &ctx->d_cap_tasks, room) == PS_OK) ctx->cap_bytes = room;  // else carry on without
       }
     }
     if (need <= ctx->cap_bytes) tasks = static_cast<CapTask*>(ctx->d_cap_tasks);

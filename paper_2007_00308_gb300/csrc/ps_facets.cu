@@ -176,7 +176,7 @@ extern "C" int ps_uniform_tessellate(ps_context* ctx, const ps_segments* seg, co
   if (!d_rib_out || !fwd->d_rib || !fwd->d_link_rib_off || !fwd->d_n_rib) return PS_ERR_INVALID;
   if (paths->n_path <= 0 || seg->n_seg < 0 || fwd->capacity < 0) return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   int64_t L = 2 * seg->n_seg + paths->n_path;
   int grid = ps_persistent_grid(ctx, (const void*)k_uniform_ribs, FC_NT, 0);
   k_uniform_ribs<<<grid, FC_NT, 0, st>>>(seg->d_type, seg->d_pts, seg->d_w, paths->d_seg_off,
@@ -193,7 +193,7 @@ extern "C" int ps_facet_stats(ps_context* ctx, const float* d_rib, const uint32_
   if (!ctx || !d_rib || !d_tag || !d_link_rib_off || !d_n_rib || !d_stats) return PS_ERR_INVALID;
   if (n_link <= 0 || capacity < 0 || !(slack >= 0.f)) return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   cudaMemsetAsync(d_stats, 0, sizeof(float) * 4 * (size_t)n_link, st);
   int grid = ps_persistent_grid(ctx, (const void*)k_facet_stats, FC_NT, 0);
   k_facet_stats<<<grid, FC_NT, 0, st>>>(reinterpret_cast<const float4*>(d_rib), d_tag,

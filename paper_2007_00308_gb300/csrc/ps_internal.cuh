@@ -78,6 +78,9 @@ struct ps_context {
   int n_occ;
   int cov_attr_done[2];  // coverage kernels' shared-memory attribute set on this device
   void* last_stream;
+  int captured;             // a call has been captured into a graph
+  void** kept;              // blocks outgrown since, [n_kept]
+  int n_kept, kept_cap;
   int32_t* d_status;        // first error recorded by a kernel
   // scan tile states (shared by the passes of one call; calls on one context
   // are serialized on the stream they are issued to)
@@ -305,7 +308,13 @@ static inline void ps_launch_after(bool overlap, void (*kernel)(P...), int grid,
 }
 
 // ---- host helpers -------------------------------------------------------------
-int ps_grow(void** p, size_t bytes);
+// Notes the stream of a call, and whether it is being captured.  From the first capture on the
+// context gives no outgrown block back before it is destroyed: the graph holds its address.
+void ps_on_stream(ps_context* ctx, void* stream);
+// The capacity to grow to: then at least half as much again, so that the kept blocks of a
+// workspace come to less than twice the one in use.
+int64_t ps_grown(const ps_context* ctx, int64_t old, int64_t want);
+int ps_grow(ps_context* ctx, void** p, size_t bytes);
 int ps_ensure_tiles(ps_context* ctx, int64_t n_tile);
 int ps_ensure_recs(ps_context* ctx, int64_t n_link);
 int ps_ensure_raster(ps_context* ctx, int64_t n_tile, int64_t n_pair);

@@ -1685,7 +1685,7 @@ static int rasterize(ps_context* ctx, const float* d_rib, const uint32_t* d_tag,
     return PS_ERR_INVALID;
   const int y0 = row0 * 256;
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   int tiles_x = (width + TILE_PX - 1) / TILE_PX, tiles_y = (height + TILE_PX - 1) / TILE_PX;
   int64_t n_tile = (int64_t)tiles_x * tiles_y;
   if (n_tile > (1 << 26)) return PS_ERR_INVALID;
@@ -1906,7 +1906,7 @@ extern "C" int ps_route_quads(ps_context* ctx, const float* d_rib, const uint32_
   if ((int64_t)width * 256 >= COORD_LIMIT || (int64_t)height * 256 >= COORD_LIMIT)
     return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   int rc = ps_cuda_check(cudaMemsetAsync(d_dest_count, 0, sizeof(int64_t) * n_dest, st));
   if (rc != PS_OK) return rc;
   const float4* rib = reinterpret_cast<const float4*>(d_rib);

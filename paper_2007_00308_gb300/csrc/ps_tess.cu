@@ -1905,7 +1905,7 @@ extern "C" int ps_tessellate_strokes(ps_context* ctx, const ps_segments* seg,
   if (seg->n_seg < 0 || paths->n_path < 0 || seg->n_seg > (int64_t)1 << 29) return PS_ERR_INVALID;
   if (paths->n_path == 0) {
     if (seg->n_seg != 0) return PS_ERR_INVALID;
-    ctx->last_stream = stream;
+    ps_on_stream(ctx, stream);
     return empty_batch(out, (cudaStream_t)stream);
   }
   if (seg->n_seg > 0 && (!seg->d_type || !seg->d_pts)) return PS_ERR_INVALID;
@@ -1918,7 +1918,7 @@ extern "C" int ps_tessellate_strokes(ps_context* ctx, const ps_segments* seg,
   if ((flags & PS_TESS_ARCLENGTH) && !(flags & PS_TESS_COUNT_ONLY) && !out->d_s)
     return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   return launch_tessellate(ctx, seg, paths, dtheta, precision, flags, out, st, 0,
                            2 * seg->n_seg + paths->n_path);
 }
@@ -1947,7 +1947,7 @@ extern "C" int ps_link_records_sync(ps_context* ctx, const ps_segments* seg, con
       !paths->d_miter || !paths->d_closed)
     return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   int rc = launch_tessellate(ctx, seg, paths, dtheta, precision, PS_TESS_COUNT_ONLY, out, st, 0,
                              2 * seg->n_seg + paths->n_path, PH_SETUP,
                              static_cast<LinkRec*>(d_records));
@@ -1965,7 +1965,7 @@ extern "C" int ps_emit_records(ps_context* ctx, const ps_segments* seg, const ps
       out->capacity < 0 || (flags & PS_TESS_COUNT_ONLY) ||
       ((flags & PS_TESS_ARCLENGTH) && !out->d_s))
     return PS_ERR_INVALID;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   return launch_tessellate(ctx, seg, paths, 1.f, precision, flags, out, (cudaStream_t)stream, 0,
                            2 * seg->n_seg + paths->n_path, PH_RIBS,
                            static_cast<LinkRec*>(const_cast<void*>(d_records)));
@@ -2005,7 +2005,7 @@ extern "C" int ps_tessellate_links(ps_context* ctx, const ps_segments* seg,
   if ((flags & PS_TESS_ARCLENGTH) && !(flags & PS_TESS_COUNT_ONLY) && !out->d_s)
     return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   // paths whose first link lies outside the range keep -1: no rib of the range
   // starts them
   int rc = ps_cuda_check(cudaMemsetAsync(out->d_path_rib_off, 0xff,
@@ -2039,7 +2039,7 @@ extern "C" int ps_add_s_carry(ps_context* ctx, float* d_s, const uint32_t* d_tag
   if (!ctx || !d_s || !d_tag || !d_n_rib || capacity < 0 || path < 0) return PS_ERR_INVALID;
   if (with_len && !d_path_len) return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   const float hi = (float)carry, lo = (float)(carry - (double)hi);
   const int grid = ps_persistent_grid(ctx, (const void*)k_add_s_carry, 256, 0);
   k_add_s_carry<<<grid, 256, 0, st>>>(d_s, d_tag, d_n_rib, capacity, (uint32_t)path, hi, lo,
@@ -2053,7 +2053,7 @@ extern "C" int ps_arclength_scan(ps_context* ctx, const float* d_rib, const uint
   if (!ctx || !d_rib || !d_tag || !d_n_rib || !d_s || capacity < 0 || n_path < 0)
     return PS_ERR_INVALID;
   cudaStream_t st = (cudaStream_t)stream;
-  ctx->last_stream = stream;
+  ps_on_stream(ctx, stream);
   int64_t scan_tiles = (capacity + SCAN_TILE - 1) / SCAN_TILE;
   int rc = ps_ensure_tiles(ctx, scan_tiles + 2);
   if (rc != PS_OK) return rc;

@@ -1,6 +1,6 @@
 """The context's workspace on the CPU, with the runtime's allocation calls stood in for: a growth
 that fails leaves no capacity that nothing stands behind, and a later, smaller call has its
-workspace again."""
+workspace again; blocks that a captured call may have been given outlive their growth."""
 import os
 import subprocess
 
@@ -96,6 +96,45 @@ int main() {
 """
 
 
+CAPTURED = MAIN + r"""
+int main() {
+  ps_context* c = nullptr;
+  CHECK(ps_create(&c) == PS_OK);
+  auto reserve = [&](int64_t n) { return ps_reserve(c, n, n, n, n); };
+  auto blocks = [&](void** b) {
+    void* all[] = {c->d_counters, c->d_recs, c->d_bin, c->d_quad_hits, c->d_tile_count, c->d_tile_off,
+                   c->d_tile_cursor, c->d_tile_list};
+    for (int i = 0; i < 8; ++i) b[i] = all[i];
+  };
+  void *before[8], *after[8];
+  ps_on_stream(c, nullptr);
+  CHECK(reserve(2000) == PS_OK);
+  blocks(before);
+  CHECK(reserve(100000) == PS_OK);  // no capture yet: the blocks go
+  for (void* b : before) CHECK(!backed(b, 1));
+  blocks(before);
+  capture = cudaStreamCaptureStatusActive;
+  ps_on_stream(c, nullptr);
+  capture = cudaStreamCaptureStatusNone;
+  ps_on_stream(c, nullptr);
+  size_t sum = 0;
+  for (int64_t n = 100000; n < 4000000; n += 5000) {  // many small steps
+    CHECK(reserve(n) == PS_OK);
+    consistent(c);
+  }
+  blocks(after);
+  for (int i = 0; i < 8; ++i) CHECK(after[i] != before[i] && backed(before[i], 1) && backed(after[i], 1));
+  for (auto& b : live) sum += b.second;
+  const size_t now = 64 + sizeof(TileState) * c->tile_cap + (sizeof(LinkRec) + 4) * c->rec_cap +
+                     4 * c->pair_cap + 8 * c->quad_hits_cap + 20 * (c->raster_tile_cap + 1);
+  CHECK(sum < 3 * now + 4096);
+  ps_destroy(c);
+  CHECK(live.empty());
+  return errors ? 1 : 0;
+}
+"""
+
+
 def run(tmp_path, source):
     src, exe = tmp_path / "main.cu", tmp_path / "main"
     src.write_text(source)
@@ -117,3 +156,7 @@ def _nvcc():
 
 def test_failed_growth_leaves_nothing_claimed(tmp_path):
     run(tmp_path, GROWTH)
+
+
+def test_captured_blocks_are_kept(tmp_path):
+    run(tmp_path, CAPTURED)
