@@ -148,7 +148,10 @@ void ps_destroy(ps_context* ctx);
 
 /* Reserve workspace for up to n_link links, n_rib ribs, n_tile raster tiles
  * and n_pair raster bin entries (any may be 0 = keep).  Allocates with
- * cudaMalloc (synchronous); call before capturing a graph. */
+ * cudaMalloc (synchronous); call before capturing a graph.  Per rib that is 9 bytes
+ * for the dash and raster calls, which is left out without an error when there is
+ * no room for it, and a twentieth of a byte of tile states; per link 305 bytes, per
+ * tile 20, per bin entry 4.5. */
 int ps_reserve(ps_context* ctx, int64_t n_link, int64_t n_rib, int64_t n_tile, int64_t n_pair);
 
 /* Host-only static bound on the rib count of n_seg segments in n_path paths

@@ -197,9 +197,10 @@ extern "C" int ps_reserve(ps_context* ctx, int64_t n_link, int64_t n_rib, int64_
   if (n_link && (rc = ps_ensure_recs(ctx, n_link)) != PS_OK) return rc;
   int64_t tiles = (n_link + 255) / 256 + (n_rib + 2047) / 2048 + 4 + n_rib / 512;
   if ((rc = ps_ensure_tiles(ctx, tiles)) != PS_OK) return rc;
-  // the dash's and the binning's words per rib
-  if (n_rib && (rc = ps_ensure_quad_hits(ctx, n_rib)) != PS_OK) return rc;
   if ((n_tile || n_pair) && (rc = ps_ensure_raster(ctx, n_tile, n_pair)) != PS_OK) return rc;
+  // the dash's and the binning's words per rib, if there is room: callers that only tessellate
+  // have no use for them, and a dash or raster call that needs them asks again
+  if (n_rib) ps_ensure_quad_hits(ctx, n_rib);
   return PS_OK;
 }
 

@@ -96,6 +96,22 @@ int main() {
 """
 
 
+TESSELLATE_ONLY = MAIN + r"""
+int main() {
+  ps_context* c = nullptr;
+  CHECK(ps_create(&c) == PS_OK);
+  most = 100000000;  // the tile states of 50 M ribs, but not 9 bytes for each
+  CHECK(ps_reserve(c, 1000, 50000000, 1000, 1000) == PS_OK);
+  consistent(c);
+  CHECK(c->tile_cap > 50000000 / 512 && c->pair_cap >= 1000 && c->rec_cap >= 1000 && c->quad_hits_cap == 0);
+  CHECK(ps_reserve(c, 0, 5000000, 0, 0) == PS_OK);
+  consistent(c);
+  CHECK(c->quad_hits_cap >= 5000000);
+  ps_destroy(c);
+  return errors ? 1 : 0;
+}
+"""
+
 CAPTURED = MAIN + r"""
 int main() {
   ps_context* c = nullptr;
@@ -160,3 +176,7 @@ def test_failed_growth_leaves_nothing_claimed(tmp_path):
 
 def test_captured_blocks_are_kept(tmp_path):
     run(tmp_path, CAPTURED)
+
+
+def test_reservation_without_room_for_the_words(tmp_path):
+    run(tmp_path, TESSELLATE_ONLY)
