@@ -514,8 +514,19 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
   int rc = ps_ensure_tiles(ctx, n_tiles + 1);
   if (rc != PS_OK) return rc;
   cudaMemsetAsync(ctx->d_counters, 0, 64 + sizeof(TileState) * (n_tiles + 1), st);
-  if ((rc = ps_ensure_quad_hits(ctx, capacity)) != PS_OK) return rc;  // 8 bytes per quad
-  unsigned long long* word = reinterpret_cast<unsigned long long*>(ctx->d_quad_hits);
+  // A word of 8 bytes per quad: the context's, or under a capture that finds too few there,
+  // the graph's own (a capture allows no cudaMalloc, and before the words a dash needed none).
+  unsigned long long* word = nullptr;
+  bool graph_word = false;
+  if (capacity > ctx->quad_hits_cap) {
+    cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+    graph_word = cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusActive;
+  }
+  if (graph_word)
+    rc = ps_cuda_check(cudaMallocAsync((void**)&word, sizeof(*word) * (size_t)capacity, st));
+  else if ((rc = ps_ensure_quad_hits(ctx, capacity)) == PS_OK)
+    word = reinterpret_cast<unsigned long long*>(ctx->d_quad_hits);
+  if (rc != PS_OK) return rc;
   const DashOut D{reinterpret_cast<float4*>(d_out_rib), d_out_s, d_out_tag, d_out_src, out_capacity};
   const int grid0 =
       ps_grid_for(ps_persistent_grid(ctx, (const void*)k_dash_count, DASH_NT, 0), capacity, DASH_TILE);
@@ -548,7 +559,9 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
                   d_tag, d_n_rib, capacity, P, word, D, tasks, ctx->d_counters, ctx->d_status);
   if (tasks)
     ps_launch_after(true, &k_dash_caps, grid2, DASH_NT, 0, st, tasks, P.j_round, D, ctx->d_counters);
-  return ps_cuda_check(cudaGetLastError());
+  rc = ps_cuda_check(cudaGetLastError());
+  if (graph_word && cudaFreeAsync(word, st) != cudaSuccess && rc == PS_OK) rc = PS_ERR_CUDA;
+  return rc;
 }
 
 extern "C" int ps_dash(ps_context* ctx, const float* d_rib, const float* d_s,
