@@ -10,6 +10,10 @@
 
 #include <cmath>
 
+#if defined(PS_HD) && !defined(PS_DF_ROUNDED)
+#error "ps_dash_walk.cuh comes before ps_df.cuh: its bounds need rounded operations"
+#endif
+#define PS_DF_ROUNDED
 #include "ps_df.cuh"
 
 namespace ps {
@@ -95,7 +99,9 @@ inline bool dash_pattern(DashPattern& P, const float* h_pattern, int n_pattern, 
 // product's FMA residual and the period's low part.  What remains for k < 2^24
 // is five roundings of values below two periods, at most 2^-24 of the period
 // each (twice that above one period), the pattern's own FP32 rounding (2^-24) and the
-// period's tail (2^-25): under 1e-6 of the period in all.  The FP64 rule's own
+// period's tail (2^-25): under 1e-6 of the period in all.  (Each operation is rounded by
+// itself, rn_*: with k period_f fused into the difference its residual would count twice,
+// k 2^-24 of a period.)  The FP64 rule's own
 // roundings are below 2^-27 of it.  eps is 4e-6 of the period, so that few
 // quads besides those that cross a boundary are left to the walk.
 // 1: inside an on-stretch (the quad is emitted whole), 0: inside a gap
@@ -103,16 +109,14 @@ inline bool dash_pattern(DashPattern& P, const float* h_pattern, int n_pattern, 
 PS_HD int dash_quick(const DashPattern& P, float sa, float sb) {
   const float per = P.period_f;
   const float eps = 4e-6f * per;
-  const float u = sa + P.offset_f;  // TwoSum: u + ul == sa + offset exactly
-  const float bv = u - sa;
-  const float ul = (sa - (u - bv)) + (P.offset_f - bv);
-  const float k = floorf(u / per);
+  const DF u = two_sum(sa, P.offset_f);
+  const float k = floorf(u.hi / per);
   if (!(fabsf(k) < 16777216.f)) return -1;
-  const float kp = k * per;
-  const float ke = fmaf(k, per, -kp);  // k per == kp + ke exactly
-  const float ph = (((u - kp) + ul) - ke) - k * P.period_lo;  // phase of sa
+  const DF kp = two_prod(k, per);
+  // phase of sa
+  const float ph = rn_sub(rn_sub(rn_add(rn_sub(u.hi, kp.hi), u.lo), kp.lo), rn_mul(k, P.period_lo));
   if (!(ph >= 0.f && ph < per)) return -1;
-  const float pe = ph + (sb - sa);  // phase of sb, beyond the period if it wraps
+  const float pe = rn_add(ph, rn_sub(sb, sa));  // phase of sb, beyond the period if it wraps
   int j = 0;  // interval [cum_f[j], cum_f[j+1]) holding ph
   while (j + 1 < P.m2 && P.cum_f[j + 1] <= ph) ++j;
   if (ph - P.cum_f[j] > eps && P.cum_f[j + 1] - pe > eps) return (j & 1) ? 0 : 1;
@@ -175,7 +179,8 @@ struct DashWalk {
 // quarter pixels, say) and the magnitude is below 2^40 g: then k period, the sums
 // and the differences are exact in pairs and in FP64, and equality is decided
 // too (at large s a quad often begins exactly at a stretch end, as s itself lies
-// on a coarse FP32 grid).  FP64 operations have a long latency here, and a tile
+// on a coarse FP32 grid).  Every operation is rounded by itself or an explicit fmaf,
+// so that the counting and the writing pass walk a quad alike.  FP64 operations have a long latency here, and a tile
 // waits for its slowest quad before it can publish its output count: with
 // every queued quad in FP64 the kernel took 141 us on the 5,031-cubic path and
 // 1,097 us on 1,000 paths with capped dashes, and 125 and 784 us this way.
@@ -186,15 +191,15 @@ struct DashWalkDF {
   PS_HD void start(const DashPattern& P, float sa_f, float sb_f) {
     sa = sa_f;
     sb = sb_f;
-    const float u = sa + P.offset_f;
+    const float u = rn_add(sa, P.offset_f);
     // the period that holds sa, or the one before where FP32 does not tell them apart
     k0 = floorf(u / P.period_f);
-    if (!(fmaf(-k0, P.period_f, u) > 4e-6f * P.period_f + 4e-7f * fabsf(u))) k0 -= 1.f;
-    const float n = (sb - sa) / P.period_f;
+    if (!(fmaf(-k0, P.period_f, u) > fmaf(4e-6f, P.period_f, rn_mul(4e-7f, fabsf(u))))) k0 -= 1.f;
+    const float n = rn_sub(sb, sa) / P.period_f;
     // (false for NaN; a period near FP32's range end has no exact products)
     sure = fabsf(k0) < 4194304.f && n < 1024.f && P.period_f > 1e-20f;
-    const float mag = (fabsf(k0) + fabsf(n) + 4.f) * P.period_f + fabsf(P.offset_f);
-    err = mag < P.exact_below ? 0.f : 2.8421709e-14f * mag;
+    const float mag = fmaf(fabsf(k0) + fabsf(n) + 4.f, P.period_f, fabsf(P.offset_f));
+    err = mag < P.exact_below ? 0.f : rn_mul(2.8421709e-14f, mag);
     g = 0;
     i = 0;
   }
@@ -212,14 +217,14 @@ struct DashWalkDF {
       const float k = k0 + (float)g;
       const DF kp = two_prod(k, P.period_f);
       const DF base = df_add_f(
-          fast_two_sum(kp.hi, kp.lo + k * P.period_lo), -P.offset_f);
+          fast_two_sum(kp.hi, fmaf(k, P.period_lo, kp.lo)), -P.offset_f);
       if (cmp(base, sb) > 0) return false;
       while (i < P.m2 && sure) {
         const DF c0{P.cum_f[i], P.cum_l[i]}, c1{P.cum_f[i + 1], P.cum_l[i + 1]};
         const bool empty = (P.empty >> (i >> 1)) & 1u;
         i += 2;
         if (empty) continue;
-        if (!((c1.hi - c0.hi) + (c1.lo - c0.lo) > 2.f * err)) sure = false;
+        if (!(rn_add(rn_sub(c1.hi, c0.hi), rn_sub(c1.lo, c0.lo)) > 2.f * err)) sure = false;
         b = df_add(base, c1);
         if (cmp(b, sa) <= 0) continue;
         a = df_add(base, c0);
@@ -249,7 +254,8 @@ struct DashWalkDF {
 PS_HD float cut_coord(float a0, float a1, DF f, float fe, bool& ok) {
   const DF dv = df_diff(a1, a0);  // exact
   const DF v = df_add_f(df_mul(f, dv), a0);
-  const float e = fmaf(fe + 5.6843419e-14f, fabsf(dv.hi), 5.6843419e-14f * (fabsf(a0) + fabsf(a1)));
+  const float e = fmaf(fe + 5.6843419e-14f, fabsf(dv.hi),
+                       rn_mul(5.6843419e-14f, fabsf(a0) + fabsf(a1)));
   ok &= v.hi + (v.lo + e) == v.hi && v.hi + (v.lo - e) == v.hi;
   return v.hi;
 }

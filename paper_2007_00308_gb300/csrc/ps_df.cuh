@@ -41,8 +41,24 @@ struct DF2 {
   DF x, y;
 };
 
+// The operations of the scalar pairs.  From plain operators a compiler may fuse a product into
+// the sum that it goes into, and its rounding error is then counted twice.  Where results rest on
+// error bounds, PS_DF_ROUNDED (defined before this header) has each rounded by itself; the
+// tessellation, which is checked against 64 bits instead, keeps the operators (rounded by
+// themselves they cost the rib kernel registers: 10,417 -> 10,539 us on a million near-cusp
+// cubics).
+#if defined(PS_DF_ROUNDED) && defined(__CUDA_ARCH__)
+PS_HD float rn_mul(float a, float b) { return __fmul_rn(a, b); }
+PS_HD float rn_add(float a, float b) { return __fadd_rn(a, b); }
+PS_HD float rn_sub(float a, float b) { return __fsub_rn(a, b); }
+#else
+PS_HD float rn_mul(float a, float b) { return a * b; }
+PS_HD float rn_add(float a, float b) { return a + b; }
+PS_HD float rn_sub(float a, float b) { return a - b; }
+#endif
+
 PS_HD DF df_of(float a) { return DF{a, 0.f}; }
-PS_HD float df_f(DF a) { return a.hi + a.lo; }
+PS_HD float df_f(DF a) { return rn_add(a.hi, a.lo); }
 PS_HD double df_d(DF a) { return (double)a.hi + (double)a.lo; }
 PS_HD DF df_from_d(double v) {
   float h = (float)v;
@@ -51,36 +67,36 @@ PS_HD DF df_from_d(double v) {
 
 // |a| >= |b| (or a == 0): s + e == a + b exactly
 PS_HD DF fast_two_sum(float a, float b) {
-  float s = a + b;
-  return DF{s, b - (s - a)};
+  float s = rn_add(a, b);
+  return DF{s, rn_sub(b, rn_sub(s, a))};
 }
 PS_HD DF two_sum(float a, float b) {
-  float s = a + b;
-  float bb = s - a;
-  return DF{s, (a - (s - bb)) + (b - bb)};
+  float s = rn_add(a, b);
+  float bb = rn_sub(s, a);
+  return DF{s, rn_add(rn_sub(a, rn_sub(s, bb)), rn_sub(b, bb))};
 }
 PS_HD DF two_prod(float a, float b) {
-  float p = a * b;
+  float p = rn_mul(a, b);
   return DF{p, fmaf(a, b, -p)};
 }
 PS_HD DF df_neg(DF a) { return DF{-a.hi, -a.lo}; }
 PS_HD DF df_add(DF a, DF b) {
   DF s = two_sum(a.hi, b.hi);
-  return fast_two_sum(s.hi, s.lo + (a.lo + b.lo));
+  return fast_two_sum(s.hi, rn_add(s.lo, rn_add(a.lo, b.lo)));
 }
 PS_HD DF df_sub(DF a, DF b) { return df_add(a, df_neg(b)); }
 PS_HD DF df_add_f(DF a, float b) {
   DF s = two_sum(a.hi, b);
-  return fast_two_sum(s.hi, s.lo + a.lo);
+  return fast_two_sum(s.hi, rn_add(s.lo, a.lo));
 }
 PS_HD DF df_mul(DF a, DF b) {
-  float p = a.hi * b.hi;
+  float p = rn_mul(a.hi, b.hi);
   float e = fmaf(a.hi, b.hi, -p);
   e = fmaf(a.hi, b.lo, fmaf(a.lo, b.hi, e));
   return fast_two_sum(p, e);
 }
 PS_HD DF df_mul_f(DF a, float b) {
-  float p = a.hi * b;
+  float p = rn_mul(a.hi, b);
   float e = fmaf(a.hi, b, -p);
   e = fmaf(a.lo, b, e);
   return fast_two_sum(p, e);
@@ -121,18 +137,16 @@ struct Acc {
 };
 // A += x y (x, y pairs)
 PS_HD void acc_prod(Acc& A, DF x, DF y) {
-  const float p = x.hi * y.hi;
-  const float pe = fmaf(x.hi, y.hi, -p);
-  const float s = A.s + p;
-  const float bb = s - A.s;
-  A.e += ((A.s - (s - bb)) + (p - bb)) + (pe + fmaf(x.hi, y.lo, x.lo * y.hi));
-  A.s = s;
+  const DF p = two_prod(x.hi, y.hi);
+  const DF t = two_sum(A.s, p.hi);
+  A.e = rn_add(A.e, rn_add(t.lo, rn_add(p.lo, fmaf(x.hi, y.lo, rn_mul(x.lo, y.hi)))));
+  A.s = t.hi;
 }
 PS_HD Acc acc_first(DF x, DF y) {
-  const float p = x.hi * y.hi;
-  return Acc{p, fmaf(x.hi, y.hi, -p) + fmaf(x.hi, y.lo, x.lo * y.hi)};
+  const DF p = two_prod(x.hi, y.hi);
+  return Acc{p.hi, rn_add(p.lo, fmaf(x.hi, y.lo, rn_mul(x.lo, y.hi)))};
 }
-PS_HD float acc_round(Acc A) { return A.s + A.e; }
+PS_HD float acc_round(Acc A) { return rn_add(A.s, A.e); }
 
 // Two pairs side by side, x and y of a point or sine and cosine of an angle: each operation is
 // the scalar one above on both, one packed FP32 instruction (two lanes, each rounded as
