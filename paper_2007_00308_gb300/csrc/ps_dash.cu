@@ -16,6 +16,8 @@
 // stretch's first piece or after its last.
 #include <cuda_runtime.h>
 
+#include <algorithm>
+
 #include "ps_dash_walk.cuh"
 #include "ps_internal.cuh"
 
@@ -315,7 +317,7 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
     const float4* __restrict__ rib, const float* __restrict__ s, const uint32_t* __restrict__ tag,
     const int64_t* __restrict__ n_rib, int64_t capacity, const __grid_constant__ DashPattern P,
     const unsigned long long* __restrict__ word, const __grid_constant__ DashOut D,
-    CapTask* __restrict__ tasks, int32_t* counters, int32_t* status) {
+    CapTask* __restrict__ tasks, int max_tasks, int32_t* counters, int32_t* status) {
   __shared__ uint8_t s_queue[DASH_NT / 32][EMIT_WQ];  // a warp's queued quads
   dep_wait(word);
   int64_t R = *n_rib;
@@ -446,7 +448,9 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
             int at = 0;
             if (lane == lead) at = atomicAdd(&counters[8], __popc(sm));
             at = __shfl_sync(0xffffffffu, at, lead) + __popc(sm & ((1u << lane) - 1u));
-            if (shared) tasks[at] = CapTask{C, tq, sv, (int32_t)r, 0, oc};
+            // (the list holds a cap for every j_round + 1 output ribs; more come up only when
+            // a look-back gave up and output ranges overlap: PS_ERR_TIMEOUT is recorded)
+            if (shared && at < max_tasks) tasks[at] = CapTask{C, tq, sv, (int32_t)r, 0, oc};
             continue;
           }
           for (unsigned m = sm; m; m &= m - 1u) {
@@ -469,11 +473,12 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
 }
 
 // Round caps, a warp to each.
-__global__ void __launch_bounds__(DASH_NT) k_dash_caps(const CapTask* __restrict__ tasks, int J,
+__global__ void __launch_bounds__(DASH_NT) k_dash_caps(const CapTask* __restrict__ tasks,
+                                                       int max_tasks, int J,
                                                        const __grid_constant__ DashOut D,
                                                        const int32_t* __restrict__ counters) {
   dep_wait(tasks, counters);
-  const int n = counters[8], lane = threadIdx.x & 31;
+  const int n = min(counters[8], max_tasks), lane = threadIdx.x & 31;
   const int stride = gridDim.x * (DASH_NT / 32);
   for (int i = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; i < n; i += stride) {
     const CapTask T = tasks[i];
@@ -536,8 +541,9 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
   // memory, or a capture under way and no room from an earlier call) the writing
   // pass writes them itself.
   CapTask* tasks = nullptr;
+  const int max_tasks = (int)std::min<int64_t>(out_capacity / (P.j_round + 1) + 1, INT32_MAX);
   if (P.path_cap && P.j_round > 4) {
-    const size_t need = sizeof(CapTask) * (size_t)(out_capacity / (P.j_round + 1) + 1);
+    const size_t need = sizeof(CapTask) * (size_t)max_tasks;
     if (need > ctx->cap_bytes) {
       cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
       if (cudaStreamIsCapturing(st, &cs) == cudaSuccess && cs == cudaStreamCaptureStatusNone) {
@@ -549,16 +555,17 @@ extern "C" int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* 
     if (need <= ctx->cap_bytes) tasks = static_cast<CapTask*>(ctx->d_cap_tasks);
   }
   const int grid2 = ps_grid_for(ps_persistent_grid(ctx, (const void*)k_dash_caps, DASH_NT, 0),
-                                out_capacity / (P.j_round + 1) + 1, 1);
+                                max_tasks, 1);
   ProfScope ps_(ctx, PK_DASH, st);
   k_dash_count<<<grid0, DASH_NT, 0, st>>>(d_s, d_tag, d_n_rib, capacity, P, word, d_n_out,
                                                     out_capacity, ctx->d_tile_state, ctx->d_counters,
                                                     ctx->d_status);
   // (one profile slot for all three: no event records in between)
   ps_launch_after(true, &k_dash, grid1, DASH_NT, 0, st, reinterpret_cast<const float4*>(d_rib), d_s,
-                  d_tag, d_n_rib, capacity, P, word, D, tasks, ctx->d_counters, ctx->d_status);
+                  d_tag, d_n_rib, capacity, P, word, D, tasks, max_tasks, ctx->d_counters, ctx->d_status);
   if (tasks)
-    ps_launch_after(true, &k_dash_caps, grid2, DASH_NT, 0, st, tasks, P.j_round, D, ctx->d_counters);
+    ps_launch_after(true, &k_dash_caps, grid2, DASH_NT, 0, st, tasks, max_tasks, P.j_round, D,
+                    ctx->d_counters);
   rc = ps_cuda_check(cudaGetLastError());
   if (graph_word && cudaFreeAsync(word, st) != cudaSuccess && rc == PS_OK) rc = PS_ERR_CUDA;
   return rc;
