@@ -9,10 +9,16 @@ from . import (PS_PREC_MIXED, Context, DeviceBatch, _backward_records, _tessella
                ps_tessellate_backward, tessellate)
 
 
+def _in_memory(grad, like):
+    """Whether the tensor's memory holds its values as ``like``'s would."""
+    return (grad.layout == torch.strided and grad.dtype == like.dtype and grad.device == like.device
+            and not grad.is_neg() and not grad._is_zerotensor())
+
+
 def _upstream(grad, like, n):
     """The gradient of the first n rows of ``like`` as the adjoint reads it: dense,
     16-byte aligned, as long as ``like``."""
-    if grad is not None and n == like.shape[0]:
+    if grad is not None and n == like.shape[0] and _in_memory(grad, like):
         grad = grad.contiguous()
         return grad if grad.data_ptr() % 16 == 0 else grad.clone()
     full = torch.zeros(like.shape, dtype=torch.float32, device=like.device)
