@@ -491,8 +491,12 @@ def _tessellate_exact(ctx: Context, db: DeviceBatch, precision, arclength=True, 
     import torch
     out = TessOutput(db.n_link, db.n_path, 0, arclength=arclength)
     records = torch.empty(lib().ps_record_bytes(db.n_link), dtype=torch.uint8, device="cuda")
-    if stream is not None:  # freed, or used by the adjoint, after work on that stream
-        records.record_stream(stream)
+    if stream is not None:
+        # the buffers come from the current stream's pool, where earlier work may still use them
+        on = (stream if isinstance(stream, torch.cuda.Stream)
+              else torch.cuda.ExternalStream(stream.cuda_stream))
+        on.wait_stream(torch.cuda.current_stream())
+        records.record_stream(on)  # given back only after the work on that stream
     seg, paths = db._structs()
     o = out._struct()
     n = ctypes.c_int64(0)
