@@ -436,7 +436,8 @@ int ps_route_quads(ps_context* ctx, const float* d_rib, const uint32_t* d_tag,
  * With profiling enabled the library records a CUDA event pair around each of its
  * kernel launches on the launching stream (as external event-record nodes when
  * the stream is being captured into a graph, so graph replays are timed too).
- * Slot s names one kernel (ps_profile_slot_name).  ps_profile_read waits for the
+ * Slot s names one kernel (ps_profile_slot_name; an empty name: none, the slot
+ * is never recorded).  ps_profile_read waits for the
  * events and returns, per slot, the duration in ms of the most recent launch,
  * or -1 if the slot has not been recorded since profiling was enabled. */
 #define PS_PROF_SLOTS 10

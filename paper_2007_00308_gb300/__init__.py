@@ -502,12 +502,12 @@ def _tessellate_exact(ctx: Context, db: DeviceBatch, precision, arclength=True, 
     n = ctypes.c_int64(0)
     _check(lib().ps_link_records_sync(ctx.handle, ctypes.byref(seg), ctypes.byref(paths), db.dtheta,
                                       int(precision), ctypes.byref(o), _ptr(records),
-                                      _stream(stream), ctypes.byref(n)), "ps_count_ribs_sync")
+                                      _stream(stream), ctypes.byref(n)), "ps_link_records_sync")
     out._allocate(max(n.value, 1), arclength, want_t, "cuda")
     o = out._struct()
     _check(lib().ps_emit_records(ctx.handle, ctypes.byref(seg), ctypes.byref(paths), int(precision),
                                  PS_TESS_ARCLENGTH if arclength else 0, ctypes.byref(o),
-                                 _ptr(records), _stream(stream)), "ps_tessellate_strokes")
+                                 _ptr(records), _stream(stream)), "ps_emit_records")
     return out, records, n.value
 
 
@@ -519,7 +519,7 @@ def _backward_records(ctx: Context, db: DeviceBatch, fwd: TessOutput, records, g
     _check(lib().ps_backward_records(ctx.handle, ctypes.byref(seg), ctypes.byref(paths),
                                      int(precision), ctypes.byref(o), _ptr(records),
                                      _ptr(grad_rib), _ptr(grad_s), _ptr(grad_pts),
-                                     _ptr(grad_width), _stream(None)), "ps_tessellate_backward")
+                                     _ptr(grad_width), _stream(None)), "ps_backward_records")
 
 
 def tessellate(ctx: Context, db: DeviceBatch, precision=PS_PREC_FP32, arclength=True,

@@ -296,7 +296,7 @@ extern "C" int ps_profile_read(ps_context* ctx, float* h_ms) {
 }
 
 extern "C" const char* ps_profile_slot_name(int slot) {
-  static const char* names[PK_COUNT] = {"k_link_path", "k_link_setup", "k_emit", "k_arclen_scan",
+  static const char* names[PK_COUNT] = {"", "k_link_setup", "k_emit", "k_arclen_scan",
                                         "k_midpoint_chords", "k_bin_count", "k_tile_scan",
                                         "k_bin_scatter", "k_coverage", "k_dash"};
   return (slot >= 0 && slot < PK_COUNT) ? names[slot] : "";

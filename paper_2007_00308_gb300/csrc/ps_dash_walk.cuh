@@ -180,9 +180,9 @@ struct DashWalk {
 // and the differences are exact in pairs and in FP64, and equality is decided
 // too (at large s a quad often begins exactly at a stretch end, as s itself lies
 // on a coarse FP32 grid).  Every operation is rounded by itself or an explicit fmaf,
-// so that the counting and the writing pass walk a quad alike.  FP64 operations have a long latency here, and a tile
-// waits for its slowest quad before it can publish its output count: with
-// every queued quad in FP64 the kernel took 141 us on the 5,031-cubic path and
+// so that the counting and the writing pass walk a quad alike.  FP64 operations have a
+// long latency here, and a tile waits for its slowest quad before it can publish its
+// output count: with every queued quad in FP64 the kernel took 141 us on the 5,031-cubic path and
 // 1,097 us on 1,000 paths with capped dashes, and 125 and 784 us this way.
 struct DashWalkDF {
   float sa, sb, k0, err;

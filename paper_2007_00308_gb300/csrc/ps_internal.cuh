@@ -55,9 +55,9 @@ static_assert(sizeof(LinkRec) == 240, "LinkRec layout");
 #define META_SPLIT_BIT(k) (1u << (21 + (k)))
 #define META_SPLIT(m, k) (((m) >> (21 + (k))) & 1u)
 
-// Profiling slots (one per kernel).
+// Profiling slots (one per kernel; the first has lost its own).
 enum {
-  PK_LINK_PATH = 0, PK_LINK_SETUP, PK_EMIT, PK_ARCLEN, PK_MIDCHORD, PK_BIN_COUNT, PK_TILE_SCAN,
+  PK_UNUSED = 0, PK_LINK_SETUP, PK_EMIT, PK_ARCLEN, PK_MIDCHORD, PK_BIN_COUNT, PK_TILE_SCAN,
   PK_BIN_SCATTER, PK_COVERAGE, PK_DASH, PK_COUNT
 };
 static_assert(PK_COUNT == PS_PROF_SLOTS, "profile slots");

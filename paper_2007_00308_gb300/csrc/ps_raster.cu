@@ -7,6 +7,8 @@
 // over paths and covered[p] sums path p's masks' popcounts.
 #include <cuda_runtime.h>
 
+#include <type_traits>
+
 #include "ps_internal.cuh"
 
 namespace {
@@ -191,6 +193,7 @@ struct RasterClear {
   int32_t* counters;           // 16
   unsigned long long* stats;  // 7
 };
+struct NoClear {};  // the scatter pass has nothing to clear
 __device__ __forceinline__ void raster_clear(const RasterClear& C) {
   const int64_t i0 = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   const int64_t n = (int64_t)gridDim.x * blockDim.x;
@@ -221,7 +224,8 @@ __global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 6) k_bin(const float4*
                                                 uint32_t* __restrict__ bin, int64_t pair_cap,
                                                 uint2* __restrict__ hits,
                                                 int32_t* __restrict__ back,  // short fill, from the end
-                                                RasterClear clear, int32_t* status) {
+                                                std::conditional_t<PASS == 0, RasterClear, NoClear> clear,
+                                                int32_t* status) {
   __shared__ BinQuad s_q[BIN_NT];
   __shared__ int s_pre[BIN_NT / 32][33];
   if (PASS == 1) dep_wait(off, hits);
@@ -229,7 +233,7 @@ __global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 6) k_bin(const float4*
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   BinQuad* wq = s_q + wid * 32;
-  if (PASS == 0) raster_clear(clear);
+  if constexpr (PASS == 0) raster_clear(clear);
   int64_t stride = (int64_t)gridDim.x * BIN_NT;
   for (int64_t base = (int64_t)blockIdx.x * BIN_NT; base < R; base += stride) {
     const int64_t r = base + threadIdx.x;
@@ -1714,8 +1718,7 @@ static int rasterize(ps_context* ctx, const float* d_rib, const uint32_t* d_tag,
                           ctx->d_tile_state, ts_grid + 1, ctx->d_counters,
                           reinterpret_cast<unsigned long long*>(ctx->d_scratch64)};
   // persistent grids, each pass at its own occupancy (the count pass holds more
-  // registers)
-  // (the count pass has the canvas to clear as well)
+  // registers, and has the canvas to clear as well)
   int grid_bin = ctx->tune[PS_TUNE_BIN_BLOCKS] > 0
                      ? ctx->num_sms * ctx->tune[PS_TUNE_BIN_BLOCKS]
                      : ps_grid_for(ps_persistent_grid(ctx, (const void*)k_bin<0>, BIN_NT, 0),
@@ -1728,8 +1731,9 @@ static int rasterize(ps_context* ctx, const float* d_rib, const uint32_t* d_tag,
   { ProfScope ps_(ctx, PK_BIN_COUNT, st);
   k_bin<0><<<grid_bin, BIN_NT, 0, st>>>(rib, d_tag, d_n_rib, capacity, width, height, y0, tiles_x,
                                       ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,
-                                      ctx->d_bin, ctx->pair_cap, reinterpret_cast<uint2*>(ctx->d_quad_hits), ctx->d_tile_cursor + n_tile + 1,
-                                      clear, ctx->d_status); }
+                                      ctx->d_bin, ctx->pair_cap,
+                                      reinterpret_cast<uint2*>(ctx->d_quad_hits),
+                                      ctx->d_tile_cursor + n_tile + 1, clear, ctx->d_status); }
   const bool overlap = !ctx->prof_on;
   { ProfScope ps_(ctx, PK_TILE_SCAN, st);
   ps_launch_after(overlap, &k_tile_scan, ts_grid, TS_NT, 0, st, ctx->d_tile_count, ctx->d_tile_off,
@@ -1739,7 +1743,7 @@ static int rasterize(ps_context* ctx, const float* d_rib, const uint32_t* d_tag,
   ps_launch_after(overlap, &k_bin<1>, grid_bin1, BIN_NT, 0, st, rib, d_tag, d_n_rib, capacity, width,
                   height, y0, tiles_x, ctx->d_tile_count, ctx->d_tile_off, ctx->d_tile_cursor,
                   ctx->d_bin, ctx->pair_cap, reinterpret_cast<uint2*>(ctx->d_quad_hits),
-                  ctx->d_tile_cursor + n_tile + 1, clear, ctx->d_status); }
+                  ctx->d_tile_cursor + n_tile + 1, NoClear{}, ctx->d_status); }
   { ProfScope ps_(ctx, PK_COVERAGE, st);
   ps_launch_after(overlap, exact ? &k_coverage<true> : &k_coverage<false>, grid_cov, CV_NT, cov_smem, st,
                   rib, d_tag, ctx->d_tile_off, ctx->d_bin, ctx->pair_cap, width, height, y0, tiles_x,

@@ -1233,8 +1233,9 @@ __global__ void __launch_bounds__(SETUP_NT, 2) k_link_setup(
     const uint8_t* __restrict__ join, const uint8_t* __restrict__ cap,
     const float* __restrict__ miter, const uint8_t* __restrict__ closed, int n_path,
     int64_t n_link, float q, float tau, LinkRec* __restrict__ recs, int32_t* __restrict__ link_path,
-    float* __restrict__ path_len, int32_t* __restrict__ link_off, int32_t* __restrict__ path_off, int64_t* __restrict__ n_rib_out, int64_t capacity,
-    TileState* state, int32_t* counters, int32_t* status, int64_t n_tiles, int64_t l_begin) {
+    float* __restrict__ path_len, int32_t* __restrict__ link_off, int32_t* __restrict__ path_off,
+    int64_t* __restrict__ n_rib_out, int64_t capacity, TileState* state, int32_t* counters,
+    int32_t* status, int64_t n_tiles, int64_t l_begin) {
   __shared__ long long sm[SETUP_NT / 32 + 1];
   __shared__ long long s_prefix;
   __shared__ int s_tile;
@@ -1884,8 +1885,8 @@ static int launch_tessellate(ps_context* ctx, const ps_segments* seg, const ps_p
     // the emitter wrote each rib's chord into s; the segmented scan turns them
     // into cumulative arc length in place
     ProfScope ps_(ctx, PK_ARCLEN, st);
-    launch_arclen_scan(ctx, 0, !ctx->prof_on, st, out->d_s, out->d_tag, out->d_n_rib, out->capacity, out->d_s,
-                       out->d_path_len, ctx->d_tile_state + n_tiles + 1, ctx->d_counters,
+    launch_arclen_scan(ctx, 0, !ctx->prof_on, st, out->d_s, out->d_tag, out->d_n_rib, out->capacity,
+                       out->d_s, out->d_path_len, ctx->d_tile_state + n_tiles + 1, ctx->d_counters,
                        ctx->d_status);
     if ((rc = ps_cuda_check(cudaGetLastError())) != PS_OK) return rc;
   }
