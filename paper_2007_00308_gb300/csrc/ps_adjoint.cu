@@ -491,9 +491,9 @@ __global__ void __launch_bounds__(256) k_adj_ribs(
 // Per link: boundary-angle adjoints -> control points.
 __global__ void k_adj_finalize(const LinkRec* __restrict__ recs, const int4* __restrict__ src,
                                int64_t n_link, const uint8_t* st, const float* sp, const float* sw,
-                               const float* __restrict__ adj_psi, float* __restrict__ gpts) {
+                               const float* adj_psi, float* __restrict__ gpts) {
   int64_t l = blockIdx.x * (int64_t)blockDim.x + threadIdx.x;
-  dep_wait(adj_psi);
+  dep_wait();
   if (l >= n_link) return;
   int4 sc = src[l];
   const LinkRec* L = recs + l;

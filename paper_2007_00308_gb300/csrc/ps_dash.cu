@@ -316,10 +316,10 @@ constexpr int EMIT_WQ = 256;  // quads per ticket of the writing pass
 __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
     const float4* __restrict__ rib, const float* __restrict__ s, const uint32_t* __restrict__ tag,
     const int64_t* __restrict__ n_rib, int64_t capacity, const __grid_constant__ DashPattern P,
-    const unsigned long long* __restrict__ word, const __grid_constant__ DashOut D,
+    const unsigned long long* word, const __grid_constant__ DashOut D,
     CapTask* __restrict__ tasks, int max_tasks, int32_t* counters, int32_t* status) {
   __shared__ uint8_t s_queue[DASH_NT / 32][EMIT_WQ];  // a warp's queued quads
-  dep_wait(word);
+  dep_wait();
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -473,11 +473,11 @@ __global__ void __launch_bounds__(DASH_NT, 3) k_dash(
 }
 
 // Round caps, a warp to each.
-__global__ void __launch_bounds__(DASH_NT) k_dash_caps(const CapTask* __restrict__ tasks,
+__global__ void __launch_bounds__(DASH_NT) k_dash_caps(const CapTask* tasks,
                                                        int max_tasks, int J,
                                                        const __grid_constant__ DashOut D,
-                                                       const int32_t* __restrict__ counters) {
-  dep_wait(tasks, counters);
+                                                       const int32_t* counters) {
+  dep_wait();
   const int n = min(counters[8], max_tasks), lane = threadIdx.x & 31;
   const int stride = gridDim.x * (DASH_NT / 32);
   for (int i = (threadIdx.x >> 5) * gridDim.x + blockIdx.x; i < n; i += stride) {

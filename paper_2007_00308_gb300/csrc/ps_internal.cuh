@@ -272,22 +272,10 @@ __device__ __forceinline__ int64_t find_link_warp(const int32_t* off, int64_t n,
 // never done before the ones it follows.  One curve on a small canvas: 61 -> 49 us; 64
 // cubics: 97 -> 84; 300 paths: 648 -> 606.  (Letting the next kernel in before a kernel's
 // CTAs are done, by launch_dependents at its start, won nothing more: 53, 86 and 606 us.)
-//   The arguments are the pointers to what the kernels before wrote.  They come out of the
-// wait as new values, so that every load through them depends on it: a memory clobber alone
-// does not hold back loads of data that the kernel is told is read-only (const __restrict__,
-// __ldg), which this is not while the writer still runs.  For the same reason it is read with
-// ordinary loads.
-template <class P>
-__device__ __forceinline__ void after_wait(P& written) {
-  size_t a = __cvta_generic_to_global((const void*)written);
-  asm volatile("" : "+l"(a) : : "memory");
-  written = (P)__cvta_global_to_generic(a);
-}
-template <class... P>
-__device__ __forceinline__ void dep_wait(P&... written) {
-  asm volatile("griddepcontrol.wait;" ::: "memory");
-  (after_wait(written), ...);
-}
+//   What the kernels before wrote is read through plain pointers, without __restrict__ or
+// __ldg: those say that nobody writes the data while the kernel runs, which is not so before
+// the wait, and the wait's memory clobber does not hold back loads of such data.
+__device__ __forceinline__ void dep_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 
 // Launch of a kernel right after another of the call; overlap = false (event records in
 // between, or anything but a kernel before it): an ordinary launch.

@@ -219,16 +219,16 @@ __global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 6) k_bin(const float4*
                                                 const int64_t* __restrict__ n_rib, int64_t capacity,
                                                 int W, int H, int y0, int tiles_x,
                                                 int32_t* __restrict__ count,
-                                                const int32_t* __restrict__ off,
+                                                const int32_t* off,
                                                 int32_t* __restrict__ cursor,
                                                 uint32_t* __restrict__ bin, int64_t pair_cap,
-                                                uint2* __restrict__ hits,
+                                                uint2* hits,
                                                 int32_t* __restrict__ back,  // short fill, from the end
                                                 std::conditional_t<PASS == 0, RasterClear, NoClear> clear,
                                                 int32_t* status) {
   __shared__ BinQuad s_q[BIN_NT];
   __shared__ int s_pre[BIN_NT / 32][33];
-  if (PASS == 1) dep_wait(off, hits);
+  if (PASS == 1) dep_wait();
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
@@ -340,12 +340,13 @@ __global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 6) k_bin(const float4*
           if (PASS == 0) {
             if (lane == leader) atomicAdd(count + td, __popc(peers));
           } else {
+            const int o0 = off[td], o1 = off[td + 1];  // (read beside the atomic, not after it)
             int basepos = 0;
             if (lane == leader) basepos = atomicAdd((tall ? cursor : back) + td, __popc(peers));
             basepos = __shfl_sync(peers, basepos, leader);
             const int rk = basepos + __popc(peers & ((1u << lane) - 1u));
-            const int64_t at = tall ? (int64_t)off[td] + rk : (int64_t)off[td + 1] - 1 - rk;
-            if (at < pair_cap && at >= off[td] && at < off[td + 1]) bin[at] = (uint32_t)r;
+            const int64_t at = tall ? (int64_t)o0 + rk : (int64_t)o1 - 1 - rk;
+            if (at < pair_cap && at >= o0 && at < o1) bin[at] = (uint32_t)r;
             else ps_record_error(status, PS_ERR_CAPACITY);
           }
         }
@@ -407,12 +408,13 @@ __global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 6) k_bin(const float4*
         if (PASS == 0) {
           if (lane == leader) atomicAdd(count + t, cntg);
         } else {
+          const int o0 = off[t], o1 = off[t + 1];
           int basepos = 0;
           if (lane == leader) basepos = atomicAdd((tl ? cursor : back) + t, cntg);
           basepos = __shfl_sync(peers, basepos, leader);
           int pos = basepos + __popc(peers & ((1u << lane) - 1u));
-          int64_t at = tl ? (int64_t)off[t] + pos : (int64_t)off[t + 1] - 1 - pos;
-          if (at < pair_cap && at >= off[t] && at < off[t + 1])
+          int64_t at = tl ? (int64_t)o0 + pos : (int64_t)o1 - 1 - pos;
+          if (at < pair_cap && at >= o0 && at < o1)
             bin[at] = (uint32_t)(base + wid * 32 + e);
           else ps_record_error(status, PS_ERR_CAPACITY);
         }
@@ -437,7 +439,7 @@ __global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 6) k_bin(const float4*
 // warp-wide decoupled look-back across CTAs.
 constexpr int TS_NT = 256, TS_IPT = 16, TS_TILE = TS_NT * TS_IPT;
 constexpr int TS_SHIFT = 38;
-__global__ void __launch_bounds__(TS_NT) k_tile_scan(const int32_t* __restrict__ count,
+__global__ void __launch_bounds__(TS_NT) k_tile_scan(const int32_t* count,
                                                      int32_t* __restrict__ off,
                                                      int32_t* __restrict__ cursor,
                                                      int32_t* __restrict__ list, int n_tile,
@@ -447,7 +449,7 @@ __global__ void __launch_bounds__(TS_NT) k_tile_scan(const int32_t* __restrict__
   __shared__ long long s_pre;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
   const long long i0 = (long long)blockIdx.x * TS_TILE + (long long)threadIdx.x * TS_IPT;
-  dep_wait(count);
+  dep_wait();
   int c[TS_IPT];
   if (i0 + TS_IPT <= n_tile) {
     const int4* cp = reinterpret_cast<const int4*>(count + i0);
@@ -1305,9 +1307,8 @@ __device__ __forceinline__ void cp_async_wait_all() { asm volatile("cp.async.wai
 template <bool EXACT>
 __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
     const float4* __restrict__ rib, const uint32_t* __restrict__ tag,
-    const int32_t* __restrict__ off, const uint32_t* __restrict__ bin, int64_t pair_cap, int W,
-    int H, int y0, int tiles_x, int n_tile, const int32_t* __restrict__ tile_list,
-    uint16_t* __restrict__ canvas,
+    const int32_t* off, const uint32_t* bin, int64_t pair_cap, int W, int H, int y0, int tiles_x,
+    int n_tile, const int32_t* tile_list, uint16_t* __restrict__ canvas,
     unsigned long long* __restrict__ covered, int n_path, int32_t* counters, int32_t* status,
     unsigned long long* __restrict__ stats) {
   extern __shared__ __align__(16) unsigned char smem[];
@@ -1328,7 +1329,7 @@ __global__ void __launch_bounds__(CV_NT, 2) k_coverage(
   __shared__ __align__(16) float4 s_pre_rib[CV_WARPS][2][32];
   __shared__ uint32_t s_pre_tag[CV_WARPS][32];
 
-  dep_wait(off, bin, tile_list);
+  dep_wait();
   const int n_list = tile_list[n_tile];  // tiles with entries (the canvas is cleared)
   if ((int)blockIdx.x >= n_list) return;  // the others' tickets reach every tile
   for (int i = threadIdx.x; i < SLOTS * MASK_WORDS; i += CV_NT) s_mask[i] = 0u;

@@ -1512,11 +1512,10 @@ __device__ __forceinline__ RibEval eval_rib(const LinkRec* L, int j) {
 
 template <bool MIXED>
 __global__ void __launch_bounds__(EMIT_NT, MIXED ? 2 : 3) k_emit(
-    const LinkRec* __restrict__ recs, const int32_t* __restrict__ link_off,
-    const int32_t* __restrict__ link_path, int64_t n_link, const int64_t* __restrict__ n_rib,
-    int64_t capacity, float4* __restrict__ rib, uint32_t* __restrict__ tag,
+    const LinkRec* recs, const int32_t* link_off, const int32_t* link_path, int64_t n_link,
+    const int64_t* n_rib, int64_t capacity, float4* __restrict__ rib, uint32_t* __restrict__ tag,
     float* __restrict__ chord, float* __restrict__ tout, int most_slabs, int32_t* status) {
-  dep_wait(recs, link_off, link_path, n_rib);
+  dep_wait();
   int64_t R = *n_rib;
   // Over a caller's records the set-up knew no capacity.  (Asked here in FP32 and at the end in
   // mixed precision: the other way round the question costs the loops registers, 0.6% on a million
@@ -1620,18 +1619,17 @@ constexpr int SCAN_TILE = SCAN_NT * SCAN_IPT;
 // tile sums are FP32 (relative error ~1e-6 of s); the carry between tiles,
 // which runs over a whole path, is a double-float pair from a warp-wide
 // look-back.
-// (Three CTAs per SM for the form without vectors, which the compiler gives up otherwise.)
 template <bool VEC>
-__global__ void __launch_bounds__(SCAN_NT, VEC ? 1 : 3) k_arclen_scan(
-    const float* chord_in, const uint32_t* __restrict__ tag, const int64_t* __restrict__ n_rib,
-    int64_t capacity, float* s_out, float* __restrict__ path_len, TileState* state,
+__global__ void __launch_bounds__(SCAN_NT, 3) k_arclen_scan(
+    const float* chord_in, const uint32_t* tag, const int64_t* n_rib, int64_t capacity,
+    float* s_out, float* __restrict__ path_len, TileState* state,
     int32_t* counters, int32_t* status) {
   __shared__ float sv[SCAN_NT / 32];
   __shared__ int sh[SCAN_NT / 32];
   __shared__ float s_carry[2];
   __shared__ int64_t s_tile;
   const int lane = threadIdx.x & 31, wid = threadIdx.x >> 5;
-  dep_wait(chord_in, tag, n_rib);
+  dep_wait();
   int64_t R = *n_rib;
   if (R > capacity) R = capacity;
   const int64_t n_tiles = (R + SCAN_TILE - 1) / SCAN_TILE;
@@ -1673,6 +1671,8 @@ __global__ void __launch_bounds__(SCAN_NT, VEC ? 1 : 3) k_arclen_scan(
     // path of the rib before this thread's first: the previous lane's last
     uint32_t prevp = __shfl_up_sync(0xffffffffu, pth[SCAN_IPT - 1], 1);
     if (lane == 0) prevp = (base > 0 && base <= R) ? tag[base - 1] >> 2 : 0xffffffffu;
+    // and the rib after its last, read here beside the tile's own
+    const uint32_t after = lane == 31 && base + SCAN_IPT < R ? tag[base + SCAN_IPT] >> 2 : 0xffffffffu;
     uint32_t hm = 0;  // bit i: rib base + i starts a path
     float acc = 0.f;
 #pragma unroll
@@ -1729,7 +1729,7 @@ __global__ void __launch_bounds__(SCAN_NT, VEC ? 1 : 3) k_arclen_scan(
     }
     // path of the rib after this thread's last: the next lane's first
     uint32_t nextp = __shfl_down_sync(0xffffffffu, pth[0], 1);
-    if (lane == 31) nextp = base + SCAN_IPT < R ? tag[base + SCAN_IPT] >> 2 : 0xffffffffu;
+    if (lane == 31) nextp = after;
     // ribs before this thread's first head continue the running total
     const DF tile_carry = (hprev || whead) ? DF{0.f, 0.f} : DF{s_carry[0], s_carry[1]};
     float run = hprev ? vprev : vprev + wcarry;
