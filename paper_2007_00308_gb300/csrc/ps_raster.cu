@@ -209,12 +209,13 @@ __device__ __forceinline__ void raster_clear(const RasterClear& C) {
   if (i0 < 7) C.stats[i0] = 0ull;
 }
 
-// Five and six CTAs per SM (48 and 40 registers): the passes wait for memory and atomics as much
-// as they issue (count 1,028 -> 909 us, scatter 815 -> 782 us on 43 M ribs, of which 60 us of the
-// count by int32 pixel ranges and by staging only the quads of three tiles and more; six and
-// eight CTAs spill: 963 and 813 us).
+// The count pass at five CTAs per SM (48 registers): it waits for memory and atomics as much as it
+// issues (1,028 -> 909 us on 43 M ribs, of which 60 us by int32 pixel ranges and by staging only the
+// quads of three tiles and more; on another such sheet 946 us against 972 without the bound; six
+// CTAs spill: 963).  The scatter pass has no bound and takes 48 registers: 761 us on the 43 M
+// ribs, 799 at six CTAs (40 registers).
 template <int PASS>
-__global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 6) k_bin(const float4* __restrict__ rib,
+__global__ void __launch_bounds__(BIN_NT, PASS == 0 ? 5 : 0) k_bin(const float4* __restrict__ rib,
                                                 const uint32_t* __restrict__ tag,
                                                 const int64_t* __restrict__ n_rib, int64_t capacity,
                                                 int W, int H, int y0, int tiles_x,
