@@ -323,7 +323,9 @@ int ps_arclength_scan(ps_context* ctx, const float* d_rib, const uint32_t* d_tag
  * quad (join, cap, cusp pivot) is kept whole iff its s is "on".
  * Outputs: d_out_rib[4 cap], d_out_s[cap], d_out_tag[cap], d_out_src[cap]
  * (index of the source quad's end rib, may be NULL), *d_n_out (device).  More
- * than out_capacity ribs records PS_ERR_CAPACITY. */
+ * than out_capacity ribs records PS_ERR_CAPACITY.  The context's workspace holds
+ * 9 bytes per rib of capacity for it (shared with the raster calls; captured
+ * without that room, the graph brings 8 bytes per rib of its own). */
 int ps_dash(ps_context* ctx, const float* d_rib, const float* d_s, const uint32_t* d_tag,
             const int64_t* d_n_rib, int64_t capacity, const float* h_pattern, int n_pattern,
             float offset, float* d_out_rib, float* d_out_s, uint32_t* d_out_tag,
@@ -340,7 +342,9 @@ int ps_dash(ps_context* ctx, const float* d_rib, const float* d_s, const uint32_
  * own (link-start tag on the first, segment bit clear) at the boundary's s,
  * written right before the stretch's first piece (start cap) or right after its
  * last piece (end cap).  Counts, offsets and errors as ps_dash; the output
- * count includes the cap ribs. */
+ * count includes the cap ribs.  Besides ps_dash's workspace the context holds 40
+ * bytes for every round cap that d_out_rib has room for, where it can be had: a
+ * call without it (captured first, say) is slower, and gives the same. */
 int ps_dash_capped(ps_context* ctx, const float* d_rib, const float* d_s, const uint32_t* d_tag,
                    const int64_t* d_n_rib, int64_t capacity, const float* h_pattern, int n_pattern,
                    float offset, const uint8_t* d_path_cap, int32_t n_path, float dtheta,

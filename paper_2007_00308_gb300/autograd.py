@@ -32,7 +32,9 @@ class PolarStroke(torch.autograd.Function):
     def forward(ctx, pts, width, batch, precision=PS_PREC_MIXED, psctx=None):
         """pts: float32 [S, 4, 2] on the GPU; width: float32 [P]; batch: the
         StrokeBatch giving types, weights, path structure, joins, caps and dtheta.
-        Returns rib [R, 4] (N.x N.y P.x P.y) and s [R]."""
+        Returns rib [R, 4] (N.x N.y P.x P.y) and s [R].  Until the backward pass the
+        graph holds the ribs and t, and the links' records of 244 bytes each (65 MB
+        for 4,096 paths of 32 segments)."""
         c = psctx or Context()
         db = DeviceBatch(batch, device=pts.device, seg_pts=pts.detach().contiguous().reshape(-1),
                          path_width=width.detach().contiguous(), wait=False)

@@ -265,13 +265,16 @@ __device__ __forceinline__ int64_t find_link_warp(const int32_t* off, int64_t n,
 }
 
 // ---- overlapped launches ---------------------------------------------------------
-// A kernel that follows another of the same call is launched while that one still runs
-// (programmatic stream serialization): its CTAs take their places as they come free and
-// wait here, before any access to memory, until every earlier kernel has finished and its
-// writes are visible.  Every such kernel calls dep_wait() first thing, so that a kernel is
-// never done before the ones it follows.  One curve on a small canvas: 61 -> 49 us; 64
-// cubics: 97 -> 84; 300 paths: 648 -> 606.  (Letting the next kernel in before a kernel's
-// CTAs are done, by launch_dependents at its start, won nothing more: 53, 86 and 606 us.)
+// A kernel that follows another of the same call is launched with programmatic stream
+// serialization.  No kernel lets the next one in early (launch_dependents), so the next
+// one's CTAs start once the last CTA of the kernel before has ended: what overlaps is the
+// launch itself and the end of the kernel before, whose writes may still be on their way.  So
+// its CTAs wait here, before any access to memory, until every earlier kernel has finished and
+// its writes are visible.  Every such kernel calls dep_wait() first thing, so that a kernel is
+// never done before the ones it follows.  One curve on a small canvas: 62 -> 51 us; 64 cubics:
+// 99 -> 86; 300 paths: 629 -> 617; a dashed path of 5,031 cubics: 581 -> 565.  (With
+// launch_dependents at every kernel's start these took 54, 94, 569 and 573 us, against 52, 92, 566
+// and 564 without in the same run.)
 //   What the kernels before wrote is read through plain pointers, without __restrict__ or
 // __ldg: those say that nobody writes the data while the kernel runs, which is not so before
 // the wait, and the wait's memory clobber does not hold back loads of such data.
